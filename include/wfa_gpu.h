@@ -84,8 +84,8 @@ enum {
                                call by call with one fixed short-read variant (the largest
                                store of the call's length class and penalty model), no
                                sampling autotuner, pairs in call order (no ordering pass),
-                               the arena kernels' work lists in pair order, and no graph
-                               replay (WFA_GPU_GRAPH is ignored); same results */
+                               the deferred pairs' work lists not sorted by cost, and no
+                               graph replay (WFA_GPU_GRAPH is ignored); same results */
   WFA_GPU_GRAPH = 16u,      /* with WFA_GPU_DEVICE_PTRS: for batches repeated with the same
                                arguments (same sizes and buffers, new contents), the first
                                call runs as usual and records the device work into a CUDA

@@ -172,7 +172,10 @@ struct wfa_gpu_ctx {
   HostBuf<int64_t> h_bounds;
   // internal
   DevBuf<int32_t> nruns, defer, defer_long, overflow;
-  DevBuf<int32_t> sorted, sorted_long, sort_aux;  // longest-first work lists (batched path)
+  // band kernels: per-pair keys, their order, the pairs left to the arena
+  // kernels, scratch
+  wfa::BandPlan band{};
+  DevBuf<int32_t> band_key, band_order, arena_list, arena_long_list, band_aux;
   DevBuf<int64_t> run_src, scan_tmp;
   DevBuf<uint32_t> runs, pool;
   int64_t pool_words = kPoolInitWords;  // CIGAR words the arena pool holds
@@ -189,6 +192,7 @@ struct wfa_gpu_ctx {
     int key_len = 0;
     int variant = -1;
     int launches = 0;  // kernels captured
+    bool band = false;  // the band kernels among them
   };
   static constexpr int kGraphs = 4;
   Graph graphs[kGraphs];
@@ -420,45 +424,64 @@ int narrow_above(const wfa_gpu_ctx* c) {
   return c->teams_narrow > c->teams_long ? 4 * c->teams_long : INT32_MAX;
 }
 
-// The arena kernels over the pairs the short kernel deferred (medium pairs
-// on one-warp teams, long ones on one-CTA teams), then retries of the pairs
-// that did not fit: fewer, larger arena slices on one-CTA teams, or a larger
-// CIGAR pool.  A pair that does not fit the whole arena gives ENOMEM.
-int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool longest_first) {
+wfa::BandBufs band_bufs(const wfa_gpu_ctx* c) {
+  return wfa::BandBufs{c->band_key.p, c->band_order.p, c->arena_list.p, c->arena_long_list.p, c->band_aux.p};
+}
+
+// The arena kernels over two work lists (medium pairs on one-warp teams,
+// long ones on one-CTA teams) of nm and nl pairs.
+bool launch_arena_lists(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a, const int32_t* medium,
+                        const int32_t* medium_count, int nm, const int32_t* lng, const int32_t* long_count, int nl) {
+  cudaStream_t st = c->stream;
+  wfa::Ctrl* dc = c->ctrl;
+  const long arena = (long)c->arena_bytes;
+  unsigned char* ab = reinterpret_cast<unsigned char*>(c->arena);
+  // no more teams than pairs: small batches leave the GPU to concurrent work
+  // and get larger arena slices
+  const int tm = std::min<int>(c->teams_medium, nm);
+  const bool narrow = nl > narrow_above(c);
+  const int tl = std::min<int>(narrow ? c->teams_narrow : c->teams_long, nl);
+  return (tm <= 0 || k.launched(wfa::launch_arena(1, a, medium, medium_count, &dc->next_medium, &dc->overflow_count,
+                                                  ab, (arena / tm) & ~255L, tm, st))) &&
+         (tl <= 0 || k.launched(wfa::launch_arena(narrow ? wfa::kLongTeamNarrow : wfa::kLongTeamWide, a, lng,
+                                                  long_count, &dc->next_long, &dc->overflow_count, ab,
+                                                  (arena / tl) & ~255L, tl, st)));
+}
+
+// The arena kernels over the pairs the band kernels left (h_ctrl mirrors the
+// device control block on entry and on return).
+bool finish_arena_lists(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a) {
+  wfa::Ctrl* dc = c->ctrl;
+  const int nm = c->h_ctrl->arena_count, nl = c->h_ctrl->arena_long_count;
+  if (nm == 0 && nl == 0) return true;
+  return launch_arena_lists(c, k, a, c->arena_list.p, &dc->arena_count, nm, c->arena_long_list.p,
+                            &dc->arena_long_count, nl) &&
+         ctrl_to_host(k, c->stream) && k.ok(cudaStreamSynchronize(c->stream));
+}
+
+// The pairs the short kernel deferred: the band kernels, the arena kernels
+// over what those leave (mode 2, arena only: over every pair), then retries
+// of the pairs that did not fit: fewer, larger arena slices on one-CTA
+// teams, or a larger CIGAR pool.  A pair that does not fit the whole arena
+// gives ENOMEM.
+int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode) {
   cudaStream_t st = c->stream;
   wfa::Ctrl* hc = c->h_ctrl;
   wfa::Ctrl* dc = c->ctrl;
-  const long arena = (long)c->arena_bytes;
-  // batched path: the longest pairs first, so that the last pairs a team
-  // takes are short ones (a shorter tail)
-  const int32_t* medium = a.defer_list;
-  const int32_t* lng = a.defer_long_list;
-  if (longest_first && hc->defer_count > 1) {
-    if (!k.launched(wfa::launch_sort_longest_first(a, a.defer_list, &dc->defer_count, hc->defer_count,
-                                                   c->sort_aux.p, c->sorted.p, st), 3))
+  if (mode == 2) {
+    if (!launch_arena_lists(c, k, a, a.defer_list, &dc->defer_count, hc->defer_count, a.defer_long_list,
+                            &dc->defer_long_count, hc->defer_long_count))
       return WFA_GPU_ECUDA;
-    medium = c->sorted.p;
+    if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+    return run_retries(c, k, a);
   }
-  if (longest_first && hc->defer_long_count > 1) {
-    if (!k.launched(wfa::launch_sort_longest_first(a, a.defer_long_list, &dc->defer_long_count,
-                                                   hc->defer_long_count, c->sort_aux.p, c->sorted_long.p, st), 3))
-      return WFA_GPU_ECUDA;
-    lng = c->sorted_long.p;
-  }
-  // no more teams than pairs: small batches leave the GPU to concurrent work
-  // and get larger arena slices
-  const int tm = std::min<int>(c->teams_medium, hc->defer_count);
-  const bool narrow = hc->defer_long_count > narrow_above(c);
-  const int tl = std::min<int>(narrow ? c->teams_narrow : c->teams_long, hc->defer_long_count);
-  if (tm > 0 && !k.launched(wfa::launch_arena(1, a, medium, &dc->defer_count, &dc->next_medium,
-                                              &dc->overflow_count, reinterpret_cast<unsigned char*>(c->arena),
-                                              (arena / tm) & ~255L, tm, st)))
-    return WFA_GPU_ECUDA;
-  if (tl > 0 && !k.launched(wfa::launch_arena(narrow ? wfa::kLongTeamNarrow : wfa::kLongTeamWide, a, lng, &dc->defer_long_count, &dc->next_long,
-                                              &dc->overflow_count, reinterpret_cast<unsigned char*>(c->arena),
-                                              (arena / tl) & ~255L, tl, st)))
+  if (!k.launched(wfa::launch_band(a, c->band, band_bufs(c), (int64_t)hc->defer_count + hc->defer_long_count,
+                                   hc->max_len, mode == 0, reinterpret_cast<unsigned char*>(c->arena),
+                                   (long)c->arena_bytes, st),
+                  wfa::kBandLaunches))
     return WFA_GPU_ECUDA;
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+  if (!finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
   return run_retries(c, k, a);
 }
 
@@ -689,6 +712,7 @@ int wfa_gpu_create(wfa_gpu_ctx** out, int device, size_t scratch_bytes) {
       rc = WFA_GPU_ECUDA;
       break;
     }
+    if (wfa::band_plan(device, &c->band) != cudaSuccess) { rc = WFA_GPU_ECUDA; break; }
     size_teams(c);
     if (const char* ev = std::getenv("WFA_GPU_TEAMS")) {  // tuning override: "<medium>,<wide>[,<narrow>]"
       int a = 0, b = 0, d = 0;
@@ -750,8 +774,8 @@ struct InStreamDrain {
   }
 };
 
-// mode: 0 default (autotuned variant, longest-first arena lists), 1 plain
-// (fixed variant, lists in pair order), 2 arena only.
+// mode: 0 default (autotuned variant, deferred pairs dearest first), 1 plain
+// (fixed variant, deferred pairs in no order), 2 arena only.
 int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t n, int mode,
                     wfa_gpu_penalties pen, int32_t* out_scores, int8_t* out_status, uint32_t* out_cigars,
                     int64_t cap, int64_t* out_off, const StreamIn* sin) {
@@ -862,7 +886,7 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
     const int64_t dc = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
     deferred += dc;
     if (dc > 0) {
-      const int rc = run_arena(ctx, k, ac, mode == 0);
+      const int rc = run_arena(ctx, k, ac, mode);
       if (rc) return rc;
       if (!scan() || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
     }
@@ -973,8 +997,9 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   }
   const int64_t slot_words = score_only ? 1 : n * (int64_t)wfa::kSlot;
   if ((e = ctx->nruns.ensure(n)) || (e = ctx->run_src.ensure(n)) || (e = ctx->defer.ensure(n)) ||
-      (e = ctx->defer_long.ensure(n)) || (e = ctx->overflow.ensure(n)) || (e = ctx->sorted.ensure(n)) ||
-      (e = ctx->sorted_long.ensure(n)) || (e = ctx->sort_aux.ensure(2 * wfa::kSortBuckets)) ||
+      (e = ctx->defer_long.ensure(n)) || (e = ctx->overflow.ensure(n)) || (e = ctx->band_key.ensure(n)) ||
+      (e = ctx->band_order.ensure(n)) || (e = ctx->arena_list.ensure(n)) || (e = ctx->arena_long_list.ensure(n)) ||
+      (e = ctx->band_aux.ensure(wfa::kBandAux)) ||
       (e = ctx->runs.ensure(slot_words)) ||
       (e = ctx->pool.ensure(score_only ? 1 : ctx->pool_words)))
     return map_alloc(e);
@@ -1051,7 +1076,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
   if (ctx->last.deferred_pairs > 0) {
-    rc = run_arena(ctx, k, a, mode == 0);
+    rc = run_arena(ctx, k, a, mode);
     if (rc) return rc;
   }
   if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
@@ -1167,7 +1192,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
                         const int32_t* plen, const char* txt, const int64_t* toff, const int32_t* tlen,
                         wfa_gpu_penalties pen, int32_t max_score, uint32_t flags, int32_t* out_scores,
                         int8_t* out_status, uint32_t* out_cigars, int64_t cap, int64_t* out_off,
-                        bool longest_first) {
+                        bool band, int max_len) {
   cudaStream_t st = c->stream;
   const bool score_only = flags & WFA_GPU_SCORE_ONLY;
   // external event records become graph nodes: replays time their phases
@@ -1201,31 +1226,11 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
                   wfa::short_launches(a, c->plan.v[c->last_variant])))
     return WFA_GPU_ECUDA;
   if (!k.ok(cudaEventRecordWithFlags(c->ev[2], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
-  const long arena = (long)c->arena_bytes;
-  unsigned char* ab = reinterpret_cast<unsigned char*>(c->arena);
-  wfa::Ctrl* dc = c->ctrl;
-  const int32_t* medium = a.defer_list;
-  const int32_t* lng = a.defer_long_list;
-  if (longest_first) {  // batched path with many deferred pairs: longest first
-    if (!k.launched(wfa::launch_sort_longest_first(a, a.defer_list, &dc->defer_count, n, c->sort_aux.p,
-                                                   c->sorted.p, st), 3) ||
-        !k.launched(wfa::launch_sort_longest_first(a, a.defer_long_list, &dc->defer_long_count, n, c->sort_aux.p,
-                                                   c->sorted_long.p, st), 3))
-      return WFA_GPU_ECUDA;
-    medium = c->sorted.p;
-    lng = c->sorted_long.p;
-  }
-  // both one-CTA widths: the deferred count picks one on the device
-  const int32_t narrow_lo = narrow_above(c);
-  if (!k.launched(wfa::launch_arena(1, a, medium, &dc->defer_count, &dc->next_medium, &dc->overflow_count,
-                                    ab, (arena / c->teams_medium) & ~255L, c->teams_medium, st)) ||
-      !k.launched(wfa::launch_arena(wfa::kLongTeamWide, a, lng, &dc->defer_long_count, &dc->next_long,
-                                    &dc->overflow_count, ab, (arena / c->teams_long) & ~255L, c->teams_long, st, 0,
-                                    narrow_lo)) ||
-      (narrow_lo < INT32_MAX &&
-       !k.launched(wfa::launch_arena(wfa::kLongTeamNarrow, a, lng, &dc->defer_long_count, &dc->next_long,
-                                     &dc->overflow_count, ab, (arena / c->teams_narrow) & ~255L, c->teams_narrow, st,
-                                     narrow_lo))))
+  // pairs the band kernels leave to the arena kernels are finished after the
+  // replay
+  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), n, max_len, true,
+                                           reinterpret_cast<unsigned char*>(c->arena), (long)c->arena_bytes, st),
+                          wfa::kBandLaunches))
     return WFA_GPU_ECUDA;
   if (!k.ok(cudaEventRecordWithFlags(c->ev[3], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
   if (!score_only) {
@@ -1252,7 +1257,8 @@ int graph_key(wfa_gpu_ctx* c, uint64_t* key, int64_t n, const void* const* ptrs,
   key[l++] = (uint64_t)(uintptr_t)c->stream;
   const void* bufs[] = {c->ctrl, c->poff.p, c->toff.p, c->scan_tmp.p, c->nruns.p, c->run_src.p, c->runs.p,
                         c->pool.p, c->defer.p, c->defer_long.p, c->overflow.p, c->arena,
-                        c->sorted.p, c->sorted_long.p, c->sort_aux.p, c->lane_words.p, c->lane_slots.p};
+                        c->band_key.p, c->band_order.p, c->arena_list.p, c->arena_long_list.p, c->band_aux.p,
+                        c->lane_words.p, c->lane_slots.p};
   for (const void* b : bufs) key[l++] = (uint64_t)(uintptr_t)b;
   key[l++] = c->pool.cap;
   key[l++] = ((uint64_t)(uint32_t)c->teams_medium << 32) | (uint32_t)c->teams_long;
@@ -1272,7 +1278,7 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
   if (!ctx || !(flags & WFA_GPU_DEVICE_PTRS)) return WFA_GPU_EINVAL;
   const bool score_only = flags & WFA_GPU_SCORE_ONLY;
   const void* ptrs[] = {pat, poff, plen, txt, toff, tlen, out_scores, out_status, out_cigars, out_off};
-  uint64_t key[40];  // 37 entries
+  uint64_t key[40];  // 39 entries
   int kl = graph_key(ctx, key, n, ptrs, 10, pen, max_score, flags, cap);
   wfa_gpu_ctx::Graph* hit = nullptr;
   for (auto& gr : ctx->graphs)
@@ -1293,11 +1299,15 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
     Call k{ctx, false};
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return WFA_GPU_ECUDA;
-    // the longest-first sorts only when the eager run deferred many pairs
-    // (a pure scheduling choice: replays stay correct either way)
-    const bool longest_first = eager_timing.deferred_pairs > 1024;
+    // the band kernels only when the eager run deferred pairs: with nothing
+    // to do their launches took 35 us of a 1.1 ms replay (a pure scheduling
+    // choice: a replay finishes what is left after it).  The longest sequence
+    // of this batch sizes their shared memory; a longer one in a later batch
+    // goes to the arena kernels
+    const bool band = eager_timing.deferred_pairs > 0;
+    const int max_len = ctx->h_ctrl->max_len;
     const int erc = enqueue_device_work(ctx, k, n, pat, poff, plen, txt, toff, tlen, pen, max_score, base,
-                                        out_scores, out_status, out_cigars, cap, out_off, longest_first);
+                                        out_scores, out_status, out_cigars, cap, out_off, band, max_len);
     const cudaError_t ee = cudaStreamEndCapture(st, &g);
     if (erc || ee != cudaSuccess || !g) {
       if (g) cudaGraphDestroy(g);
@@ -1311,6 +1321,7 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
     slot.exec = exec;
     slot.variant = ctx->last_variant;
     slot.launches = k.launches;
+    slot.band = band;
     kl = graph_key(ctx, key, n, ptrs, 10, pen, max_score, flags, cap);
     std::memcpy(slot.key, key, kl * sizeof(uint64_t));
     slot.key_len = kl;
@@ -1330,13 +1341,19 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
   if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (ctx->h_ctrl->bad_input) return WFA_GPU_EINVAL;
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
-  if (ctx->h_ctrl->overflow_count > 0) {
-    // rare: pairs that outgrew their arena slice, retried outside the graph
+  const bool left = hit->band ? ctx->h_ctrl->overflow_count > 0 || ctx->h_ctrl->arena_count > 0 ||
+                                    ctx->h_ctrl->arena_long_count > 0
+                              : ctx->last.deferred_pairs > 0;
+  if (left) {
+    // deferred pairs of a graph without the band kernels, pairs left to the
+    // arena kernels, or (rare) that outgrew their arena slice: finished
+    // outside the graph
     const int64_t* d_poff = poff ? poff : ctx->poff.p;
     const int64_t* d_toff = toff ? toff : ctx->toff.p;
     wfa::AlignArgs a = device_args(ctx, n, pat, d_poff, plen, txt, d_toff, tlen, pen, max_score, score_only,
                                    out_scores, out_status);
-    const int rc = run_retries(ctx, k, a);
+    if (hit->band && !finish_arena_lists(ctx, k, a)) return WFA_GPU_ECUDA;
+    const int rc = hit->band ? run_retries(ctx, k, a) : run_arena(ctx, k, a, 0);
     if (rc) return rc;
     if (!score_only) {
       if (!k.launched(wfa::launch_scan(ctx->nruns.p, n, 0, out_off, ctx->scan_tmp.p, st), 3) ||
@@ -1512,7 +1529,8 @@ void wfa_gpu_destroy(wfa_gpu_ctx* c) {
   c->poff.release(); c->toff.release(); c->score.release(); c->status.release();
   c->cig_off.release(); c->cig.release(); c->nruns.release(); c->defer.release();
   c->overflow.release(); c->run_src.release(); c->scan_tmp.release(); c->runs.release();
-  c->sorted.release(); c->sorted_long.release(); c->sort_aux.release();
+  c->band_key.release(); c->band_order.release(); c->arena_list.release(); c->arena_long_list.release();
+  c->band_aux.release();
   c->defer_long.release(); c->pool.release();
   if (c->in_stream) cudaStreamSynchronize(c->in_stream);
   c->h_score.release(); c->h_status.release(); c->h_off.release(); c->h_cig.release();

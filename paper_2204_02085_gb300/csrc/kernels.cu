@@ -65,13 +65,8 @@ __global__ void __launch_bounds__(kLaneGroup) lane_order_kernel(const AlignArgs 
 template <int WPP>
 __global__ void __launch_bounds__(WPP == 1 ? 128 : 32 * WPP)
     arena_kernel(const AlignArgs a, const int32_t* list, const int32_t* count, int32_t* next, int32_t* overflow_count,
-                 unsigned char* arena, long slot_bytes, int nteams, int seq_words, int32_t count_lo,
-                 int32_t count_hi) {
+                 unsigned char* arena, long slot_bytes, int nteams, int seq_words) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int32_t c = *(volatile const int32_t*)count;
-  // nothing deferred (a graph replays the launch anyway), or the other team
-  // width takes this list
-  if (c <= count_lo || c > count_hi) return;
   arena_body<WPP>(a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words, smem);
 }
 
@@ -480,45 +475,6 @@ __global__ void __launch_bounds__(kAuxBlock) pack_kernel(int64_t n, const char* 
   }
 }
 
-// ------------------------------------------------ longest-first work order
-
-__device__ __forceinline__ int len_bucket(const AlignArgs& a, int32_t pair, int max_len) {
-  const int L = max(a.plen[pair], a.tlen[pair]);
-  const int b = (int)(((long long)L * kSortBuckets) / ((long long)max_len + 1));
-  return b < kSortBuckets ? b : kSortBuckets - 1;
-}
-
-__global__ void sort_hist_kernel(const AlignArgs a, const int32_t* list, const int32_t* count, int32_t* hist) {
-  __shared__ int h[kSortBuckets];
-  for (int i = threadIdx.x; i < kSortBuckets; i += blockDim.x) h[i] = 0;
-  __syncthreads();
-  const int n = *count, ml = a.ctrl->max_len;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    atomicAdd(&h[len_bucket(a, list[i], ml)], 1);
-  __syncthreads();
-  for (int i = threadIdx.x; i < kSortBuckets; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], h[i]);
-}
-
-// bucket starts, longest bucket first (one thread: 64 buckets)
-__global__ void sort_scan_kernel(const int32_t* hist, int32_t* cursor) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int at = 0;
-  for (int b = kSortBuckets - 1; b >= 0; --b) {
-    cursor[b] = at;
-    at += hist[b];
-  }
-}
-
-__global__ void sort_scatter_kernel(const AlignArgs a, const int32_t* list, const int32_t* count, int32_t* cursor,
-                                    int32_t* out) {
-  const int n = *count, ml = a.ctrl->max_len;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int32_t p = list[i];
-    out[atomicAdd(&cursor[len_bucket(a, p, ml)], 1)] = p;
-  }
-}
-
 __global__ void add_kernel(int64_t* p, int64_t count, int64_t v) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
     p[i] += v;
@@ -807,7 +763,7 @@ cudaError_t arena_occupancy(int team_warps, int* teams_per_sm) {
 
 cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list, const int32_t* count,
                          int32_t* next, int32_t* overflow_count, unsigned char* arena, long slot_bytes, int nteams,
-                         cudaStream_t st, int32_t count_lo, int32_t count_hi) {
+                         cudaStream_t st) {
   if (nteams < 1) return cudaSuccess;
   if (team_warps == 1) {
     // four one-warp teams per block; sequences of medium pairs in shared memory
@@ -815,30 +771,18 @@ cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list
     const size_t smem = 4 * (sizeof(TeamShm) + 2 * (size_t)seq_words * sizeof(uint64_t));
     const int grid = (nteams + 3) / 4;
     arena_kernel<1><<<grid, 128, smem, st>>>(a, list, count, next, overflow_count, arena, slot_bytes, nteams,
-                                            seq_words, count_lo, count_hi);
+                                            seq_words);
   } else {
     // one CTA per team; sequences up to 32,768 bases in shared memory
     const int seq_words = 32768 / 32 + 2;
     const size_t smem = sizeof(TeamShm) + 2 * (size_t)seq_words * sizeof(uint64_t);
     if (team_warps == kLongTeamNarrow)
       arena_kernel<kLongTeamNarrow><<<nteams, 32 * kLongTeamNarrow, smem, st>>>(
-          a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words, count_lo, count_hi);
+          a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words);
     else
       arena_kernel<kLongTeamWide><<<nteams, 32 * kLongTeamWide, smem, st>>>(
-          a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words, count_lo, count_hi);
+          a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words);
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sort_longest_first(const AlignArgs& a, const int32_t* list, const int32_t* count, int64_t n_cap,
-                                      int32_t* aux, int32_t* out, cudaStream_t st) {
-  if (n_cap <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(aux, 0, kSortBuckets * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  const int grid = std::min(aux_grid(n_cap, current_device()), 2 * sm_count(current_device()));
-  sort_hist_kernel<<<grid, kAuxBlock, 0, st>>>(a, list, count, aux);
-  sort_scan_kernel<<<1, 32, 0, st>>>(aux, aux + kSortBuckets);
-  sort_scatter_kernel<<<grid, kAuxBlock, 0, st>>>(a, list, count, aux + kSortBuckets, out);
   return cudaGetLastError();
 }
 

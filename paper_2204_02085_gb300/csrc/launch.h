@@ -13,8 +13,8 @@ namespace wfa {
 struct Ctrl {
   int32_t bad_input;        // a length or offset out of range
   int32_t internal_error;   // stored wavefronts inconsistent in a backtrace
-  int32_t defer_count;      // pairs handed to the one-warp arena kernel
-  int32_t defer_long_count; // pairs handed to the one-CTA arena kernel
+  int32_t defer_count;      // deferred pairs: medium (at most kMediumMaxLen bases)
+  int32_t defer_long_count; // and long
   int32_t next_medium;      // work-queue heads of the arena kernels
   int32_t next_long;
   int32_t retry_count;      // pairs of the current retry list
@@ -26,6 +26,12 @@ struct Ctrl {
   long long txt_extent;     // max(offset + length) over texts
   int32_t max_len;          // longest pattern or text
   int32_t lane_next;        // work-queue head of the lane kernel on ordered input
+  // the band kernels (band_path.cuh): queue heads, and the deferred pairs by
+  // who takes them: teams and single warps of the band kernel, or the arena
+  // kernels (medium and long pairs)
+  int32_t bound_next, team_next, warp_next;
+  int32_t team_count, warp_count, arena_count, arena_long_count;
+  int32_t pad;
 };
 
 struct AlignArgs {
@@ -52,8 +58,8 @@ struct AlignArgs {
   uint32_t* runs;     // [n * kSlot] per-pair slots of the short kernel
   uint32_t* pool;     // runs of arena-kernel pairs, reserved by atomics
   int64_t pool_cap;   // words in the pool
-  int32_t* defer_list;       // [n] pairs for the one-warp arena kernel
-  int32_t* defer_long_list;  // [n] pairs for the one-CTA arena kernel
+  int32_t* defer_list;       // [n] deferred medium pairs
+  int32_t* defer_long_list;  // [n] deferred long pairs
   int32_t* overflow_list;    // [n]
   Ctrl* ctrl;
   // lane-per-pair kernel input order (both null: pairs in call order).  Each
@@ -153,22 +159,42 @@ cudaError_t launch_route_all(const AlignArgs& a, cudaStream_t st);
 // (1: one-warp teams of medium pairs; kLongTeamWide or kLongTeamNarrow:
 // one-CTA teams of long pairs).
 cudaError_t arena_occupancy(int team_warps, int* teams_per_sm);
-// The launch works through the list only while count_lo < *count <=
-// count_hi: a graph holds both one-CTA widths and the count, known on the
-// device only, picks the one that runs.
 cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list, const int32_t* count,
                          int32_t* next, int32_t* overflow_count, unsigned char* arena, long slot_bytes, int nteams,
-                         cudaStream_t st, int32_t count_lo = 0, int32_t count_hi = 0x7fffffff);
+                         cudaStream_t st);
 
-// Longest-first order of a work list (batched path): list[0 .. *count) ->
-// out, by the longer sequence of each pair in kSortBuckets equal-width
-// buckets over [0, ctrl->max_len], longest bucket first (order inside a
-// bucket unspecified).  aux: 2 * kSortBuckets ints of scratch.  n_cap bounds
-// *count (sizes the grid).  Reads the count on the device, so it can be
-// captured into a graph.
-constexpr int kSortBuckets = 64;
-cudaError_t launch_sort_longest_first(const AlignArgs& a, const int32_t* list, const int32_t* count, int64_t n_cap,
-                                      int32_t* aux, int32_t* out, cudaStream_t st);
+// The band kernels over the deferred pairs (a.defer_list, a.defer_long_list
+// and their counts in a.ctrl): each pair's score bound, the pairs ordered by
+// cost (largest first; in call order when `ordered` is false), then the band
+// kernel over those it takes.  The rest -- sequences of kBandMaxLen bases and
+// more, scaled penalties above kBandMaxPen, rows wider than a team's shared
+// memory -- end up in arena_list / arena_long_list (ctrl->arena_count,
+// arena_long_count), pairs that outgrow their arena slice in
+// a.overflow_list.  Counts are read on the device, so that the launches can
+// be captured into a graph.
+struct BandPlan {
+  // by the longest sequence of the call, ascending: CTAs per SM and shared
+  // memory of the band kernel
+  static constexpr int kSizes = 3;
+  int max_len[kSizes], per_sm[kSizes], smem[kSizes];
+  int nsm;
+};
+struct BandBufs {
+  int32_t* key;    // [n] by pair: score bound, and its bin in the order
+  int32_t* order;  // [n] the band kernel's pairs: teams' first, then single warps'
+  int32_t* arena_list;
+  int32_t* arena_long_list;
+  int32_t* aux;  // kBandAux ints of scratch
+};
+constexpr int kBandBins = 128;
+constexpr int kBandAux = 2 * kBandBins;
+cudaError_t band_plan(int device, BandPlan* plan);
+// pairs: at most this many are deferred; max_len: the longest sequence among
+// the call's (sizes the shared memory; a pair longer than that still ends up
+// right, in the arena lists).  launches: kernels enqueued.
+cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int max_len,
+                        bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
+constexpr int kBandLaunches = 3;
 
 // Offsets of back-to-back patterns and texts (both exclusive scans of the
 // lengths, [n] = totals) and the checks and extents of launch_validate, in

@@ -10,9 +10,12 @@ namespace wfa {
 
 constexpr int kShortBlock = 128;
 
-// Hand a pair to the arena kernels: pairs with a sequence longer than
-// kMediumMaxLen to the one-CTA kernel, the rest to the one-warp kernel.
+// Hand a pair to the band and arena kernels: pairs with a sequence longer
+// than kMediumMaxLen on the long list, the rest on the medium one; no CIGAR
+// until one of them aligns it (a replayed graph may compact before).
 __device__ __forceinline__ void defer_pair(const AlignArgs& a, int64_t pair) {
+  a.nruns[pair] = 0;
+  a.run_src[pair] = 0;
   if (max(a.plen[pair], a.tlen[pair]) > kMediumMaxLen) {
     const int idx = atomicAdd(&a.ctrl->defer_long_count, 1);
     a.defer_long_list[idx] = (int32_t)pair;
