@@ -135,13 +135,19 @@ struct wfa_gpu_ctx {
   // penalties, and for scaled penalties 2/4/1 the small stores with their
   // geometry compiled in (per-score code: for the large stores its size
   // costs more in instruction fetch than the constants save)
-  int lane_variants[4] = {15, 16, 17, 18};
-  int lane_ct_variants[4] = {19, 20, 17, 18};
+  // (the last of each list takes ordered input only)
+  int lane_variants[5] = {15, 16, 17, 18, 23};
+  int lane_ct_variants[5] = {19, 20, 17, 18, 23};
+  // ordered input: the gap-linear model, and sequences of up to 191 and 255
+  // bases (either model)
+  int lane_lin_variants[2] = {24, 25};
+  int lane_191_variants[2] = {26, 27};
+  int lane_255_variants[2] = {28, 29};
   bool lane_on = true;      // WFA_GPU_LANE=0 turns them off (comparisons)
   // the lane kernel's pairs sorted by estimated score in groups (default
   // path; WFA_GPU_LANE_ORDER=0: call order), and the ordering's buffers
   bool lane_order = true;
-  int lane_sort_min = 12;        // the ordering sorts for stores of scores 0-12 and up (WFA_GPU_LANE_SORT_MIN)
+  int lane_sort_min = 12;        // the ordering bounds each pair for stores of this bound and up (WFA_GPU_LANE_SORT_MIN)
   int64_t pipe_chunk = 1 << 19;  // pairs per chunk of a pipelined host call (WFA_GPU_PIPE_CHUNK)
   DevBuf<uint32_t> lane_words;
   DevBuf<int2> lane_slots;
@@ -537,15 +543,16 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
 
 constexpr int64_t kTuneSample = 4096;
 
-// The lane ordering's buffers for calls of up to n pairs: allocated here
-// (eager calls), or only taken when already large enough (captured work,
-// which must not allocate); left null when the context keeps call order.
-cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, bool may_alloc) {
+// The lane ordering's buffers for calls of up to n pairs of sequences up to
+// max_len: allocated here (eager calls), or only taken when already large
+// enough (captured work, which must not allocate); left null when the
+// context keeps call order, or for longer sequences.
+cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int max_len, bool may_alloc) {
   a.lane_words = nullptr;
   a.lane_slots = nullptr;
-  if (!c->lane_order || n <= 0) return cudaSuccess;
-  const int64_t slots = (n + wfa::kLaneGroup - 1) / wfa::kLaneGroup * wfa::kLaneGroup;
-  const size_t words = (size_t)slots * 2 * wfa::kLaneNW;
+  if (!c->lane_order || !c->lane_on || n <= 0 || max_len > 255) return cudaSuccess;
+  const int64_t slots = (n + wfa::kLaneGroupMax - 1) / wfa::kLaneGroupMax * wfa::kLaneGroupMax;
+  const size_t words = (size_t)slots * 4 * wfa::lane_plane_words(max_len <= 127 ? 127 : max_len <= 191 ? 191 : 255);
   if (may_alloc) {
     cudaError_t e;
     if ((e = c->lane_words.ensure(words)) || (e = c->lane_slots.ensure((size_t)slots))) return e;
@@ -558,33 +565,53 @@ cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, bool m
   return cudaSuccess;
 }
 
-// Pick the short-kernel variant for a batch of sequences <= 127 bases: the
-// large-store variant scores the first kTuneSample pairs (score only); the
-// smallest store that holds nearly all of them (more pairs resident per SM,
-// and for the lane-per-pair kernel fewer lockstep cells) runs the batch.
-// Gap-affine global calls use the lane-per-pair variants unless the context
-// turned them off.  Returns the variant index, or -1 on a CUDA error.
-int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t n) {
+// Pick the short-kernel variant for a batch of sequences <= 127 bases (<= 255
+// on ordered input): the large-store variant scores the first kTuneSample
+// pairs (score only); the smallest store that holds nearly all of them (more
+// pairs resident per SM, and for the lane-per-pair kernel in call order fewer
+// lockstep cells) runs the batch.  Gap-affine global calls use the
+// lane-per-pair variants unless the context turned them off.  Returns the
+// variant index, or -1 on a CUDA error.
+int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t n, int max_len) {
   const int model = a_in.oes == a_in.es ? 1 : 0;  // o = 0: gap-linear
   if ((a_in.pb | a_in.pe | a_in.tb | a_in.te) != 0) return c->variant_ef[model];  // ends-free: one variant
-  if (c->variant_forced >= 0) {
+  if (c->variant_forced >= 0 && max_len <= 127) {
     const wfa::ShortVariant& f = c->plan.v[c->variant_forced];
     const bool ct_ok = f.ct_x == 0 || (f.ct_x == a_in.xs && f.ct_oe == a_in.oes && f.ct_e == a_in.es);
-    if (f.linear == model && !f.ends_free && ct_ok) return c->variant_forced;
+    if (f.linear == model && !f.ends_free && ct_ok && (f.kernel || wfa::lane_ordered(a_in, f)))
+      return c->variant_forced;
   }
   const wfa::ScaledPen pen{a_in.xs, a_in.oes, a_in.es};
   const bool lane = model == 0 && c->lane_on;
+  const bool ordered = c->lane_on && wfa::lane_ordered(a_in, c->plan.v[c->lane_variants[4]]);
   const wfa::ShortVariant& ct = c->plan.v[c->lane_ct_variants[0]];
   const bool lane_ct = lane && ct.ct_x == a_in.xs && ct.ct_oe == a_in.oes && ct.ct_e == a_in.es;
   // (the compiled-in variants serve only their penalties: any other entry of
   // the list is a table-driven one)
   const int* cand = lane_ct ? c->lane_ct_variants : lane ? c->lane_variants : c->variants_small[model];
-  const int ncand = lane ? 4 : 3;
+  int ncand = lane ? (ordered ? 5 : 4) : 3;
+  if (ordered && max_len > 191) {
+    cand = c->lane_255_variants;
+    ncand = 2;
+  } else if (ordered && max_len > 127) {
+    cand = c->lane_191_variants;
+    ncand = 2;
+  } else if (ordered && model == 1) {
+    cand = c->lane_lin_variants;
+    ncand = 2;
+  }
   const int big = cand[ncand - 1];
-  int s_store[4];
+  // a batch no larger than the sample leaves most of the GPU idle whatever
+  // the store: sampling it first would be the larger part of the call
+  if (n <= kTuneSample) return big;
+  int s_store[5];
   for (int j = 0; j < ncand; ++j) {
     const wfa::ShortVariant& v = c->plan.v[cand[j]];
-    if (v.kind == 1) {
+    if (wfa::lane_ordered(a_in, v)) {
+      wfa::LaneBand lb;
+      wfa::lane_band_plan(a_in, v, &lb);
+      s_store[j] = lb.s_store;
+    } else if (v.kind == 1) {
       wfa::LaneGeo g;
       wfa::lane_geometry(a_in, v.cells, v.rw, &g);
       s_store[j] = g.s_store;
@@ -613,7 +640,7 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   if (!k.ok(cudaMemsetAsync(a.score, 0xff, m * sizeof(int32_t), st))) return -1;
   if (!k.launched(wfa::launch_short(a, c->plan.v[big], st), wfa::short_launches(a, c->plan.v[big]))) return -1;
   if (!k.ok(d2h(c->h_tune, c->tune_score.p, m * sizeof(int32_t), st)) || !k.ok(cudaStreamSynchronize(st))) return -1;
-  int64_t fit[4] = {0, 0, 0, 0}, tot = 0;
+  int64_t fit[5] = {0, 0, 0, 0, 0}, tot = 0;
   for (int64_t i = 0; i < m; ++i) {
     const int sc = c->h_tune[i];
     if (sc < 0) continue;  // deferred, invalid or over the bound: not informative
@@ -623,6 +650,12 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   for (int j = 0; j < ncand; ++j)
     if (tot == 0 || fit[j] * 100 >= tot * 99) return cand[j];
   return big;
+}
+
+// Whether a global call of sequences of 128-255 bases runs on ordered input.
+bool short_ordered(const wfa_gpu_ctx* c, const wfa::AlignArgs& a, int max_len) {
+  return max_len <= 255 && (a.pb | a.pe | a.tb | a.te) == 0 &&
+         wfa::lane_ordered(a, c->plan.v[c->lane_255_variants[0]]);
 }
 
 // The plain baseline's short-read variant: the largest store of the call's
@@ -688,7 +721,7 @@ int wfa_gpu_create(wfa_gpu_ctx** out, int device, size_t scratch_bytes) {
     c->own_arena = c->arena;
     c->own_arena_bytes = c->arena_bytes;
     if (wfa::short_plan(device, &c->plan) != cudaSuccess) { rc = WFA_GPU_ECUDA; break; }
-    if (c->plan.count < 23 || c->plan.v[c->lane_variants[0]].kind != 1 || c->plan.v[c->lane_variants[3]].kind != 1 ||
+    if (c->plan.count < 30 || c->plan.v[c->lane_variants[0]].kind != 1 || c->plan.v[c->lane_variants[3]].kind != 1 ||
         c->plan.v[c->lane_ct_variants[0]].ct_x == 0 || c->plan.v[c->lane_ct_variants[1]].ct_x == 0) {
       rc = WFA_GPU_ECUDA;
       break;
@@ -860,8 +893,8 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
     } else {
       if (vi < 0) {
         vi = fixed_variant(ctx, ac, staged.max_len);
-        if (mode == 0 && staged.max_len <= 127) {
-          vi = autotune_short(ctx, k, ac, m);
+        if (mode == 0 && (staged.max_len <= 127 || short_ordered(ctx, ac, staged.max_len))) {
+          vi = autotune_short(ctx, k, ac, m, staged.max_len);
           if (vi < 0) return fail_cuda(k);
         }
         ctx->last_variant = vi;
@@ -1042,7 +1075,8 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
     const StreamIn sin{patterns, texts};
     const bool streamed = host_seqs && !pattern_offsets && !text_offsets && mapped_range(patterns, pe) &&
                           mapped_range(texts, te);
-    if (mode == 0 && (e = lane_order_args(ctx, a, std::min(n, ctx->pipe_chunk), true))) return map_alloc(e);
+    if (mode == 0 && (e = lane_order_args(ctx, a, std::min(n, ctx->pipe_chunk), ctx->h_ctrl->max_len, true)))
+      return map_alloc(e);
     rc = align_pipelined(ctx, k, a, n, mode, pen, out_scores, out_status, out_cigars, cap, out_cigar_offsets,
                          streamed ? &sin : nullptr);
     if (rc < 0 && rc != WFA_GPU_ECIGAR_CAPACITY) return rc;
@@ -1062,10 +1096,10 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   if (arena_only) {
     if (!k.launched(wfa::launch_route_all(a, st))) return fail_cuda(k);
   } else {
-    if (!plain && (e = lane_order_args(ctx, a, n, true))) return map_alloc(e);
+    if (!plain && (e = lane_order_args(ctx, a, n, ctx->h_ctrl->max_len, true))) return map_alloc(e);
     int vi = fixed_variant(ctx, a, ctx->h_ctrl->max_len);
-    if (!plain && ctx->h_ctrl->max_len <= 127) {
-      vi = autotune_short(ctx, k, a, n);
+    if (!plain && (ctx->h_ctrl->max_len <= 127 || short_ordered(ctx, a, ctx->h_ctrl->max_len))) {
+      vi = autotune_short(ctx, k, a, n, ctx->h_ctrl->max_len);
       if (vi < 0) return fail_cuda(k);
     }
     ctx->last_variant = vi;
@@ -1221,7 +1255,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
   wfa::AlignArgs a = device_args(c, n, pat, d_poff, plen, txt, d_toff, tlen, pen, max_score, score_only,
                                  out_scores, out_status);
   if (c->last_variant < 0) return WFA_GPU_ECUDA;
-  if (lane_order_args(c, a, n, false) != cudaSuccess) return WFA_GPU_ECUDA;
+  if (lane_order_args(c, a, n, c->plan.v[c->last_variant].max_len, false) != cudaSuccess) return WFA_GPU_ECUDA;
   if (!k.launched(wfa::launch_short(a, c->plan.v[c->last_variant], st),
                   wfa::short_launches(a, c->plan.v[c->last_variant])))
     return WFA_GPU_ECUDA;

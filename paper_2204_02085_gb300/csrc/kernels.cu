@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kShortBlock, 8) short_kernel(const AlignArgs a
   short_body<G, LMAX, CELLS, SCAP, Off, LIN, EF>(a, smem, &s_last);
 }
 
+
 // One lane per pair, the warp's pairs in lockstep (lane_path.cuh); Fwd is
 // the forward pass: geometry from the table (any penalties) or fixed at
 // compile time (one scaled penalty set).
@@ -50,14 +51,6 @@ template <int LMAX, int CELLS, int RW, int SPAN, int WPB, class Fwd>
 __global__ void __launch_bounds__(32 * WPB, 1) lane_kernel_wide(const AlignArgs a, const LaneGeo g) {
   extern __shared__ __align__(16) unsigned char smem[];
   lane_body<LMAX, CELLS, RW, SPAN, Fwd>(a, g, smem);
-}
-
-// The lane kernel's ordering pass: a block per group of kLaneGroup pairs
-// (lane_path.cuh).
-template <int LMAX>
-__global__ void __launch_bounds__(kLaneGroup) lane_order_kernel(const AlignArgs a, int est_cap) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  lane_order_body<LMAX>(a, est_cap, smem);
 }
 
 // ----------------------------------------------------------- arena kernels
@@ -550,26 +543,10 @@ constexpr int kLaneSpan1 = 4096;
 // memory, with 30 row positions: the 4/6/2 geometry's rows need 30, penalty
 // sets whose rows are wider keep a shorter store)
 constexpr int kWide197 = 18;
-
-// The ordering pass's shared memory and its resident grid (the same for
-// every lane variant).
-using OrderShm = LaneOrderShm<127>;
-
-cudaError_t plan_order(int device, int* grid) {
-  auto k = lane_order_kernel<127>;
-  const size_t smem = sizeof(OrderShm);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kLaneGroup, smem);
-  if (e != cudaSuccess) return e;
-  *grid = sm_count(device) * (per_sm < 1 ? 1 : per_sm);
-  return cudaSuccess;
-}
-
 // A lane-per-pair variant; CT_X, CT_OE, CT_E: the scaled penalties whose
 // geometry is compiled in (0: any penalties, geometry from the table).
-template <int LMAX, int CELLS, int RW, int WPB, int CT_X = 0, int CT_OE = 0, int CT_E = 0, int SPAN = kLaneSpan>
+template <int LMAX, int CELLS, int RW, int WPB, int STORE, int CT_X = 0, int CT_OE = 0, int CT_E = 0,
+          int SPAN = kLaneSpan>
 cudaError_t plan_lane(int device, ShortVariant* v, const char* name) {
   using C = LaneCfg<LMAX, CELLS, RW, SPAN>;
   using Fwd = typename std::conditional<CT_X == 0, LaneRunForward,
@@ -601,7 +578,7 @@ cudaError_t plan_lane(int device, ShortVariant* v, const char* name) {
   v->ct_x = CT_X;
   v->ct_oe = CT_OE;
   v->ct_e = CT_E;
-  return plan_order(device, &v->order_grid);
+  return plan_lane_band(device, v, LMAX, STORE);
 }
 
 }  // namespace
@@ -677,14 +654,30 @@ cudaError_t short_plan(int device, ShortPlan* plan) {
   // and 0-16 under 4/6/2; any penalties (15-18), and with the geometry of
   // scaled penalties x = 2, o + e = 4, e = 1 (4/6/2 and its multiples)
   // compiled in (19-22)
-  if ((e = plan_lane<127, 40, 16, 4, 0, 0, 0, kLaneSpan1>(device, &plan->v[i++], "lane_l127_c40"))) return e;
-  if ((e = plan_lane<127, 64, 16, 4, 0, 0, 0, kLaneSpan1>(device, &plan->v[i++], "lane_l127_c64"))) return e;
-  if ((e = plan_lane<127, 104, 32, 2>(device, &plan->v[i++], "lane_l127_c104"))) return e;
-  if ((e = plan_lane<127, 197, 30, kWide197>(device, &plan->v[i++], "lane_l127_c197"))) return e;
-  if ((e = plan_lane<127, 40, 16, 4, 2, 4, 1, kLaneSpan1>(device, &plan->v[i++], "lane_ct241_l127_c40"))) return e;
-  if ((e = plan_lane<127, 64, 16, 4, 2, 4, 1, kLaneSpan1>(device, &plan->v[i++], "lane_ct241_l127_c64"))) return e;
-  if ((e = plan_lane<127, 104, 32, 2, 2, 4, 1>(device, &plan->v[i++], "lane_ct241_l127_c104"))) return e;
-  if ((e = plan_lane<127, 197, 32, 2, 2, 4, 1>(device, &plan->v[i++], "lane_ct241_l127_c197"))) return e;
+  if ((e = plan_lane<127, 40, 16, 4, kLaneStore8, 0, 0, 0, kLaneSpan1>(device, &plan->v[i++], "lane_l127_c40"))) return e;
+  if ((e = plan_lane<127, 64, 16, 4, kLaneStore10, 0, 0, 0, kLaneSpan1>(device, &plan->v[i++], "lane_l127_c64"))) return e;
+  if ((e = plan_lane<127, 104, 32, 2, kLaneStore12>(device, &plan->v[i++], "lane_l127_c104"))) return e;
+  if ((e = plan_lane<127, 197, 30, kWide197, kLaneStore16>(device, &plan->v[i++], "lane_l127_c197"))) return e;
+  if ((e = plan_lane<127, 40, 16, 4, kLaneStore8, 2, 4, 1, kLaneSpan1>(device, &plan->v[i++], "lane_ct241_l127_c40"))) return e;
+  if ((e = plan_lane<127, 64, 16, 4, kLaneStore10, 2, 4, 1, kLaneSpan1>(device, &plan->v[i++], "lane_ct241_l127_c64"))) return e;
+  if ((e = plan_lane<127, 104, 32, 2, kLaneStore12, 2, 4, 1>(device, &plan->v[i++], "lane_ct241_l127_c104"))) return e;
+  if ((e = plan_lane<127, 197, 32, 2, kLaneStore16, 2, 4, 1>(device, &plan->v[i++], "lane_ct241_l127_c197"))) return e;
+  // ordered input only: a store for costlier pairs, the gap-linear model, and
+  // reads of up to 191 bases (bytes still hold every distance) and of up to
+  // 255 (16-bit rows)
+  if ((e = plan_ordered(device, &plan->v[i++], 127, kLaneStore18, false, "lane_l127_t18"))) return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 127, kLaneStoreLin6, true, "lane_l127_s_lin"))) return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 127, kLaneStore16, true, "lane_l127_m_lin"))) return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 191, lane_band_store(2304, 1408, 10, 191), false, "lane_l191_t12")))
+    return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 191, lane_band_store(3072, 2688, 14, 191), false, "lane_l191_t16")))
+    return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 255, lane_band_store(2304, 1408, 10, 255, 2), false,
+                        "lane_l255_t12_i16")))
+    return e;
+  if ((e = plan_ordered(device, &plan->v[i++], 255, lane_band_store(3072, 2688, 14, 255, 2), false,
+                        "lane_l255_t16_i16")))
+    return e;
   plan->count = i;
   // the one-CTA arena kernels keep two sequences of up to 32,768 bases in
   // shared memory
@@ -696,37 +689,20 @@ cudaError_t short_plan(int device, ShortPlan* plan) {
                               (int)arena_smem);
 }
 
-// Ordered input only for sequences in device memory (the ordering pass
-// reads each pair's bytes with its own loads, which page-locked host memory
-// read in place over the link would turn into many small transfers).
-static bool lane_ordered(const AlignArgs& a, const ShortVariant& v) {
-  return a.n > 0 && v.kind == 1 && a.lane_slots && a.lane_words && !a.host_seqs;
-}
-
 int short_launches(const AlignArgs& a, const ShortVariant& v) { return lane_ordered(a, v) ? 2 : 1; }
 
 cudaError_t launch_short(const AlignArgs& a, const ShortVariant& v, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
-  int grid = v.grid;
   AlignArgs copy = a;
-  const bool ordered = lane_ordered(a, v);
-  if (!ordered) copy.lane_words = nullptr, copy.lane_slots = nullptr;
-  const int64_t groups = (a.n + kLaneGroup - 1) / kLaneGroup;
-  const int64_t units = ordered ? groups * kLaneGroup : a.n;  // pairs, or slots of whole groups
-  const int64_t need = (units + v.pairs_per_block - 1) / v.pairs_per_block;
+  if (lane_ordered(a, v)) return launch_lane_ordered(a, v, st);
+  copy.lane_words = nullptr, copy.lane_slots = nullptr;
+  if (!v.kernel) return cudaErrorInvalidValue;  // an ordered-only variant is chosen for ordered input only
+  int grid = v.grid;
+  const int64_t need = (a.n + v.pairs_per_block - 1) / v.pairs_per_block;
   if (need < grid) grid = (int)need;
   if (v.kind == 1) {
     LaneGeo g;
     lane_geometry(a, v.cells, v.rw, &g);
-    if (ordered) {
-      // estimates above the store's last score all mean "deferred": the
-      // greedy walk stops there; a small store is ordered by packing alone
-      const int cap = g.s_store < a.lane_sort_min ? 0 : std::min(g.s_store + 1, kLaneEstMax);
-      const int og = groups < v.order_grid ? (int)groups : v.order_grid;
-      lane_order_kernel<127><<<og, kLaneGroup, sizeof(OrderShm), st>>>(copy, cap);
-      const cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
     void* args[] = {&copy, &g};
     return cudaLaunchKernel(v.kernel, dim3(grid), dim3(v.block), args, v.smem, st);
   }

@@ -173,17 +173,18 @@ struct LaneSt {
   int s_fin;           // scaled score once finished
 };
 
-// Matches from pattern position v and text position h, up to 32 (kLaneNW
-// packed words at pw[j * 32], tw[j * 32]): the XOR of the two 32-base
-// windows in two 32-bit halves, leading zeros halved.  A window's third word
-// past the last one (j + 2 = kLaneNW) would hold only positions beyond any
-// sequence's end, which no caller counts: the last word stands in for it.
+// Matches from pattern position v and text position h, up to 32 (NW packed
+// words at pw[j * 32], tw[j * 32]): the XOR of the two 32-base windows in two
+// 32-bit halves, leading zeros halved.  A window's third word past the last
+// one (j + 2 = NW) would hold only positions beyond any sequence's end, which
+// no caller counts: the last word stands in for it.
+template <int NW>
 __device__ __forceinline__ int lane_match32(const uint32_t* pw, int v, const uint32_t* tw, int h) {
   const int jp = v >> 4, sp = (v & 15) << 1, jt = h >> 4, st = (h & 15) << 1;
   const uint32_t p1 = pw[(jp + 1) * 32];
   const uint32_t t1 = tw[(jt + 1) * 32];
-  const uint32_t p2 = pw[min(jp + 2, kLaneNW - 1) * 32];
-  const uint32_t t2 = tw[min(jt + 2, kLaneNW - 1) * 32];
+  const uint32_t p2 = pw[min(jp + 2, NW - 1) * 32];
+  const uint32_t t2 = tw[min(jt + 2, NW - 1) * 32];
   const uint32_t dh = __funnelshift_l(p1, pw[jp * 32], sp) ^ __funnelshift_l(t1, tw[jt * 32], st);
   const uint32_t dl = __funnelshift_l(p2, p1, sp) ^ __funnelshift_l(t2, t1, st);
   return dh ? (int)(__clz(dh) >> 1) : 16 + (int)(__clz(dl) >> 1);
@@ -204,7 +205,7 @@ __device__ __forceinline__ void lane_pending(LaneSt& st, uint32_t pend, int lo, 
       ch = cb - (int)st.H[(base + ci) * 32];
     }
     if (ci >= 0) {
-      const int eq = lane_match32(st.pw, ch - ck, st.tw, ch);
+      const int eq = lane_match32<lane_words_of(127)>(st.pw, ch - ck, st.tw, ch);
       ch += eq;
       if (eq < 32 || ch >= cb) {
         st.H[(base + ci) * 32] = (uint8_t)(cb - min(ch, cb));
@@ -463,266 +464,6 @@ __device__ __forceinline__ int lane_backtrace(const UGeo* tab, const uint8_t* H,
   return over ? -1 : nr;
 }
 
-// ------------------------------------------------------------ ordering
-//
-// The warp's 32 pairs run in lockstep until the last of them ends, so a
-// warp's cost is set by its highest score.  The ordering pass puts pairs of
-// similar score into the same warp: every group of kLaneGroup consecutive
-// pairs is packed, each pair gets a cheap upper bound on its scaled score,
-// and the group is sorted by it (stable counting sort, in the block).  The
-// packed words go out in the sorted order, so the lane kernel reads them
-// with coalesced loads and packs nothing itself.
-
-// Largest estimate kept apart; empty slots take it too.
-constexpr int kLaneEstMax = 63;
-
-// The furthest offset of diagonal k from offset h (packed words at W[j * 32]):
-// 32 bases a round.
-__device__ __forceinline__ int lane_extend32(const uint32_t* pw, const uint32_t* tw, int n, int m, int k, int h) {
-  for (;;) {
-    const int rem = min(n - (h - k), m - h);
-    if (rem <= 0) return h;
-    const int eq = lane_match32(pw, h - k, tw, h);
-    if (eq >= rem) return h + rem;
-    h += eq;
-    if (eq < 32) return h;
-  }
-}
-
-// Cost of a greedy alignment, an upper bound on the optimal scaled score,
-// followed only up to cap (a higher bound changes nothing: such a pair
-// passes the store): from the furthest point of diagonal 0, repeatedly take
-// one edit and extend.  A mismatch followed by at least four matches is
-// taken at once; otherwise the mismatch, one inserted and one deleted base
-// (each priced as a fresh event) are all tried, and the one whose extension
-// ends furthest along v + h, less its cost, is taken.  The rest of the
-// longer sequence at an end is one gap.  Packed words at pw[j * 32].
-__device__ __forceinline__ int lane_estimate(const uint32_t* pw, const uint32_t* tw, int n, int m, int X, int OE,
-                                             int E, int cap) {
-  int k = 0, h = lane_extend32(pw, tw, n, m, 0, 0), cost = 0;
-#pragma unroll 1
-  while (cost < cap) {  // every edit costs at least 1
-    const int v = h - k;
-    if (v >= n || h >= m) {
-      const int rem = (n - v) + (m - h);
-      return min(cost + (rem > 0 ? OE + E * (rem - 1) : 0), cap);
-    }
-    const int hx = lane_extend32(pw, tw, n, m, k, h + 1);  // mismatch: v + 1, h + 1
-    if (hx - h >= 5 || hx - k >= n || hx >= m) {
-      h = hx;
-      cost += X;
-      continue;
-    }
-    const int hi = lane_extend32(pw, tw, n, m, k + 1, h + 1);  // insertion: h + 1
-    const int hd = lane_extend32(pw, tw, n, m, k - 1, h);      // deletion: v + 1
-    // v + h after the extension, less the edit's cost (v = h - k)
-    const int gx = 2 * hx - k - X, gi = 2 * hi - (k + 1) - OE, gd = 2 * hd - (k - 1) - OE;
-    if (gx >= gi && gx >= gd) {
-      h = hx;
-      cost += X;
-    } else if (gi >= gd) {
-      ++k;
-      h = hi;
-      cost += OE;
-    } else {
-      --k;
-      h = hd;
-      cost += OE;
-    }
-  }
-  return cap;
-}
-
-// 16 ASCII bytes -> 16 two-bit codes, first byte in the top bits (A C G T
-// = 0 1 2 3 in either case: bits 1 and 2 of the byte, XORed), and whether a
-// byte is not A/C/G/T: the upper-case letter of each byte's code is picked
-// from "ACGT" by a byte permute with the codes as selectors and compared
-// with the byte folded to upper case.  Only when some byte differs is the
-// per-byte mask (bit i: byte i) worked out.
-__device__ __forceinline__ uint32_t lane_code16(uint4 v, uint32_t* bad16) {
-  const uint32_t q[4] = {v.x, v.y, v.z, v.w};
-  uint32_t code = 0u, xs[4], any = 0u;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t w = q[i];
-    const uint32_t c = ((w >> 1) ^ (w >> 2)) & 0x03030303u;  // byte j's code in bits 8j, 8j + 1
-    const uint32_t sel = __byte_perm(c | (c >> 4), 0u, 0x4420u);  // nibble j = byte j's code
-    xs[i] = (w & 0xDFDFDFDFu) ^ __byte_perm(0x54474341u, 0u, sel);  // zero byte <=> valid
-    any |= xs[i];
-    code = (code << 8) | ((c * 0x40100401u) >> 24);
-  }
-  uint32_t bad = 0u;
-  if (any) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t x = xs[i];
-      const uint32_t hb = ((((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) >> 7) & 0x01010101u;  // 1 per nonzero byte
-      bad |= ((hb * 0x01020408u) >> 24 & 0xFu) << (4 * i);
-    }
-  }
-  *bad16 = bad;
-  return code;
-}
-
-// One lane packs one sequence of at most 16 * NCH - 15 bases from device
-// memory into words 0 .. NCH - 1 (16 bases each, first base in the top bits,
-// zero past the end) at out[j * 32]: every aligned 16-byte chunk holding a
-// base is loaded at once, then the words are cut from the chunks' 2-bit
-// codes.  Returns whether a byte of the sequence is not A/C/G/T.
-template <int NCH>
-__device__ __forceinline__ bool lane_pack_direct(const char* seq, int len, uint32_t* out) {
-  const unsigned long long a0 = reinterpret_cast<uintptr_t>(seq), b0 = a0 & ~15ull;
-  const int h = (int)(a0 - b0);
-  const int nch = (h + len + 15) >> 4;
-  uint4 raw[NCH];
-#pragma unroll
-  for (int c = 0; c < NCH; ++c)  // all loads first: their latencies overlap
-    raw[c] = c < nch ? __ldg(reinterpret_cast<const uint4*>(b0 + 16ull * c)) : make_uint4(0u, 0u, 0u, 0u);
-  uint32_t code[NCH + 1], bad[NCH + 1];
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) {
-    code[c] = 0u;
-    bad[c] = 0u;
-    if (c < nch) code[c] = lane_code16(raw[c], &bad[c]);
-  }
-  code[NCH] = 0u;
-  bad[NCH] = 0u;
-  const int nw = (len + 15) >> 4;
-  bool any_bad = false;
-#pragma unroll
-  for (int j = 0; j < NCH; ++j) {
-    uint32_t word = 0u;
-    if (j < nw) {
-      const int rem = min(16, len - 16 * j);
-      word = __funnelshift_l(code[j + 1], code[j], 2 * h);
-      if (rem < 16) word &= ~0u << (32 - 2 * rem);
-      const uint32_t in = (rem >= 16 ? 0xFFFFu : ((1u << rem) - 1u)) << h;  // the word's bytes in chunks j, j + 1
-      if ((bad[j] | (bad[j + 1] << 16)) & in) any_bad = true;
-    }
-    out[j * 32] = word;
-  }
-  return any_bad;
-}
-
-// Shared memory of the ordering pass: per warp the packed words of its 32
-// pairs; the per-warp counts of each estimate and each estimate's first slot.
-template <int LMAX>
-struct LaneOrderShm {
-  static constexpr int NW = LMAX / 16 + 2;
-  static constexpr int kWarps = kLaneGroup / 32;
-  struct Warp {
-    uint32_t pw[NW * 32];
-    uint32_t tw[NW * 32];
-  } w[kWarps];
-  int cnt[2][kWarps][kLaneEstMax + 1];  // alternate groups use alternate halves
-  int start[kLaneEstMax + 1];
-};
-
-// The ordering pass (block of kLaneGroup threads, one per pair of a group;
-// sequences in device memory, each lane reading its own pair's aligned
-// 16-byte chunks).  est_cap = 0: pack only, every slot keeps its pair's
-// place in the group (for stores so small that every warp ends within a few
-// scores anyway, where the estimate would cost more than it saves).  Pairs longer than LMAX are deferred and pairs with a
-// byte other than A/C/G/T get their status here; both, and the slots past
-// the last pair, become empty slots (pair -1) at the end of their group.
-template <int LMAX>
-__device__ void lane_order_body(const AlignArgs& a, int est_cap, unsigned char* smem) {
-  using S_t = LaneOrderShm<LMAX>;
-  constexpr int NW = S_t::NW, WG = S_t::kWarps, NK = kLaneEstMax + 1;
-  static_assert(NW == kLaneNW, "packed words per sequence");
-  static_assert(NK <= 64, "two estimates per lane in the scan");
-  constexpr unsigned FULL = 0xffffffffu;
-  if (*(volatile int32_t*)&a.ctrl->bad_input) return;  // inputs rejected by the validation kernel
-  auto& S = *reinterpret_cast<S_t*>(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto& W = S.w[warp];
-  const int64_t groups = (a.n + kLaneGroup - 1) / kLaneGroup;
-  for (int i = threadIdx.x; i < 2 * WG * NK; i += kLaneGroup) (&S.cnt[0][0][0])[i] = 0;
-  __syncthreads();
-  int half = 0;
-  for (int64_t gi = blockIdx.x; gi < groups; gi += gridDim.x, half ^= 1) {
-    const int64_t pair = gi * kLaneGroup + threadIdx.x;
-    bool active = pair < a.n;
-    int n = 0, m = 0;
-    int64_t po = 0, to = 0;
-    if (active) {
-      n = a.plen[pair];
-      m = a.tlen[pair];
-      po = a.poff[pair];  // with the lengths: one round trip for all four
-      to = a.toff[pair];
-      if (n > LMAX || m > LMAX) {
-        defer_pair(a, pair);
-        active = false;
-      }
-    }
-    if (active) {
-      static_assert(16 * NW - 15 >= LMAX, "chunks of the longest sequence");
-      const bool bad = lane_pack_direct<NW>(a.pat + po, n, W.pw + lane) |
-                       lane_pack_direct<NW>(a.txt + to, m, W.tw + lane);
-      if (bad) {
-        write_result(a, pair, 2, -1, 0, 0);
-        active = false;
-      }
-    }
-    if (est_cap <= 0) {  // call order (uniform over the launch)
-      uint32_t* out = a.lane_words + gi * (2 * NW * kLaneGroup) + threadIdx.x;
-#pragma unroll
-      for (int j = 0; j < NW; ++j) {
-        out[j * kLaneGroup] = active ? W.pw[j * 32 + lane] : 0u;
-        out[(NW + j) * kLaneGroup] = active ? W.tw[j * 32 + lane] : 0u;
-      }
-      a.lane_slots[pair] = make_int2(active ? (int)pair : -1, active ? n | (m << 8) : 0);
-      continue;
-    }
-    const int key = active ? lane_estimate(W.pw + lane, W.tw + lane, n, m, a.xs, a.oes, a.es, est_cap) : kLaneEstMax;
-    // stable: a pair's slot follows every pair of a lower estimate and every
-    // earlier pair of its own.  This group's counts are in half `half` (zero:
-    // cleared while the group before used the other half)
-    auto& cnt = S.cnt[half];
-    const unsigned same = __match_any_sync(FULL, key);
-    const int before = __popc(same & ((1u << lane) - 1u));
-    if (before == 0) cnt[warp][key] = __popc(same);
-    __syncthreads();
-    // every warp is past its reads of the other half (the group before)
-    for (int i = threadIdx.x; i < WG * NK; i += kLaneGroup) (&S.cnt[half ^ 1][0][0])[i] = 0;
-    if (warp == 0) {
-      // lane l: estimates 2l and 2l + 1; each warp's count becomes the count
-      // of the warps before it, then each estimate's first slot
-      int tot[2] = {0, 0};
-      for (int q = 0; q < 2; ++q) {
-        const int e = 2 * lane + q;
-        if (e >= NK) continue;
-        int run = 0;
-        for (int w = 0; w < WG; ++w) {
-          const int c = cnt[w][e];
-          cnt[w][e] = run;
-          run += c;
-        }
-        tot[q] = run;
-      }
-      const int both = tot[0] + tot[1];
-      int incl = both;
-      for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(FULL, incl, d);
-        if (lane >= d) incl += o;
-      }
-      if (2 * lane < NK) S.start[2 * lane] = incl - both;
-      if (2 * lane + 1 < NK) S.start[2 * lane + 1] = incl - both + tot[0];
-    }
-    __syncthreads();
-    const int slot = S.start[key] + cnt[warp][key] + before;
-    uint32_t* out = a.lane_words + gi * (2 * NW * kLaneGroup) + slot;
-#pragma unroll
-    for (int j = 0; j < NW; ++j) {
-      out[j * kLaneGroup] = active ? W.pw[j * 32 + lane] : 0u;
-      out[(NW + j) * kLaneGroup] = active ? W.tw[j * 32 + lane] : 0u;
-    }
-    a.lane_slots[gi * kLaneGroup + slot] = make_int2(active ? (int)pair : -1, active ? n | (m << 8) : 0);
-    // no barrier here: the next group's first barrier comes after every
-    // warp's reads of this group's counts and first slots
-  }
-}
-
 // The lane-per-pair kernel body (global gap-affine alignment, both sequences
 // <= LMAX).  Pairs longer than LMAX, or whose score passes the last stored
 // wavefront (but not the caller's max_score), are deferred to the arena
@@ -753,68 +494,19 @@ __device__ __forceinline__ void lane_body(const AlignArgs& a, const LaneGeo& lg,
   st.s_hi = min(s_store, a.s_cap);
   const int64_t wpb = blockDim.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * wpb * 32;
-  // ordered input: slots of the ordering pass, whole groups, taken by the
-  // warps in batches of 32 from a queue (within a group the batches' costs
-  // rise with the estimates, so a fixed share would give some warps only
-  // the dearest batches); call order: a fixed stride
-  const bool ordered = a.lane_slots != nullptr;
-  static_assert(C::NW == kLaneNW, "packed words per sequence");
-  const int64_t total = ordered ? (a.n + kLaneGroup - 1) / kLaneGroup * kLaneGroup : a.n;
-  // ordered input: the next batch's slot and packed words are loaded into
-  // registers while the current batch computes
-  int64_t next = total;
-  int2 nsl = make_int2(-1, 0);
-  uint32_t nwd[2 * kLaneNW];
-  auto grab = [&]() -> int64_t {
-    int b = 0;
-    if (lane == 0) b = atomicAdd(&a.ctrl->lane_next, 1);
-    return (int64_t)__shfl_sync(0xffffffffu, b, 0) * 32;
-  };
-  auto fetch = [&](int64_t f) {
-    if (f >= total) return;
-    nsl = a.lane_slots[f + lane];
-    const uint32_t* src = a.lane_words + (f / kLaneGroup) * (2 * kLaneNW * kLaneGroup) + f % kLaneGroup + lane;
-#pragma unroll
-    for (int j = 0; j < 2 * kLaneNW; ++j) nwd[j] = src[j * kLaneGroup];
-  };
-  if (ordered) {
-    next = grab();
-    fetch(next);
-  }
-  for (int64_t first = ((int64_t)blockIdx.x * wpb + warp) * 32;; first += stride) {
-    if (ordered) first = next;
-    if (first >= total) break;
-    int64_t pair;
-    bool active;
+  for (int64_t first = ((int64_t)blockIdx.x * wpb + warp) * 32; first < a.n; first += stride) {
+    const int64_t pair = first + lane;
+    bool active = pair < a.n;
     int n = 0, m = 0;
-    if (ordered) {
-      const int2 sl = nsl;
-#pragma unroll
-      for (int j = 0; j < kLaneNW; ++j) {
-        W->pw[j * 32 + lane] = nwd[j];
-        W->tw[j * 32 + lane] = nwd[kLaneNW + j];
-      }
-      next = grab();
-      fetch(next);
-      pair = sl.x;
-      active = pair >= 0;
-      n = sl.y & 255;
-      m = sl.y >> 8;
-      if (active && s_store < 0) {
+    if (active) {
+      n = a.plen[pair];
+      m = a.tlen[pair];
+      if (n > LMAX || m > LMAX || s_store < 0) {
         defer_pair(a, pair);
         active = false;
       }
-    } else {
-      pair = first + lane;
-      active = pair < a.n;
-      if (active) {
-        n = a.plen[pair];
-        m = a.tlen[pair];
-        if (n > LMAX || m > LMAX || s_store < 0) {
-          defer_pair(a, pair);
-          active = false;
-        }
-      }
+    }
+    {
       // all lanes take part: the warp reads its pairs' sequences together
       uint32_t* scratch = reinterpret_cast<uint32_t*>(W->u);
       const char* ps = active ? a.pat + a.poff[pair] : nullptr;
@@ -833,7 +525,7 @@ __device__ __forceinline__ void lane_body(const AlignArgs& a, const LaneGeo& lg,
         active = false;
       }
     }
-    const bool real = ordered ? pair >= 0 : pair < a.n;
+    const bool real = pair < a.n;
     __syncwarp();  // the packer's scratch becomes the store
     {
       // the I and D rows start null

@@ -63,20 +63,26 @@ struct AlignArgs {
   int32_t* overflow_list;    // [n]
   Ctrl* ctrl;
   // lane-per-pair kernel input order (both null: pairs in call order).  Each
-  // group of kLaneGroup consecutive pairs is packed and sorted by an
-  // estimate of its score; slot q of group j holds its pair's packed words
-  // at lane_words[(j * 2 * kLaneNW + w) * kLaneGroup + q] (w < kLaneNW the
-  // pattern's word w, then the text's) and (pair or -1, n | m << 8) at
-  // lane_slots[j * kLaneGroup + q].
+  // group of G = lane_group_of(longest sequence) consecutive pairs is packed
+  // and sorted by a bound on its score; slot q of group j holds its pair's
+  // bit planes at lane_words[(j * 4 * NP + w) * G + q] (NP =
+  // lane_plane_words(...): the pattern's NP words of plane 0, of plane 1, then
+  // the text's) and (pair or -1, n | m << 8 | bound << 16) at
+  // lane_slots[j * G + q].
   uint32_t* lane_words;
   int2* lane_slots;
-  int lane_sort_min;  // smallest store (last stored score) whose ordering sorts
+  int lane_sort_min;  // smallest store (largest bound) whose ordering bounds each pair
 };
 
-// Pairs the lane ordering sorts together, and packed 16-base words per
-// sequence of at most 127 bases the lane kernel reads.
-constexpr int kLaneGroup = 1024;
-constexpr int kLaneNW = 127 / 16 + 2;
+// Packed 16-base words per sequence of at most lmax bases the lane kernel in
+// call order reads; 32-base words per bit plane the one on ordered input
+// reads (a position past the last base included); and the pairs the ordering
+// sorts together (two a thread; longer sequences need more registers and
+// shared memory each).
+__host__ __device__ constexpr int lane_words_of(int lmax) { return lmax / 16 + 2; }
+__host__ __device__ constexpr int lane_plane_words(int lmax) { return lmax / 32 + 1; }
+__host__ __device__ constexpr int lane_group_of(int lmax) { return lmax <= 127 ? 1024 : 512; }
+constexpr int kLaneGroupMax = 1024;
 
 // longest sequence handled by a one-warp arena team; longer pairs go to a
 // one-CTA team
@@ -106,10 +112,16 @@ struct ShortVariant {
   int kind;     // 0 shared-lane, 1 lane-per-pair
   int rw;       // kind 1: positions of each in-place I and D row
   int ct_x, ct_oe, ct_e;  // kind 1: scaled penalties compiled in (0: any)
-  int order_grid;         // kind 1: blocks of the ordering pass that fit the GPU at once
+  // kind 1, ordered input (lane_band.cu): bytes of masks, rows and choices a
+  // warp of the kernel over the diagonals within the bound keeps, the cell
+  // size of its rows, its shared memory, its resident blocks (for scaled
+  // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's.
+  // `kernel` takes call order (null: the variant runs on ordered input only)
+  int band_store, band_cell, band_grid[3], order_grid;
+  size_t band_smem;
 };
 struct ShortPlan {
-  ShortVariant v[24];
+  ShortVariant v[32];
   int count;
 };
 cudaError_t short_plan(int device, ShortPlan* plan);
@@ -147,6 +159,33 @@ struct LaneGeo {
 // diagonals wide, fit the rows, and whose row reads each find the previous
 // score's value or a position not yet written).
 void lane_geometry(const AlignArgs& a, int cells, int rw, LaneGeo* g);
+
+// What the lane kernel over the diagonals within the bound needs of a call
+// (a kernel parameter): row positions, words of choices, the largest
+// bound its store holds (-1: it takes no pair), the shared memory of a warp,
+// and the scores whose rows run (bit s; a score without a wavefront whose rows nobody wrote is left
+// out).
+struct LaneBand {
+  int32_t pitch, words, s_store, warp_bytes;
+  uint32_t run;
+};
+void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb);
+// Whether launch_short runs the ordering pass and the band kernel of v.
+bool lane_ordered(const AlignArgs& a, const ShortVariant& v);
+cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st);
+// Fill the ordered half of a lane variant, or a variant that has no other,
+// for sequences of up to lmax bases and `store` bytes a warp.
+cudaError_t plan_lane_band(int device, ShortVariant* v, int lmax, int store);
+cudaError_t plan_ordered(int device, ShortVariant* v, int lmax, int store, bool linear, const char* name);
+// The bytes of rows (cells of `cell` bytes), choices and `diags` diagonals'
+// masks, and what bounds of 8, 10, 12, 16 and 18 take under scaled penalties
+// 2/4/1, and of 6 under 1/1/1 (the edit distance), for up to 127 bases.
+constexpr int lane_band_store(int rows, int choices, int diags, int lmax, int cell = 1) {
+  return rows * cell + choices + diags * lane_plane_words(lmax) * 128;
+}
+constexpr int kLaneStore8 = lane_band_store(1536, 896, 6, 127), kLaneStore10 = lane_band_store(1920, 1152, 8, 127),
+              kLaneStore12 = lane_band_store(2304, 1408, 10, 127), kLaneStore16 = lane_band_store(3072, 2688, 14, 127),
+              kLaneStore18 = lane_band_store(3456, 3328, 16, 127), kLaneStoreLin6 = lane_band_store(960, 896, 8, 127);
 
 // Arena kernels for pairs deferred by the short kernel: pairs list[0 ..
 // *count), taken through the work-queue head *next; `nteams` teams (one
