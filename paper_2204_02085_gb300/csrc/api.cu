@@ -189,7 +189,8 @@ struct wfa_gpu_ctx {
   DevBuf<int32_t> tune_score, tune_aux;
   DevBuf<int8_t> tune_status;
   DevBuf<int64_t> tune_src;
-  int32_t* h_tune = nullptr;  // pinned [kTuneSample]
+  int32_t* h_tune = nullptr;  // pinned [kTuneSample]: sampled scores, or the sample's bounds (histogram)
+  int32_t* h_tune_dev = nullptr;
   // captured device work of repeated WFA_GPU_GRAPH calls (a few kinds of
   // call, replaced round robin)
   struct Graph {
@@ -323,12 +324,25 @@ const void* mapped_range(const void* p, size_t bytes) {
   return a0.devicePointer;
 }
 
+constexpr int64_t kTuneSample = 4096;
+
+// The bounds of the call's first pairs (a has its penalties and sequences on
+// the device): a histogram in h_tune once the stream is done.
+bool launch_sample_bounds(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs a) {
+  a.n = std::min(a.n, kTuneSample);
+  if (c->tune_score.ensure(wfa::kLaneBoundBins) != cudaSuccess) return k.ok(cudaErrorMemoryAllocation);
+  return k.launched(wfa::launch_lane_bounds(a, c->tune_score.p, c->h_tune_dev, c->stream), 2);
+}
+
 // Lengths, offsets and sequences on the device (or mapped from page-locked
-// host memory); validates them.  Returns 0 or a negative WFA_GPU_* code.
+// host memory); validates them.  sample (device-pointer calls): the call's
+// penalties, to bound its first pairs before the wait.  Returns 0 or a
+// negative WFA_GPU_* code.
 int stage_inputs(wfa_gpu_ctx* c, Call& k, int64_t n, bool dev, const char* pat, const int64_t* poff,
                  const int32_t* plen, const char* txt, const int64_t* toff, const int32_t* tlen,
                  const char** d_pat, const int64_t** d_poff, const int32_t** d_plen, const char** d_txt,
-                 const int64_t** d_toff, const int32_t** d_tlen, bool* host_seqs = nullptr) {
+                 const int64_t** d_toff, const int32_t** d_tlen, bool* host_seqs = nullptr,
+                 const wfa::AlignArgs* sample = nullptr) {
   cudaStream_t st = c->stream;
   cudaError_t e;
   if (dev) {
@@ -391,6 +405,12 @@ int stage_inputs(wfa_gpu_ctx* c, Call& k, int64_t n, bool dev, const char* pat, 
   if (!validated && (!ctrl_to_device(k, c->ctrl, wfa::Ctrl{}, st) ||
                      !k.launched(wfa::launch_validate(n, *d_poff, *d_plen, *d_toff, *d_tlen, c->ctrl, st))))
     return WFA_GPU_ECUDA;
+  if (sample) {
+    wfa::AlignArgs a = *sample;
+    a.pat = pat; a.poff = *d_poff; a.plen = *d_plen;
+    a.txt = txt; a.toff = *d_toff; a.tlen = *d_tlen;
+    if (!launch_sample_bounds(c, k, a)) return WFA_GPU_ECUDA;
+  }
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (c->h_ctrl->bad_input) return WFA_GPU_EINVAL;
   if (dev) {
@@ -541,8 +561,6 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
   return 0;
 }
 
-constexpr int64_t kTuneSample = 4096;
-
 // The lane ordering's buffers for calls of up to n pairs of sequences up to
 // max_len: allocated here (eager calls), or only taken when already large
 // enough (captured work, which must not allocate); left null when the
@@ -566,13 +584,16 @@ cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int ma
 }
 
 // Pick the short-kernel variant for a batch of sequences <= 127 bases (<= 255
-// on ordered input): the large-store variant scores the first kTuneSample
-// pairs (score only); the smallest store that holds nearly all of them (more
-// pairs resident per SM, and for the lane-per-pair kernel in call order fewer
-// lockstep cells) runs the batch.  Gap-affine global calls use the
-// lane-per-pair variants unless the context turned them off.  Returns the
-// variant index, or -1 on a CUDA error.
-int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t n, int max_len) {
+// on ordered input): the smallest store that holds nearly all of a sample of
+// kTuneSample pairs (more pairs resident per SM, and for the lane-per-pair
+// kernel in call order fewer lockstep cells) runs the batch.  Ordered input:
+// by the sample's score bounds (in h_tune already when `sampled`), nine tenths
+// of which the store has to hold -- the greedy bounds of 2 to 7 % of the
+// paper's pairs overshoot a store that holds all their scores.  Call order:
+// the large-store variant scores the sample (score only).  Gap-affine global
+// calls use the lane-per-pair variants unless the context turned them off.
+// Returns the variant index, or -1 on a CUDA error.
+int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t n, int max_len, bool sampled) {
   const int model = a_in.oes == a_in.es ? 1 : 0;  // o = 0: gap-linear
   if ((a_in.pb | a_in.pe | a_in.tb | a_in.te) != 0) return c->variant_ef[model];  // ends-free: one variant
   if (c->variant_forced >= 0 && max_len <= 127) {
@@ -622,6 +643,22 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   }
   const int64_t m = std::min(n, kTuneSample);
   cudaStream_t st = c->stream;
+  if (ordered) {
+    if (!sampled) {
+      wfa::AlignArgs a = a_in;
+      a.n = n;
+      if (!launch_sample_bounds(c, k, a) || !k.ok(cudaStreamSynchronize(st))) return -1;
+    }
+    int64_t all = 0, fit[5] = {0, 0, 0, 0, 0};
+    for (int t = 0; t < wfa::kLaneBoundBins; ++t) {
+      all += c->h_tune[t];
+      for (int j = 0; j < ncand; ++j)
+        if (t <= s_store[j]) fit[j] += c->h_tune[t];
+    }
+    for (int j = 0; j < ncand; ++j)
+      if (all == 0 || fit[j] * 10 >= all * 9) return cand[j];
+    return big;
+  }
   if (c->tune_score.ensure(m) || c->tune_status.ensure(m) || c->tune_aux.ensure(m) || c->tune_src.ensure(m))
     return big;
   wfa::AlignArgs a = a_in;
@@ -702,8 +739,9 @@ int wfa_gpu_create(wfa_gpu_ctx** out, int device, size_t scratch_bytes) {
       if (cudaEventCreate(&c->ev[i]) != cudaSuccess) { rc = WFA_GPU_ECUDA; break; }
     if (rc) break;
     if (cudaMalloc(reinterpret_cast<void**>(&c->ctrl), 2 * sizeof(wfa::Ctrl)) != cudaSuccess) { rc = WFA_GPU_ENOMEM; break; }
-    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_tune), kTuneSample * sizeof(int32_t), cudaHostAllocDefault) !=
-        cudaSuccess) {
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_tune), kTuneSample * sizeof(int32_t), cudaHostAllocMapped) !=
+            cudaSuccess ||
+        cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->h_tune_dev), c->h_tune, 0) != cudaSuccess) {
       rc = WFA_GPU_ENOMEM;
       break;
     }
@@ -894,7 +932,7 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
       if (vi < 0) {
         vi = fixed_variant(ctx, ac, staged.max_len);
         if (mode == 0 && (staged.max_len <= 127 || short_ordered(ctx, ac, staged.max_len))) {
-          vi = autotune_short(ctx, k, ac, m, staged.max_len);
+          vi = autotune_short(ctx, k, ac, m, staged.max_len, false);
           if (vi < 0) return fail_cuda(k);
         }
         ctx->last_variant = vi;
@@ -968,6 +1006,104 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
   return over ? WFA_GPU_ECIGAR_CAPACITY : WFA_GPU_OK;
 }
 
+wfa::AlignArgs device_args(wfa_gpu_ctx* c, int64_t n, const char* pat, const int64_t* poff, const int32_t* plen,
+                           const char* txt, const int64_t* toff, const int32_t* tlen, wfa_gpu_penalties pen,
+                           int32_t max_score, bool score_only, int32_t* out_scores, int8_t* out_status);
+
+// Calls that take the small-call path: a warp per pair, one block for the
+// offsets and one for the CIGAR offsets.  On 37 reads of 100 bases the
+// sampling, ordering and lane kernels took 126 us in six waits; the line lies
+// where the sample of a larger call begins (4,096 pairs of 100 bases at E =
+// 4 % fill the GPU's warps once).
+bool small_call(const wfa_gpu_ctx* c, int64_t n) {
+  return n <= wfa::kDirectPairs && c->lane_on && c->variant_forced < 0;
+}
+
+cudaError_t ensure_work(wfa_gpu_ctx* c, int64_t n, int64_t slot_words, bool score_only) {
+  cudaError_t e;
+  if ((e = c->nruns.ensure(n)) || (e = c->run_src.ensure(n)) || (e = c->defer.ensure(n)) ||
+      (e = c->defer_long.ensure(n)) || (e = c->overflow.ensure(n)) || (e = c->band_key.ensure(n)) ||
+      (e = c->band_order.ensure(n)) || (e = c->arena_list.ensure(n)) || (e = c->arena_long_list.ensure(n)) ||
+      (e = c->band_aux.ensure(wfa::kBandAux)) || (e = c->runs.ensure(slot_words)))
+    return e;
+  return c->pool.ensure(score_only ? 1 : c->pool_words);
+}
+
+// The device work of a small device-pointer call (a.poff / a.toff null:
+// offsets to be worked out into the context's buffers), its control block and
+// CIGAR total in the host mirrors at the end; band: the deferred pairs too.
+bool enqueue_small(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int64_t* out_off, uint32_t* out_cigars, int64_t cap,
+                   bool band, int max_len) {
+  cudaStream_t st = c->stream;
+  unsigned char* ab = reinterpret_cast<unsigned char*>(c->arena);
+  if (!k.launched(wfa::launch_small_front(a.n, a.poff, a.plen, a.toff, a.tlen, c->poff.p, c->toff.p, c->ctrl, st)))
+    return false;
+  if (!a.poff) a.poff = c->poff.p;
+  if (!a.toff) a.toff = c->toff.p;
+  k.rec(1);
+  if (!k.launched(wfa::launch_direct(a, c->band, ab, (long)c->arena_bytes, st))) return false;
+  k.rec(2);
+  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), a.n, max_len, true, ab, (long)c->arena_bytes, st),
+                          wfa::kBandLaunches))
+    return false;
+  k.rec(3);
+  if (!k.launched(wfa::launch_small_finish(a.n, a.nruns, a.score_only ? nullptr : out_off, c->ctrl, c->h_ctrl_dev,
+                                           c->h_total_dev, st)))
+    return false;
+  return a.score_only || k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars,
+                                                        cap, c->ctrl, st));
+}
+
+// After a call's device work with a wait behind it (h_ctrl mirrors the
+// control block): what is left of its pairs -- every deferred one when the
+// band kernels have not run (`band` false), else those they left -- and the
+// CIGARs once more.  Device-pointer calls.
+int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* out_off, uint32_t* out_cigars,
+                int64_t cap) {
+  const wfa::Ctrl* hc = c->h_ctrl;
+  const bool deferred = hc->defer_count > 0 || hc->defer_long_count > 0;
+  const bool left = hc->overflow_count > 0 || (band ? hc->arena_count > 0 || hc->arena_long_count > 0 : deferred);
+  if (!left) return 0;
+  cudaStream_t st = c->stream;
+  cudaError_t e;
+  if (band && !finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
+  const int rc = band || !deferred ? run_retries(c, k, a) : run_arena(c, k, a, 0);
+  if (rc) return rc;
+  if (!a.score_only) {
+    if ((e = c->scan_tmp.ensure(wfa::scan_tmp_elems(a.n)))) return map_alloc(e);
+    if (!k.launched(wfa::launch_scan(a.nruns, a.n, 0, out_off, c->scan_tmp.p, st), 3) ||
+        !k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars, cap, c->ctrl,
+                                        st)) ||
+        !total_to_host(k, out_off + a.n, st))
+      return WFA_GPU_ECUDA;
+  }
+  return k.ok(cudaStreamSynchronize(st)) ? 0 : WFA_GPU_ECUDA;
+}
+
+// A small device-pointer call on the default path.
+int align_small(wfa_gpu_ctx* ctx, Call& k, wfa::AlignArgs& a, uint32_t* out_cigars, int64_t cap, int64_t* out_off) {
+  cudaStream_t st = ctx->stream;
+  if (!enqueue_small(ctx, k, a, out_off, out_cigars, cap, false, 0)) return WFA_GPU_ECUDA;
+  if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+  if (ctx->h_ctrl->bad_input) return WFA_GPU_EINVAL;
+  ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
+  const int rc = finish_left(ctx, k, a, false, out_off, out_cigars, cap);
+  if (rc) return rc;
+  if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
+  if (k.timing) {
+    k.rec(4);
+    k.rec(5);
+    if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+    ctx->last.align_ms = elapsed(ctx, 1, 2);
+    ctx->last.general_ms = elapsed(ctx, 2, 3);
+    ctx->last.cigar_ms = elapsed(ctx, 3, 4);
+    ctx->last.total_ms = elapsed(ctx, 0, 5);
+  }
+  ctx->last.kernel_launches = k.launches;
+  ctx->last.short_variant = -1;
+  return !a.score_only && *ctx->h_total > cap ? WFA_GPU_ECIGAR_CAPACITY : WFA_GPU_OK;
+}
+
 int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t* pattern_offsets,
                 const int32_t* pattern_lengths, const char* texts, const int64_t* text_offsets,
                 const int32_t* text_lengths, wfa_gpu_penalties pen, int32_t max_score, uint32_t flags,
@@ -1012,12 +1148,33 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   const int64_t *d_poff, *d_toff;
   const int32_t *d_plen, *d_tlen;
   bool host_seqs = false;
+  cudaError_t e;
+  const bool small = mode == 0 && small_call(ctx, n);
+  if (small && dev) {
+    if ((e = ctx->poff.ensure(n + 1)) || (e = ctx->toff.ensure(n + 1)) || (e = ensure_work(ctx, n, 1, score_only)))
+      return map_alloc(e);
+    wfa::AlignArgs a = device_args(ctx, n, patterns, pattern_offsets, pattern_lengths, texts, text_offsets,
+                                   text_lengths, pen, max_score, score_only, out_scores, out_status);
+    return align_small(ctx, k, a, out_cigars, cap, out_cigar_offsets);
+  }
+  // the sample's bounds with the input checks, in one wait
+  wfa::AlignArgs pens{};
+  pens.n = n;
+  pens.g = g;
+  pens.xs = pen.x / g;
+  pens.es = pen.e / g;
+  pens.oes = (pen.o + pen.e) / g;
+  pens.s_cap = max_score > 0 ? max_score / g : INT_MAX;
+  pens.ctrl = ctx->ctrl;
+  const int32_t* ef = ctx->ends_free;
+  const bool sample = dev && mode == 0 && ctx->lane_on && ctx->lane_order && ctx->variant_forced < 0 &&
+                      (ef[0] | ef[1] | ef[2] | ef[3]) == 0;
   int rc = stage_inputs(ctx, k, n, dev, patterns, pattern_offsets, pattern_lengths, texts, text_offsets,
-                        text_lengths, &d_pat, &d_poff, &d_plen, &d_txt, &d_toff, &d_tlen, &host_seqs);
+                        text_lengths, &d_pat, &d_poff, &d_plen, &d_txt, &d_toff, &d_tlen, &host_seqs,
+                        sample ? &pens : nullptr);
   if (rc) return rc;
   k.rec(1);
 
-  cudaError_t e;
   // host-pointer outputs come back through device buffers and one bulk copy
   // each (kernel stores straight into mapped host memory cross the C2C link
   // in small pieces and measured several times slower)
@@ -1029,13 +1186,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
     d_status = ctx->status.p;
   }
   const int64_t slot_words = score_only ? 1 : n * (int64_t)wfa::kSlot;
-  if ((e = ctx->nruns.ensure(n)) || (e = ctx->run_src.ensure(n)) || (e = ctx->defer.ensure(n)) ||
-      (e = ctx->defer_long.ensure(n)) || (e = ctx->overflow.ensure(n)) || (e = ctx->band_key.ensure(n)) ||
-      (e = ctx->band_order.ensure(n)) || (e = ctx->arena_list.ensure(n)) || (e = ctx->arena_long_list.ensure(n)) ||
-      (e = ctx->band_aux.ensure(wfa::kBandAux)) ||
-      (e = ctx->runs.ensure(slot_words)) ||
-      (e = ctx->pool.ensure(score_only ? 1 : ctx->pool_words)))
-    return map_alloc(e);
+  if ((e = ensure_work(ctx, n, slot_words, score_only))) return map_alloc(e);
 
   wfa::AlignArgs a{};
   a.n = n;
@@ -1095,11 +1246,15 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
 
   if (arena_only) {
     if (!k.launched(wfa::launch_route_all(a, st))) return fail_cuda(k);
+  } else if (small) {
+    if (!k.launched(wfa::launch_direct(a, ctx->band, reinterpret_cast<unsigned char*>(ctx->arena),
+                                       (long)ctx->arena_bytes, st)))
+      return fail_cuda(k);
   } else {
     if (!plain && (e = lane_order_args(ctx, a, n, ctx->h_ctrl->max_len, true))) return map_alloc(e);
     int vi = fixed_variant(ctx, a, ctx->h_ctrl->max_len);
     if (!plain && (ctx->h_ctrl->max_len <= 127 || short_ordered(ctx, a, ctx->h_ctrl->max_len))) {
-      vi = autotune_short(ctx, k, a, n, ctx->h_ctrl->max_len);
+      vi = autotune_short(ctx, k, a, n, ctx->h_ctrl->max_len, sample);
       if (vi < 0) return fail_cuda(k);
     }
     ctx->last_variant = vi;
@@ -1107,13 +1262,32 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
       return fail_cuda(k);
   }
   k.rec(2);
+  const auto scan_compact = [&]() {  // device-pointer calls (the compaction checks the capacity)
+    return score_only || (k.launched(wfa::launch_scan(ctx->nruns.p, n, 0, out_cigar_offsets, ctx->scan_tmp.p, st), 3) &&
+                          total_to_host(k, out_cigar_offsets + n, st) &&
+                          k.launched(wfa::launch_compact(n, ctx->nruns.p, ctx->run_src.p, ctx->runs.p, ctx->pool.p,
+                                                         out_cigar_offsets, out_cigars, cap, ctx->ctrl, st)));
+  };
+  // a device-pointer call whose pairs all fit their kernel is done with this
+  // wait; deferred pairs are aligned and the CIGARs laid out again after it
+  const bool ahead = dev && mode == 0;
+  if (ahead && !k.timing && !scan_compact()) return fail_cuda(k);
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
-  if (ctx->last.deferred_pairs > 0) {
-    rc = run_arena(ctx, k, a, mode);
+  const bool deferred = ctx->last.deferred_pairs > 0;
+  if (deferred || ctx->h_ctrl->overflow_count > 0) {
+    rc = deferred ? run_arena(ctx, k, a, mode) : run_retries(ctx, k, a);
     if (rc) return rc;
   }
   if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
+  if (ahead && !k.timing) {
+    if (deferred || ctx->h_ctrl->overflow_count > 0) {
+      if (!scan_compact() || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
+    }
+    ctx->last.kernel_launches = k.launches;
+    ctx->last.short_variant = ctx->last_variant;
+    return !score_only && *ctx->h_total > cap ? WFA_GPU_ECIGAR_CAPACITY : WFA_GPU_OK;
+  }
   k.rec(3);
 
   int64_t total = 0;
@@ -1231,6 +1405,14 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
   const bool score_only = flags & WFA_GPU_SCORE_ONLY;
   // external event records become graph nodes: replays time their phases
   if (!k.ok(cudaEventRecordWithFlags(c->ev[0], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+  if (small_call(c, n)) {
+    wfa::AlignArgs a =
+        device_args(c, n, pat, poff, plen, txt, toff, tlen, pen, max_score, score_only, out_scores, out_status);
+    for (int i : {1, 2, 3})
+      if (!k.ok(cudaEventRecordWithFlags(c->ev[i], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+    if (!enqueue_small(c, k, a, out_off, out_cigars, cap, band, max_len)) return WFA_GPU_ECUDA;
+    return k.ok(cudaEventRecordWithFlags(c->ev[4], st, cudaEventRecordExternal)) ? 0 : WFA_GPU_ECUDA;
+  }
   if (!k.ok(cudaMemsetAsync(c->ctrl, 0, sizeof(wfa::Ctrl), st))) return WFA_GPU_ECUDA;
   const int64_t* d_poff = poff;
   const int64_t* d_toff = toff;
@@ -1370,33 +1552,20 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
   if (!k.ok(cudaGraphLaunch(hit->exec, st))) return WFA_GPU_ECUDA;
   k.launches += hit->launches;  // the kernels the graph holds
   int64_t total = 0;
-  if (!k.ok(d2h(ctx->h_ctrl, ctx->ctrl, sizeof(wfa::Ctrl), st))) return WFA_GPU_ECUDA;
-  if (!score_only && !k.ok(d2h(ctx->h_total, out_off + n, sizeof(int64_t), st))) return WFA_GPU_ECUDA;
+  if (!small_call(ctx, n)) {  // (a small call's kernels write the mirrors)
+    if (!k.ok(d2h(ctx->h_ctrl, ctx->ctrl, sizeof(wfa::Ctrl), st))) return WFA_GPU_ECUDA;
+    if (!score_only && !k.ok(d2h(ctx->h_total, out_off + n, sizeof(int64_t), st))) return WFA_GPU_ECUDA;
+  }
   if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (ctx->h_ctrl->bad_input) return WFA_GPU_EINVAL;
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
-  const bool left = hit->band ? ctx->h_ctrl->overflow_count > 0 || ctx->h_ctrl->arena_count > 0 ||
-                                    ctx->h_ctrl->arena_long_count > 0
-                              : ctx->last.deferred_pairs > 0;
-  if (left) {
-    // deferred pairs of a graph without the band kernels, pairs left to the
-    // arena kernels, or (rare) that outgrew their arena slice: finished
-    // outside the graph
+  {
     const int64_t* d_poff = poff ? poff : ctx->poff.p;
     const int64_t* d_toff = toff ? toff : ctx->toff.p;
     wfa::AlignArgs a = device_args(ctx, n, pat, d_poff, plen, txt, d_toff, tlen, pen, max_score, score_only,
                                    out_scores, out_status);
-    if (hit->band && !finish_arena_lists(ctx, k, a)) return WFA_GPU_ECUDA;
-    const int rc = hit->band ? run_retries(ctx, k, a) : run_arena(ctx, k, a, 0);
+    const int rc = finish_left(ctx, k, a, hit->band, out_off, out_cigars, cap);
     if (rc) return rc;
-    if (!score_only) {
-      if (!k.launched(wfa::launch_scan(ctx->nruns.p, n, 0, out_off, ctx->scan_tmp.p, st), 3) ||
-          !k.launched(wfa::launch_compact(n, ctx->nruns.p, ctx->run_src.p, ctx->runs.p, ctx->pool.p, out_off,
-                                          out_cigars, cap, ctx->ctrl, st)) ||
-          !k.ok(d2h(ctx->h_total, out_off + n, sizeof(int64_t), st)))
-        return WFA_GPU_ECUDA;
-    }
-    if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   }
   if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
   if (!score_only) total = *ctx->h_total;

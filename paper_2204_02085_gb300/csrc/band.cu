@@ -69,13 +69,8 @@ __global__ void __launch_bounds__(32 * kBandWarps) bound_kernel(const AlignArgs 
         }
         continue;
       }
-      // every base a mismatch and the length difference one gap, or one gap
-      // for each sequence
-      const int d = abs(n - m), o = a.oes - a.es;
-      const int one = a.xs * min(n, m) + (d ? o + a.es * d : 0);
-      const int two = (n ? o + a.es * n : 0) + (m ? o + a.es * m : 0);
       BandGeo g = band_geo(a, n, m, 0);
-      T = band_bound(pw, tw, g, a.xs, a.oes, a.es, min(min(one, two), a.s_cap), ring);
+      T = band_bound(pw, tw, g, a.xs, a.oes, a.es, min(band_worst(n, m, a.xs, a.oes, a.es), a.s_cap), ring);
       __syncwarp();
       g = band_geo(a, n, m, T);
       const int need = band_bytes(a, g), width = g.kmax - g.kmin + 1;
@@ -197,10 +192,63 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
   }
 }
 
+// Small calls: a warp per pair from its bytes to its CIGAR, the bound and the
+// exact wavefronts one after the other, every pair of the call at once.  The
+// time is one pair's latency: 37 reads of 100 bases took the ordering pass
+// and the lane kernel 38 us (one lane runs a pair's cells in turn).  Pairs
+// longer than kDirectMaxLen, or whose rows do not fit, are deferred.
+constexpr int kDirectMaxLen = 512;
+template <bool CIG, bool EF>
+__global__ void __launch_bounds__(32 * kBandWarps, 8)
+    direct_kernel(const AlignArgs a, unsigned char* arena, long slot_bytes, int warp_smem) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (*(volatile const int32_t*)&a.ctrl->bad_input) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* my = smem + warp * warp_smem;
+  TeamShm* ts = reinterpret_cast<TeamShm*>(my);
+  my += sizeof(TeamShm);
+  const int room = warp_smem - (int)sizeof(TeamShm);
+  const bool pen_ok = a.xs <= kBandMaxPen && a.oes <= kBandMaxPen && a.es <= kBandMaxPen;
+  const int w0 = (int)blockIdx.x * kBandWarps + warp, nw = (int)gridDim.x * kBandWarps;
+  int round = 0;
+  for (int64_t pair = w0; pair < a.n; pair += nw) {
+    const int n = a.plen[pair], m = a.tlen[pair];
+    const int seq = (4 * (band_words(n) + band_words(m)) + 15) & ~15;
+    bool mine = pen_ok && n <= kDirectMaxLen && m <= kDirectMaxLen && seq + 64 * band_rows(a.xs, a.oes, a.es) <= room;
+    if (mine) {
+      uint32_t* pw = reinterpret_cast<uint32_t*>(my);
+      uint32_t* tw = pw + band_words(n);
+      const bool okp = team_pack32<1>(a.pat + a.poff[pair], n, pw, ts->flags, round);
+      const bool okt = team_pack32<1>(a.txt + a.toff[pair], m, tw, ts->flags, round);
+      if (!(okp && okt)) {
+        if (lane == 0) write_result(a, pair, 2, -1, 0, 0);
+        __syncwarp();
+        continue;
+      }
+      const int T = band_bound(pw, tw, band_geo(a, n, m, 0), a.xs, a.oes, a.es,
+                               min(band_worst(n, m, a.xs, a.oes, a.es), a.s_cap),
+                               reinterpret_cast<uint16_t*>(my + seq));
+      __syncwarp();
+      mine = band_bytes(a, band_geo(a, n, m, T)) <= room;
+      if (mine)
+        band_pair<1, CIG, EF>(a, pair, T, my, ts, round, arena + (size_t)w0 * (size_t)slot_bytes, slot_bytes,
+                              &a.ctrl->overflow_count, true);
+    }
+    if (!mine && lane == 0) defer_pair(a, pair);
+    __syncwarp();
+  }
+}
+
 using BandKernel = void (*)(const AlignArgs, const int32_t*, const int32_t*, unsigned char*, long, int);
 BandKernel band_kernel_of(bool cig, bool ef) {
   return cig ? (ef ? band_kernel<true, true> : band_kernel<true, false>)
              : (ef ? band_kernel<false, true> : band_kernel<false, false>);
+}
+
+using DirectKernel = void (*)(const AlignArgs, unsigned char*, long, int);
+DirectKernel direct_kernel_of(bool cig, bool ef) {
+  return cig ? (ef ? direct_kernel<true, true> : direct_kernel<true, false>)
+             : (ef ? direct_kernel<false, true> : direct_kernel<false, false>);
 }
 
 constexpr int kMaxSmem = 227 * 1024;
@@ -222,6 +270,9 @@ cudaError_t band_plan(int device, BandPlan* plan) {
   for (int q = 0; q < 4; ++q) {
     const BandKernel k = band_kernel_of(q & 1, q & 2);
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem))) return e;
+    if ((e = cudaFuncSetAttribute(direct_kernel_of(q & 1, q & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kMaxSmem)))
+      return e;
   }
   if ((e = cudaFuncSetAttribute(bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem))) return e;
   for (int i = 0; i < BandPlan::kSizes; ++i) {
@@ -237,6 +288,19 @@ cudaError_t band_plan(int device, BandPlan* plan) {
     }
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned char* arena, long arena_bytes,
+                          cudaStream_t st) {
+  if (a.n <= 0) return cudaSuccess;
+  const int smem = plan.smem[0];
+  int64_t grid = std::min<int64_t>((int64_t)plan.nsm * plan.per_sm[0], (a.n + kBandWarps - 1) / kBandWarps);
+  grid = std::max<int64_t>(1, std::min<int64_t>(grid, arena_bytes / (kBandWarps * (64L << 10))));
+  const long slot = (long)(arena_bytes / (grid * kBandWarps)) & ~255L;
+  const bool ef = (a.pb | a.pe | a.tb | a.te) != 0;
+  direct_kernel_of(!a.score_only, ef)<<<(unsigned)grid, 32 * kBandWarps, smem, st>>>(a, arena, slot,
+                                                                                     (smem / kBandWarps) & ~15);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int max_len,

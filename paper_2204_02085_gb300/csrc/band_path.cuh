@@ -315,6 +315,15 @@ __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t
   return -1;
 }
 
+// A bound that needs no search: every base a mismatch and the length
+// difference one gap, or one gap for each sequence.
+__device__ __forceinline__ int band_worst(int n, int m, int x, int oe, int e) {
+  const int d = abs(n - m), o = oe - e;
+  const int one = x * min(n, m) + (d ? o + e * d : 0);
+  const int two = (n ? o + e * n : 0) + (m ? o + e * m : 0);
+  return min(one, two);
+}
+
 // ---------------------------------------------------------------- CIGAR
 
 // Walk back from (M, s, k) over the choice bits and write the events to
@@ -451,12 +460,11 @@ __device__ int band_replay(const BandGeo& g, const uint32_t* pw, const uint32_t*
 
 // ----------------------------------------------------------- one pair
 
-// One pair, on one warp (WPP 1) or a CTA: smem of smem_bytes (at least
-// band_bytes), slot_bytes of the arena at slot.  shared: two words of the
-// team (the end flag and a broadcast slot) besides the reduction words.
+// One pair, on one warp (WPP 1) or a CTA: smem of at least band_bytes,
+// slot_bytes of the arena at slot.  packed: the sequences are at smem already.
 template <int WPP, bool CIG, bool EF>
 __device__ void band_pair(const AlignArgs& a, int64_t pair, int T, unsigned char* smem, TeamShm* ts, int& round,
-                          unsigned char* slot, long slot_bytes, int32_t* overflow_count) {
+                          unsigned char* slot, long slot_bytes, int32_t* overflow_count, bool packed = false) {
   using T_ = Team<WPP>;
   const int r = T_::rank();
   const int n = a.plen[pair], m = a.tlen[pair];
@@ -469,8 +477,10 @@ __device__ void band_pair(const AlignArgs& a, int64_t pair, int T, unsigned char
     return;
   }
   if (EF && r == 0) ts->bcast = 0;
-  team_pack32<WPP>(a.pat + a.poff[pair], n, pw, ts->flags, round);  // the bound pass checked the bytes
-  team_pack32<WPP>(a.txt + a.toff[pair], m, tw, ts->flags, round);
+  if (!packed) {
+    team_pack32<WPP>(a.pat + a.poff[pair], n, pw, ts->flags, round);  // the bound pass checked the bytes
+    team_pack32<WPP>(a.txt + a.toff[pair], m, tw, ts->flags, round);
+  }
   int k_end = 0;
   uint4* bits = reinterpret_cast<uint4*>(slot);
   const int s = band_forward<WPP, CIG, EF>(g, pw, tw, rows, a.xs, a.oes, a.es, bits, &ts->bcast, &k_end);

@@ -388,6 +388,122 @@ __global__ void __launch_bounds__(kScanBlock) scan_apply(const int32_t* in, int6
   for (int r = 0; r < kScanItems; ++r) scan_store4(out, base + r * 4 * kScanBlock, n, vout, carry + ex[r], v[r]);  // out[n] = total
 }
 
+// ------------------------------------------------------------ small calls
+//
+// One block of kSmallBlock threads, kSmallItems consecutive elements each:
+// the work of five launches of a large call, whose launch latencies are most
+// of a small one.
+
+constexpr int kSmallBlock = 1024;
+constexpr int kSmallItems = kDirectPairs / kSmallBlock;
+static_assert(kSmallItems * kSmallBlock == kDirectPairs, "whole items per thread");
+
+// Exclusive sum of v over the block in thread order; *total = all of it.
+__device__ __forceinline__ int64_t small_exclusive(int64_t v, int64_t* total, int64_t* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sh[warp] = x;
+  __syncthreads();
+  int64_t w = sh[lane], inc = w;  // 32 warps
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  *total = __shfl_sync(0xffffffffu, inc, 31);
+  const int64_t before = __shfl_sync(0xffffffffu, inc - w, warp);
+  __syncthreads();  // sh may be used again
+  return before + x - v;
+}
+
+__global__ void __launch_bounds__(kSmallBlock) small_front_kernel(int n, const int64_t* poff, const int32_t* plen,
+                                                                  const int64_t* toff, const int32_t* tlen,
+                                                                  int64_t* out_poff, int64_t* out_toff, Ctrl* ctrl) {
+  __shared__ int64_t sh[32];
+  if (threadIdx.x == 0) *ctrl = Ctrl{};
+  const int i0 = threadIdx.x * kSmallItems;
+  int pl[kSmallItems], tl[kSmallItems];
+  int64_t ps = 0, ts = 0;
+#pragma unroll
+  for (int j = 0; j < kSmallItems; ++j) {
+    pl[j] = i0 + j < n ? plen[i0 + j] : 0;
+    tl[j] = i0 + j < n ? tlen[i0 + j] : 0;
+    ps += pl[j];
+    ts += tl[j];
+  }
+  int64_t total;
+  int64_t pe = poff ? 0 : small_exclusive(ps, &total, sh);
+  int64_t te = toff ? 0 : small_exclusive(ts, &total, sh);
+  long long px = 0, tx = 0;
+  int ml = 0;
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < kSmallItems; ++j) {
+    const int i = i0 + j;
+    if (i >= n) break;
+    if (poff) pe = poff[i];
+    else out_poff[i] = pe;
+    if (toff) te = toff[i];
+    else out_toff[i] = te;
+    if (pl[j] < 0 || tl[j] < 0 || pl[j] > ((1 << 28) - 1) || tl[j] > ((1 << 28) - 1) || pe < 0 || te < 0) {
+      bad = true;
+    } else {
+      px = max(px, (long long)(pe + pl[j]));
+      tx = max(tx, (long long)(te + tl[j]));
+      ml = max(ml, max(pl[j], tl[j]));
+    }
+    pe += pl[j];
+    te += tl[j];
+  }
+  px = warp_max64(px);
+  tx = warp_max64(tx);
+  ml = __reduce_max_sync(0xffffffffu, ml);
+  const bool any_bad = __any_sync(0xffffffffu, bad);
+  __syncthreads();  // the control block is zero
+  if ((threadIdx.x & 31) == 0) {
+    if (px) atomicMax(&ctrl->pat_extent, px);
+    if (tx) atomicMax(&ctrl->txt_extent, tx);
+    if (ml) atomicMax(&ctrl->max_len, ml);
+    if (any_bad) atomicExch(&ctrl->bad_input, 1);
+  }
+}
+
+__global__ void __launch_bounds__(kSmallBlock) small_finish_kernel(int n, const int32_t* nruns, int64_t* off,
+                                                                   const Ctrl* ctrl, Ctrl* h_ctrl, int64_t* h_total) {
+  __shared__ int64_t sh[32];
+  // (rejected inputs: no pair has a run count; the host sees the flag)
+  const bool bad_input = ctrl->bad_input != 0;
+  if (off && !bad_input) {
+    const int i0 = threadIdx.x * kSmallItems;
+    int v[kSmallItems];
+    int64_t sum = 0;
+#pragma unroll
+    for (int j = 0; j < kSmallItems; ++j) {
+      v[j] = i0 + j < n ? nruns[i0 + j] : 0;
+      sum += v[j];
+    }
+    int64_t total;
+    int64_t at = small_exclusive(sum, &total, sh);
+#pragma unroll
+    for (int j = 0; j < kSmallItems; ++j) {
+      if (i0 + j < n) off[i0 + j] = at;
+      at += v[j];
+    }
+    if (threadIdx.x == 0) {
+      off[n] = total;
+      *h_total = total;
+    }
+  }
+  for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 4); i += kSmallBlock)
+    reinterpret_cast<int32_t*>(h_ctrl)[i] = reinterpret_cast<const int32_t*>(ctrl)[i];
+  __threadfence_system();  // page-locked host mirrors: visible once the stream is done
+}
+
 // ---------------------------------------------------------------- compact
 
 // One warp per 32 consecutive pairs: the lanes write the pairs' words to
@@ -399,7 +515,7 @@ __global__ void __launch_bounds__(kAuxBlock) compact_kernel(int64_t n, const int
                                                              const uint32_t* runs, const uint32_t* pool,
                                                              const int64_t* off, uint32_t* out, int64_t cap,
                                                              const Ctrl* ctrl) {
-  if (off[n] > cap || (ctrl && *(volatile const int32_t*)&ctrl->bad_input)) return;
+  if ((ctrl && *(volatile const int32_t*)&ctrl->bad_input) || off[n] > cap) return;
   __shared__ int64_t s_off[kAuxBlock / 32][32];
   __shared__ int64_t s_src[kAuxBlock / 32][32];
   __shared__ int32_t s_cnt[kAuxBlock / 32][32];
@@ -759,6 +875,21 @@ cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list
       arena_kernel<kLongTeamWide><<<nteams, 32 * kLongTeamWide, smem, st>>>(
           a, list, count, next, overflow_count, arena, slot_bytes, nteams, seq_words);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_small_front(int64_t n, const int64_t* poff, const int32_t* plen, const int64_t* toff,
+                               const int32_t* tlen, int64_t* out_poff, int64_t* out_toff, Ctrl* ctrl,
+                               cudaStream_t st) {
+  if (n <= 0 || n > kDirectPairs) return cudaErrorInvalidValue;
+  small_front_kernel<<<1, kSmallBlock, 0, st>>>((int)n, poff, plen, toff, tlen, out_poff, out_toff, ctrl);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_small_finish(int64_t n, const int32_t* nruns, int64_t* off, const Ctrl* ctrl, Ctrl* h_ctrl,
+                                int64_t* h_total, cudaStream_t st) {
+  if (n <= 0 || n > kDirectPairs) return cudaErrorInvalidValue;
+  small_finish_kernel<<<1, kSmallBlock, 0, st>>>((int)n, nruns, off, ctrl, h_ctrl, h_total);
   return cudaGetLastError();
 }
 

@@ -15,33 +15,59 @@ constexpr int kLaneBandSmem = 96 * 1024;       // more than any variant asks for
 
 // The lane kernels' ordering pass: a block per group of pairs
 // (lane_band.cuh).
-template <int LMAX>
-__global__ void __launch_bounds__(lane_group_of(LMAX) / 2, LMAX <= 127 ? 2 : 3) lane_order_kernel(const AlignArgs a, int cap, int walk) {
+template <int LMAX, int GROUP, int PER>
+__global__ void __launch_bounds__(GROUP / PER, GROUP >= 512 ? 2 : 1)
+    lane_order_kernel(const AlignArgs a, int cap, int walk) {
   extern __shared__ __align__(16) unsigned char smem[];
-  lane_order_body<LMAX>(a, cap, walk != 0, smem);
+  lane_order_body<LMAX, GROUP, PER>(a, cap, walk != 0, smem);
+}
+
+// The sample's bounds (autotuner).
+constexpr int kBoundsBlock = 64;
+__global__ void __launch_bounds__(kBoundsBlock) lane_bounds_kernel(const AlignArgs a, int cap, int32_t* hist) {
+  // a row past the planes: a window that starts in the last word of the
+  // text's last plane reads the word behind it
+  __shared__ __align__(16) unsigned char smem[(kBoundsBlock / 32 * 4 * lane_plane_words(255) + 1) * 128];
+  lane_bounds_body<255, kBoundsBlock>(a, cap, hist, smem);
+}
+
+// Its histogram to the host's mirror.
+__global__ void lane_bounds_out_kernel(const int32_t* hist, int32_t* host) {
+  host[threadIdx.x] = hist[threadIdx.x];
+  __threadfence_system();
 }
 
 // One lane per pair on the ordering pass's output, over the diagonals within
 // the pairs' bounds.
-template <typename U, int LMAX, int PX, int POE, int PE>
+template <typename U, int LMAX, int PX, int POE, int PE, int GROUP>
 __global__ void __launch_bounds__(32 * kLaneBandWarps) lane_band_kernel(const AlignArgs a, const LaneBand lb) {
   extern __shared__ __align__(16) unsigned char smem[];
-  lane_band_body<U, LMAX, PX, POE, PE>(a, lb, smem);
+  lane_band_body<U, LMAX, PX, POE, PE, GROUP>(a, lb, smem);
 }
+
+// Pairs of a group: 1,024 (512 above 127 bases) where whole groups fill the
+// GPU, so that a group sorts well; 128 for smaller calls, whose time is the
+// latency of a group: 20,000 pairs of 60 bases took 165 us in groups of 1,024.
+constexpr int kSmallGroup = 128;
+constexpr int64_t kSmallGroupPairs = 1 << 17;
+int group_for(int lmax, int64_t n) { return n <= kSmallGroupPairs ? kSmallGroup : lane_group_of(lmax); }
 
 using LaneBandKernel = void (*)(const AlignArgs, const LaneBand);
 
 // The kernel of a sequence class and scaled penalties: compiled in for
 // 2/4/1 (4/6/2 and its multiples) and 1/1/1 (the edit distance), else read at
 // run time.
-LaneBandKernel lane_band_kernel_of(int lmax, int x, int oe, int e) {
+LaneBandKernel lane_band_kernel_of(int lmax, int group, int x, int oe, int e) {
   const bool p241 = x == 2 && oe == 4 && e == 1, p111 = x == 1 && oe == 1 && e == 1;
+  if (lmax <= 127 && group == 1024)
+    return p241   ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 1024>
+           : p111 ? lane_band_kernel<uint8_t, 127, 1, 1, 1, 1024>
+                  : lane_band_kernel<uint8_t, 127, 0, 0, 0, 0>;
   if (lmax <= 127)
-    return p241   ? lane_band_kernel<uint8_t, 127, 2, 4, 1>
-           : p111 ? lane_band_kernel<uint8_t, 127, 1, 1, 1>
-                  : lane_band_kernel<uint8_t, 127, 0, 0, 0>;
-  if (lmax <= 191) return p241 ? lane_band_kernel<uint8_t, 191, 2, 4, 1> : lane_band_kernel<uint8_t, 191, 0, 0, 0>;
-  return lane_band_kernel<uint16_t, 255, 0, 0, 0>;
+    return p241 ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 0> : lane_band_kernel<uint8_t, 127, 0, 0, 0, 0>;
+  if (lmax <= 191)
+    return p241 ? lane_band_kernel<uint8_t, 191, 2, 4, 1, 0> : lane_band_kernel<uint8_t, 191, 0, 0, 0, 0>;
+  return lane_band_kernel<uint16_t, 255, 0, 0, 0, 0>;
 }
 
 int sm_count(int device) {
@@ -50,23 +76,38 @@ int sm_count(int device) {
   return v > 0 ? v : 1;
 }
 
-template <int LMAX>
+template <int LMAX, int GROUP, int PER>
 cudaError_t plan_order(int device, int* grid) {
-  auto k = lane_order_kernel<LMAX>;
-  const size_t smem = sizeof(LaneOrderShm<LMAX>);
+  auto k = lane_order_kernel<LMAX, GROUP, PER>;
+  const size_t smem = sizeof(LaneOrderShm<LMAX, GROUP>);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, lane_group_of(LMAX) / 2, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, GROUP / PER, smem);
   if (e != cudaSuccess) return e;
   *grid = sm_count(device) * (per_sm < 1 ? 1 : per_sm);
   return cudaSuccess;
 }
 
-template <int LMAX>
-cudaError_t launch_order(const AlignArgs& a, int grid, int cap, int walk, cudaStream_t st) {
-  lane_order_kernel<LMAX><<<grid, lane_group_of(LMAX) / 2, sizeof(LaneOrderShm<LMAX>), st>>>(a, cap, walk);
+template <int LMAX, int GROUP, int PER>
+cudaError_t launch_order_as(const AlignArgs& a, int grid, int cap, int walk, cudaStream_t st) {
+  lane_order_kernel<LMAX, GROUP, PER><<<grid, GROUP / PER, sizeof(LaneOrderShm<LMAX, GROUP>), st>>>(a, cap, walk);
   return cudaGetLastError();
+}
+
+template <int LMAX>
+cudaError_t plan_orders(int device, int grid[2]) {
+  const cudaError_t e = plan_order<LMAX, lane_group_of(LMAX), 2>(device, &grid[0]);
+  return e != cudaSuccess ? e : plan_order<LMAX, kSmallGroup, 1>(device, &grid[1]);
+}
+
+template <int LMAX>
+cudaError_t launch_order(const AlignArgs& a, const ShortVariant& v, int group, int cap, int walk, cudaStream_t st) {
+  const int64_t groups = (a.n + group - 1) / group;
+  const int most = v.order_grid[group == kSmallGroup ? 1 : 0];
+  const int grid = groups < most ? (int)groups : most;
+  return group == kSmallGroup ? launch_order_as<LMAX, kSmallGroup, 1>(a, grid, cap, walk, st)
+                              : launch_order_as<LMAX, lane_group_of(LMAX), 2>(a, grid, cap, walk, st);
 }
 
 }  // namespace
@@ -79,17 +120,19 @@ cudaError_t plan_lane_band(int device, ShortVariant* v, int lmax, int store) {
   v->kind = 1;
   const int pens[3][3] = {{2, 4, 1}, {1, 1, 1}, {0, 0, 0}};
   for (int q = 0; q < 3; ++q) {
-    const LaneBandKernel k = lane_band_kernel_of(lmax, pens[q][0], pens[q][1], pens[q][2]);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLaneBandSmem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * kLaneBandWarps, v->band_smem);
-    if (e != cudaSuccess) return e;
-    v->band_grid[q] = sm_count(device) * (per_sm < 1 ? 1 : per_sm);
+    for (int group : {kSmallGroup, lane_group_of(lmax)}) {
+      const LaneBandKernel k = lane_band_kernel_of(lmax, group, pens[q][0], pens[q][1], pens[q][2]);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLaneBandSmem);
+      if (e != cudaSuccess) return e;
+      int per_sm = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * kLaneBandWarps, v->band_smem);
+      if (e != cudaSuccess) return e;
+      v->band_grid[q] = sm_count(device) * (per_sm < 1 ? 1 : per_sm);
+    }
   }
-  return lmax <= 127   ? plan_order<127>(device, &v->order_grid)
-         : lmax <= 191 ? plan_order<191>(device, &v->order_grid)
-                       : plan_order<255>(device, &v->order_grid);
+  return lmax <= 127   ? plan_orders<127>(device, v->order_grid)
+         : lmax <= 191 ? plan_orders<191>(device, v->order_grid)
+                       : plan_orders<255>(device, v->order_grid);
 }
 
 cudaError_t plan_ordered(int device, ShortVariant* v, int lmax, int store, bool linear, const char* name) {
@@ -100,7 +143,7 @@ cudaError_t plan_ordered(int device, ShortVariant* v, int lmax, int store, bool 
 }
 
 static void lane_band_solve(const AlignArgs& a, const ShortVariant& v, LaneBand* lb) {
-  *lb = LaneBand{4, 0, -1, (int)(v.band_smem / kLaneBandWarps), 0u};
+  *lb = LaneBand{4, 0, -1, (int)(v.band_smem / kLaneBandWarps), 0, 0u};
   if ((a.pb | a.pe | a.tb | a.te) != 0 ) return;  // global alignment only
   const int X = a.xs, OE = a.oes, E = a.es, R = X > OE ? X : OE, rows = lane_band_rows(X, OE, E);
   if (R > 31 || E > 31) return;
@@ -172,21 +215,30 @@ bool lane_ordered(const AlignArgs& a, const ShortVariant& v) {
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st) {
   LaneBand lb;
   lane_band_plan(a, v, &lb);
-  const int group = lane_group_of(v.max_len);
+  const int group = lb.group = group_for(v.max_len, a.n);
   const int64_t groups = (a.n + group - 1) / group;
   // bounds above the store's mean "deferred" (or over the caller's largest
   // score): the greedy walk stops there
   const int cap = std::max(0, std::min(lb.s_store, a.s_cap));
   const int walk = lb.s_store >= a.lane_sort_min ? 1 : 0;
-  const int og = groups < v.order_grid ? (int)groups : v.order_grid;
-  const cudaError_t e = v.max_len <= 127   ? launch_order<127>(a, og, cap, walk, st)
-                        : v.max_len <= 191 ? launch_order<191>(a, og, cap, walk, st)
-                                           : launch_order<255>(a, og, cap, walk, st);
+  const cudaError_t e = v.max_len <= 127   ? launch_order<127>(a, v, group, cap, walk, st)
+                        : v.max_len <= 191 ? launch_order<191>(a, v, group, cap, walk, st)
+                                           : launch_order<255>(a, v, group, cap, walk, st);
   if (e != cudaSuccess) return e;
   const int64_t need = (groups * group + 32 * kLaneBandWarps - 1) / (32 * kLaneBandWarps);
   const int q = a.xs == 2 && a.oes == 4 && a.es == 1 ? 0 : a.xs == 1 && a.oes == 1 && a.es == 1 ? 1 : 2;
-  lane_band_kernel_of(v.max_len, a.xs, a.oes, a.es)<<<(unsigned)std::min<int64_t>(v.band_grid[q], need),
+  lane_band_kernel_of(v.max_len, group, a.xs, a.oes, a.es)<<<(unsigned)std::min<int64_t>(v.band_grid[q], need),
                                                       32 * kLaneBandWarps, v.band_smem, st>>>(a, lb);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_lane_bounds(const AlignArgs& a, int32_t* hist, int32_t* host, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(hist, 0, kLaneBoundBins * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  static_assert(kLaneBoundMax < kLaneBoundBins, "bins");
+  lane_bounds_kernel<<<(unsigned)((a.n + kBoundsBlock - 1) / kBoundsBlock), kBoundsBlock, 0, st>>>(
+      a, std::max(0, std::min(kLaneBoundMax, a.s_cap)), hist);
+  lane_bounds_out_kernel<<<1, kLaneBoundBins, 0, st>>>(hist, host);
   return cudaGetLastError();
 }
 

@@ -59,7 +59,7 @@ constexpr int kLaneBoundMax = kLaneKeys / 8 - 2;  // largest bound (and stored s
 // planes of both sequences (P: the pattern's NP words of plane 0, then of
 // plane 1, then the text's; word j at P[j * 32]; position i in bit
 // 31 - i % 32 of word i / 32).  Positions past a sequence's end count as
-// whatever lies there: callers clamp.
+// whatever lies there: callers clamp.  Reads up to word 4 * NP of P.
 template <int NP>
 __device__ __forceinline__ int plane_match32(const uint32_t* P, int v, int h) {
   const uint32_t* p = P + (v >> 5) * 32;
@@ -208,37 +208,38 @@ __device__ __forceinline__ bool lane_pack_planes(const char* seq, int len, uint3
 
 // Shared memory of the ordering pass: per warp the bit planes of its 32
 // pairs; per key its count and its first slot.
-template <int LMAX>
+template <int LMAX, int GROUP>
 struct LaneOrderShm {
   static constexpr int NP = lane_plane_words(LMAX);
-  static constexpr int kGroup = lane_group_of(LMAX);
-  uint32_t planes[kGroup / 32][4 * NP * 32];  // per warp: word j of lane l at [j * 32 + l]
+  static constexpr int kGroup = GROUP;
+  uint32_t planes[kGroup / 32][4 * NP * 32];  // per warp: word j of lane l at [j * 32 + l] (cnt behind the last: see
+                                              // plane_match32)
   int cnt[2][kLaneKeys];  // alternate groups use alternate halves
   int start[kLaneKeys];
   int2 slot[kGroup];        // the group's slots in order
   uint16_t from[kGroup];    // and which of its pairs each one holds
 };
 
-// The ordering pass (a block of kGroup / 2 threads, two pairs of a group each;
+// The ordering pass (a block of GROUP / PER threads, PER pairs of a group each;
 // sequences in device memory, each lane reading its own pair's aligned
-// 16-byte chunks).  Two blocks share an SM, so that one packs while the other
-// waits for its bytes or its slowest warp: with one block of kGroup threads
-// half the issue slots were idle.  cap: the largest bound of interest (the last score the
+// 16-byte chunks).  Large groups: two pairs a thread and two blocks an SM, so
+// that one packs while the other waits for its bytes or its slowest warp
+// (with one block of GROUP threads half the issue slots were idle).  cap: the largest bound of interest (the last score the
 // store holds, or the caller's largest); pairs above it get it.  walk =
 // false: every pair at cap, sorted by end diagonal alone (for stores so small
 // that the greedy walk would cost more than it saves).  Pairs longer than LMAX are
 // deferred and pairs with a byte other than A/C/G/T get their status here;
 // both, and the slots past the last pair, become empty slots (pair -1).
-template <int LMAX>
+template <int LMAX, int GROUP, int PER>
 __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned char* smem) {
-  using S_t = LaneOrderShm<LMAX>;
+  using S_t = LaneOrderShm<LMAX, GROUP>;
   constexpr int NP = S_t::NP, G = S_t::kGroup;
   constexpr unsigned FULL = 0xffffffffu;
   if (*(volatile int32_t*)&a.ctrl->bad_input) return;  // inputs rejected by the validation kernel
   auto& S = *reinterpret_cast<S_t*>(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t groups = (a.n + G - 1) / G;
-  constexpr int kThreads = G / 2;
+  constexpr int kThreads = G / PER;
   for (int i = threadIdx.x; i < 2 * kLaneKeys; i += kThreads) (&S.cnt[0][0])[i] = 0;
   __syncthreads();
   int half = 0;
@@ -246,10 +247,10 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
     // this group's counts are in half `half` (zero: cleared while the group
     // before used the other half)
     int* cnt = S.cnt[half];
-    int key[2], at[2];
-    int2 slot[2];
+    int key[PER], at[PER];
+    int2 slot[PER];
 #pragma unroll 1
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < PER; ++q) {
       const int64_t pair = gi * G + q * kThreads + threadIdx.x;
       uint32_t* const P = S.planes[q * (kThreads / 32) + warp] + lane;
       bool active = pair < a.n;
@@ -285,7 +286,7 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
       const int rank = __shfl_sync(FULL, first, leader) + __popc(same & ((1u << lane) - 1u));
       const int2 sl = make_int2(active ? (int)pair : -1, active ? n | (m << 8) | (T << 16) : 0);
       if (q == 0) key[0] = kq, at[0] = rank, slot[0] = sl;
-      else key[1] = kq, at[1] = rank, slot[1] = sl;
+      else key[PER - 1] = kq, at[PER - 1] = rank, slot[PER - 1] = sl;
     }
     __syncthreads();
     // every warp is past its reads of the other half (the group before)
@@ -312,7 +313,7 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < PER; ++q) {
       const int to = S.start[key[q]] + at[q];
       S.slot[to] = slot[q];
       S.from[to] = (uint16_t)(q * kThreads + threadIdx.x);
@@ -322,7 +323,7 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
     // written from where the pairs were packed, a store touched up to 32
     // sectors, and the pass waited for them
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < PER; ++q) {
       const int to = q * kThreads + threadIdx.x, from = S.from[to];
       const uint32_t* const P = S.planes[from >> 5] + (from & 31);
       uint32_t* out = a.lane_words + gi * (4 * NP * G) + to;
@@ -332,6 +333,23 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
     }
     __syncthreads();  // the planes are the next group's
   }
+}
+
+// The bounds alone, of the first pairs of a call whose longest sequence is
+// not known yet: hist[T] counts the pairs with bound T (at most cap).  A
+// thread per pair; longer sequences and other bytes count nowhere.
+template <int LMAX, int BLOCK>
+__device__ void lane_bounds_body(const AlignArgs& a, int cap, int32_t* hist, unsigned char* smem) {
+  constexpr int NP = lane_plane_words(LMAX);
+  if (*(volatile int32_t*)&a.ctrl->bad_input) return;
+  uint32_t* const P = reinterpret_cast<uint32_t*>(smem) + (threadIdx.x >> 5) * (4 * NP * 32) + (threadIdx.x & 31);
+  const int64_t pair = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
+  if (pair >= a.n) return;
+  const int n = a.plen[pair], m = a.tlen[pair];
+  const int64_t po = a.poff[pair], to = a.toff[pair];
+  if (n > LMAX || m > LMAX) return;
+  if (lane_pack_planes<NP>(a.pat + po, n, P) | lane_pack_planes<NP>(a.txt + to, m, P + 2 * NP * 32)) return;
+  atomicAdd(&hist[lane_estimate<NP>(P, n, m, a.xs, a.oes, a.es, cap)], 1);
 }
 
 // ------------------------------------------------------------ the kernel
@@ -365,14 +383,16 @@ __host__ __device__ constexpr int lane_band_rows(int x, int oe, int e) { return 
 
 // Pairs of the ordering pass, one per lane, in batches of 32 slots taken
 // from a queue (within a group the batches' costs rise with the bounds).
-// PX, POE, PE: the scaled penalties when known at compile time, else 0.
+// PX, POE, PE: the scaled penalties when known at compile time, else 0; GROUP
+// likewise (the loads of a batch at constant strides: 2 % of an E = 2 % call).
 // Pairs whose score passes their bound's cap are deferred (or over the
 // caller's bound), as are pairs whose CIGAR needs more than kSlot runs.  A
 // batch whose end diagonals spread too far for the store (around the border
 // of two bounds) runs in two or more passes.
-template <typename U, int LMAX, int PX, int POE, int PE>
+template <typename U, int LMAX, int PX, int POE, int PE, int GROUP>
 __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBand& lb, unsigned char* smem) {
-  constexpr int NP = lane_plane_words(LMAX), G = lane_group_of(LMAX);
+  constexpr int NP = lane_plane_words(LMAX);
+  const int64_t G = GROUP ? GROUP : lb.group;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr uint32_t kNull = sizeof(U) == 1 ? 0xFFu : 0xFFFFu;
   // a null loses at most one a score; LMAX and the null range stay apart
@@ -393,7 +413,7 @@ __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBan
   uint32_t* const bits = reinterpret_cast<uint32_t*>(store + row_bytes) + lane;  // choice word j at bits[j * 32]
   uint16_t* const ev = reinterpret_cast<uint16_t*>(store) + lane;  // events of the walk, over the rows
   const bool cig = !a.score_only;
-  const int64_t total = (a.n + G - 1) / G * G;
+  const int64_t total = (a.n + G - 1) & ~(G - 1);
   int2 nsl = make_int2(-1, 0);
   uint32_t pl[4 * NP];  // the batch's bit planes, until its masks are built
   auto grab = [&]() -> int64_t {
@@ -404,7 +424,7 @@ __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBan
   auto fetch = [&](int64_t f) {
     if (f >= total) return;
     nsl = a.lane_slots[f + lane];
-    const uint32_t* src = a.lane_words + (f / G) * (4 * NP * G) + f % G + lane;
+    const uint32_t* src = a.lane_words + (f & ~(G - 1)) * (4 * NP) + (f & (G - 1)) + lane;
 #pragma unroll
     for (int j = 0; j < 4 * NP; ++j) pl[j] = src[j * G];
   };

@@ -63,7 +63,7 @@ struct AlignArgs {
   int32_t* overflow_list;    // [n]
   Ctrl* ctrl;
   // lane-per-pair kernel input order (both null: pairs in call order).  Each
-  // group of G = lane_group_of(longest sequence) consecutive pairs is packed
+  // group of G (LaneBand::group) consecutive pairs is packed
   // and sorted by a bound on its score; slot q of group j holds its pair's
   // bit planes at lane_words[(j * 4 * NP + w) * G + q] (NP =
   // lane_plane_words(...): the pattern's NP words of plane 0, of plane 1, then
@@ -115,9 +115,10 @@ struct ShortVariant {
   // kind 1, ordered input (lane_band.cu): bytes of masks, rows and choices a
   // warp of the kernel over the diagonals within the bound keeps, the cell
   // size of its rows, its shared memory, its resident blocks (for scaled
-  // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's.
+  // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's (large
+  // and small groups).
   // `kernel` takes call order (null: the variant runs on ordered input only)
-  int band_store, band_cell, band_grid[3], order_grid;
+  int band_store, band_cell, band_grid[3], order_grid[2];
   size_t band_smem;
 };
 struct ShortPlan {
@@ -167,12 +168,18 @@ void lane_geometry(const AlignArgs& a, int cells, int rw, LaneGeo* g);
 // out).
 struct LaneBand {
   int32_t pitch, words, s_store, warp_bytes;
+  int32_t group;  // pairs of a group of the ordering pass (a power of two)
   uint32_t run;
 };
 void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb);
 // Whether launch_short runs the ordering pass and the band kernel of v.
 bool lane_ordered(const AlignArgs& a, const ShortVariant& v);
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st);
+// Bounds of a sample of global pairs (those of at most 255 bases): host[T] =
+// the pairs with score bound T (the last bin: that much or more), through
+// hist on the device; two kernels.
+constexpr int kLaneBoundBins = 32;
+cudaError_t launch_lane_bounds(const AlignArgs& a, int32_t* hist, int32_t* host, cudaStream_t st);
 // Fill the ordered half of a lane variant, or a variant that has no other,
 // for sequences of up to lmax bases and `store` bytes a warp.
 cudaError_t plan_lane_band(int device, ShortVariant* v, int lmax, int store);
@@ -234,12 +241,27 @@ cudaError_t band_plan(int device, BandPlan* plan);
 cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int max_len,
                         bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
 constexpr int kBandLaunches = 3;
+// Calls of at most kDirectPairs pairs: every pair on a warp of its own, what
+// does not fit deferred.
+constexpr int kDirectPairs = 4096;
+cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned char* arena, long arena_bytes,
+                          cudaStream_t st);
 
 // Offsets of back-to-back patterns and texts (both exclusive scans of the
 // lengths, [n] = totals) and the checks and extents of launch_validate, in
 // one pass of three kernels; ctrl must be zeroed first.
 cudaError_t launch_offsets_validate(const int32_t* plen, const int32_t* tlen, int64_t n, int64_t* poff,
                                     int64_t* toff, int64_t* tmp, Ctrl* ctrl, cudaStream_t st);
+
+// Calls of at most kDirectPairs pairs, one block each: the control block
+// zeroed, the offsets that are missing (poff / toff null: the exclusive scans
+// to out_poff / out_toff) and the checks and extents of launch_validate; and
+// the CIGAR offsets (out[n] = the total) with the control block and the
+// total in their host mirrors (device addresses; off null: score only).
+cudaError_t launch_small_front(int64_t n, const int64_t* poff, const int32_t* plen, const int64_t* toff,
+                               const int32_t* tlen, int64_t* out_poff, int64_t* out_toff, Ctrl* ctrl, cudaStream_t st);
+cudaError_t launch_small_finish(int64_t n, const int32_t* nruns, int64_t* off, const Ctrl* ctrl, Ctrl* h_ctrl,
+                                int64_t* h_total, cudaStream_t st);
 
 // Validate lengths / offsets, record max(offset + length) extents.
 cudaError_t launch_validate(int64_t n, const int64_t* poff, const int32_t* plen, const int64_t* toff,
