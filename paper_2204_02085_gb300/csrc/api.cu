@@ -502,7 +502,7 @@ int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode) {
     return run_retries(c, k, a);
   }
   if (!k.launched(wfa::launch_band(a, c->band, band_bufs(c), (int64_t)hc->defer_count + hc->defer_long_count,
-                                   hc->max_len, mode == 0, reinterpret_cast<unsigned char*>(c->arena),
+                                   hc->defer_long_count, hc->max_len, mode == 0, reinterpret_cast<unsigned char*>(c->arena),
                                    (long)c->arena_bytes, st),
                   wfa::kBandLaunches))
     return WFA_GPU_ECUDA;
@@ -1033,7 +1033,7 @@ cudaError_t ensure_work(wfa_gpu_ctx* c, int64_t n, int64_t slot_words, bool scor
 // offsets to be worked out into the context's buffers), its control block and
 // CIGAR total in the host mirrors at the end; band: the deferred pairs too.
 bool enqueue_small(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int64_t* out_off, uint32_t* out_cigars, int64_t cap,
-                   bool band, int max_len) {
+                   bool band, int64_t nlong, int max_len) {
   cudaStream_t st = c->stream;
   unsigned char* ab = reinterpret_cast<unsigned char*>(c->arena);
   if (!k.launched(wfa::launch_small_front(a.n, a.poff, a.plen, a.toff, a.tlen, c->poff.p, c->toff.p, c->ctrl, st)))
@@ -1043,7 +1043,7 @@ bool enqueue_small(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int64_t* out_off,
   k.rec(1);
   if (!k.launched(wfa::launch_direct(a, c->band, ab, (long)c->arena_bytes, st))) return false;
   k.rec(2);
-  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), a.n, max_len, true, ab, (long)c->arena_bytes, st),
+  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), a.n, nlong, max_len, true, ab, (long)c->arena_bytes, st),
                           wfa::kBandLaunches))
     return false;
   k.rec(3);
@@ -1083,7 +1083,7 @@ int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* 
 // A small device-pointer call on the default path.
 int align_small(wfa_gpu_ctx* ctx, Call& k, wfa::AlignArgs& a, uint32_t* out_cigars, int64_t cap, int64_t* out_off) {
   cudaStream_t st = ctx->stream;
-  if (!enqueue_small(ctx, k, a, out_off, out_cigars, cap, false, 0)) return WFA_GPU_ECUDA;
+  if (!enqueue_small(ctx, k, a, out_off, out_cigars, cap, false, 0, 0)) return WFA_GPU_ECUDA;
   if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (ctx->h_ctrl->bad_input) return WFA_GPU_EINVAL;
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
@@ -1400,7 +1400,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
                         const int32_t* plen, const char* txt, const int64_t* toff, const int32_t* tlen,
                         wfa_gpu_penalties pen, int32_t max_score, uint32_t flags, int32_t* out_scores,
                         int8_t* out_status, uint32_t* out_cigars, int64_t cap, int64_t* out_off,
-                        bool band, int max_len) {
+                        bool band, int64_t nlong, int max_len) {
   cudaStream_t st = c->stream;
   const bool score_only = flags & WFA_GPU_SCORE_ONLY;
   // external event records become graph nodes: replays time their phases
@@ -1410,7 +1410,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
         device_args(c, n, pat, poff, plen, txt, toff, tlen, pen, max_score, score_only, out_scores, out_status);
     for (int i : {1, 2, 3})
       if (!k.ok(cudaEventRecordWithFlags(c->ev[i], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
-    if (!enqueue_small(c, k, a, out_off, out_cigars, cap, band, max_len)) return WFA_GPU_ECUDA;
+    if (!enqueue_small(c, k, a, out_off, out_cigars, cap, band, nlong, max_len)) return WFA_GPU_ECUDA;
     return k.ok(cudaEventRecordWithFlags(c->ev[4], st, cudaEventRecordExternal)) ? 0 : WFA_GPU_ECUDA;
   }
   if (!k.ok(cudaMemsetAsync(c->ctrl, 0, sizeof(wfa::Ctrl), st))) return WFA_GPU_ECUDA;
@@ -1444,7 +1444,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
   if (!k.ok(cudaEventRecordWithFlags(c->ev[2], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
   // pairs the band kernels leave to the arena kernels are finished after the
   // replay
-  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), n, max_len, true,
+  if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), n, nlong, max_len, true,
                                            reinterpret_cast<unsigned char*>(c->arena), (long)c->arena_bytes, st),
                           wfa::kBandLaunches))
     return WFA_GPU_ECUDA;
@@ -1522,8 +1522,9 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
     // goes to the arena kernels
     const bool band = eager_timing.deferred_pairs > 0;
     const int max_len = ctx->h_ctrl->max_len;
+    const int64_t nlong = ctx->h_ctrl->defer_long_count;
     const int erc = enqueue_device_work(ctx, k, n, pat, poff, plen, txt, toff, tlen, pen, max_score, base,
-                                        out_scores, out_status, out_cigars, cap, out_off, band, max_len);
+                                        out_scores, out_status, out_cigars, cap, out_off, band, nlong, max_len);
     const cudaError_t ee = cudaStreamEndCapture(st, &g);
     if (erc || ee != cudaSuccess || !g) {
       if (g) cudaGraphDestroy(g);

@@ -152,28 +152,30 @@ __global__ void __launch_bounds__(kPlaceBlock) place_kernel(const AlignArgs a, c
 // 21.8 -> 12.7 ms, 4,000 x 10 kbp score-only 25.8 -> 6.6 ms, 2,000 x 10 kbp
 // with CIGARs 17.7 -> 5.5 ms, 200,000 reads in 100-300 bp windows with free
 // text ends 42.3 -> 2.1 ms.
-template <bool CIG, bool EF>
-__global__ void __launch_bounds__(32 * kBandWarps, 8)
+// WARPS: a CTA of four, or of eight when few pairs are long (launch_band).
+template <bool CIG, bool EF, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
     band_kernel(const AlignArgs a, const int32_t* key, const int32_t* order, unsigned char* arena, long slot_bytes,
                 int warp_smem) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (*(volatile const int32_t*)&a.ctrl->bad_input) return;
+  const uint32_t absent = EF ? band_absent(a.xs, a.oes, a.es) : 0u;
   constexpr int kBoundMask = (1 << kKeyBits) - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nteam = *(volatile const int32_t*)&a.ctrl->team_count;
   const int nwarp = *(volatile const int32_t*)&a.ctrl->warp_count;
-  unsigned char* cta_slot = arena + (size_t)blockIdx.x * kBandWarps * (size_t)slot_bytes;
+  unsigned char* cta_slot = arena + (size_t)blockIdx.x * WARPS * (size_t)slot_bytes;
   if (nteam > 0) {
     TeamShm* ts = reinterpret_cast<TeamShm*>(smem);
     if (threadIdx.x == 0) ts->flags[0] = ts->flags[1] = ts->flags[2] = 0;
     __syncthreads();
     int round = 0;
     for (;;) {
-      const int i = Team<kBandWarps>::broadcast(threadIdx.x == 0 ? atomicAdd(&a.ctrl->team_next, 1) : 0, &ts->bcast);
+      const int i = Team<WARPS>::broadcast(threadIdx.x == 0 ? atomicAdd(&a.ctrl->team_next, 1) : 0, &ts->bcast);
       if (i >= nteam) break;
       const int32_t pair = order[i];
-      band_pair<kBandWarps, CIG, EF>(a, pair, key[pair] & kBoundMask, smem + sizeof(TeamShm), ts, round, cta_slot,
-                                     kBandWarps * slot_bytes, &a.ctrl->overflow_count);
+      band_pair<WARPS, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, smem + sizeof(TeamShm), ts, round, cta_slot,
+                                     WARPS * slot_bytes, &a.ctrl->overflow_count);
     }
     __syncthreads();
   }
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
     i = __shfl_sync(0xffffffffu, i, 0);
     if (i >= nwarp) break;
     const int32_t pair = order[nteam + i];
-    band_pair<1, CIG, EF>(a, pair, key[pair] & kBoundMask, my + sizeof(TeamShm), ts, round,
+    band_pair<1, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, my + sizeof(TeamShm), ts, round,
                           cta_slot + warp * slot_bytes, slot_bytes, &a.ctrl->overflow_count);
     __syncwarp();
   }
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
   const int room = warp_smem - (int)sizeof(TeamShm);
   const bool pen_ok = a.xs <= kBandMaxPen && a.oes <= kBandMaxPen && a.es <= kBandMaxPen;
   const int w0 = (int)blockIdx.x * kBandWarps + warp, nw = (int)gridDim.x * kBandWarps;
+  const uint32_t absent = EF ? band_absent(a.xs, a.oes, a.es) : 0u;
   int round = 0;
   for (int64_t pair = w0; pair < a.n; pair += nw) {
     const int n = a.plen[pair], m = a.tlen[pair];
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
       __syncwarp();
       mine = band_bytes(a, band_geo(a, n, m, T)) <= room;
       if (mine)
-        band_pair<1, CIG, EF>(a, pair, T, my, ts, round, arena + (size_t)w0 * (size_t)slot_bytes, slot_bytes,
+        band_pair<1, CIG, EF>(a, absent, pair, T, my, ts, round, arena + (size_t)w0 * (size_t)slot_bytes, slot_bytes,
                               &a.ctrl->overflow_count, true);
     }
     if (!mine && lane == 0) defer_pair(a, pair);
@@ -240,9 +243,13 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
 }
 
 using BandKernel = void (*)(const AlignArgs, const int32_t*, const int32_t*, unsigned char*, long, int);
-BandKernel band_kernel_of(bool cig, bool ef) {
-  return cig ? (ef ? band_kernel<true, true> : band_kernel<true, false>)
-             : (ef ? band_kernel<false, true> : band_kernel<false, false>);
+template <int WARPS>
+BandKernel band_kernel_as(bool cig, bool ef) {
+  return cig ? (ef ? band_kernel<true, true, WARPS> : band_kernel<true, false, WARPS>)
+             : (ef ? band_kernel<false, true, WARPS> : band_kernel<false, false, WARPS>);
+}
+BandKernel band_kernel_of(int warps, bool cig, bool ef) {
+  return warps == kBandWarps ? band_kernel_as<kBandWarps>(cig, ef) : band_kernel_as<2 * kBandWarps>(cig, ef);
 }
 
 using DirectKernel = void (*)(const AlignArgs, unsigned char*, long, int);
@@ -257,19 +264,23 @@ constexpr int kMaxSmem = 227 * 1024;
 
 cudaError_t band_plan(int device, BandPlan* plan) {
   cudaError_t e;
-  // shared memory for 8, 6 and 3 CTAs an SM (a CTA costs 1 KB besides its
-  // own): under 4/6/2 (9 rows, 18 bytes a diagonal) rows up to about 1,500,
-  // 1,900 and 3,700 diagonals wide on a team: reads of 2,048, 12,000 and
-  // 32,000 bases at up to some 10, 5 and 4 % edits; 8 CTAs are what 64
-  // registers allow
-  const int len[BandPlan::kSizes] = {kMediumMaxLen, 12000, kBandMaxLen};
-  const int want[BandPlan::kSizes] = {8, 6, 3};
+  // CTAs an SM (a CTA costs 1 KB of shared memory besides its own): under
+  // 4/6/2 (9 rows, 18 bytes a diagonal) a team's rows may be about 1,500,
+  // 1,900 and 3,900 diagonals wide: reads of 2,048, 12,000 and 32,000 bases
+  // at up to some 10, 5 and 4 % edits.  Eight CTAs of four warps are what 64
+  // registers allow; the second size has a form with half as many CTAs of
+  // eight warps, the third only that.
+  const int len[BandPlan::kSizes] = {kMediumMaxLen, 12000, 12000, kBandMaxLen};
+  const int warps[BandPlan::kSizes] = {kBandWarps, kBandWarps, 2 * kBandWarps, 2 * kBandWarps};
+  const int want[BandPlan::kSizes] = {8, 6, 3, 3};
   int nsm = 0;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device))) return e;
   plan->nsm = nsm > 0 ? nsm : 1;
   for (int q = 0; q < 4; ++q) {
-    const BandKernel k = band_kernel_of(q & 1, q & 2);
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem))) return e;
+    for (int w : {kBandWarps, 2 * kBandWarps})
+      if ((e = cudaFuncSetAttribute(band_kernel_of(w, q & 1, q & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kMaxSmem)))
+        return e;
     if ((e = cudaFuncSetAttribute(direct_kernel_of(q & 1, q & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   kMaxSmem)))
       return e;
@@ -277,12 +288,13 @@ cudaError_t band_plan(int device, BandPlan* plan) {
   if ((e = cudaFuncSetAttribute(bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem))) return e;
   for (int i = 0; i < BandPlan::kSizes; ++i) {
     plan->max_len[i] = len[i];
+    plan->warps[i] = warps[i];
     plan->smem[i] = (228 * 1024 / want[i] - 1024) & ~127;
     plan->per_sm[i] = want[i];
     for (int q = 0; q < 4; ++q) {
       int got = 0;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, band_kernel_of(q & 1, q & 2), 32 * kBandWarps,
-                                                             plan->smem[i])))
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, band_kernel_of(warps[i], q & 1, q & 2),
+                                                             32 * warps[i], plan->smem[i])))
         return e;
       plan->per_sm[i] = std::max(1, std::min(plan->per_sm[i], got));
     }
@@ -303,13 +315,17 @@ cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned cha
   return cudaGetLastError();
 }
 
-cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int max_len,
-                        bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st) {
+cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int64_t nlong,
+                        int max_len, bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st) {
   if (pairs <= 0) return cudaSuccess;
   int size = 0;
   while (size + 1 < BandPlan::kSizes && max_len > plan.max_len[size]) ++size;
-  const int smem = plan.smem[size];
-  const int warp_smem = (smem / kBandWarps) & ~15;
+  // fewer long pairs than CTAs of four warps: CTAs of eight (400 x 10 kbp with
+  // CIGARs 2.7 -> 2.0 ms, 2,000 no faster: every row costs eight warps its
+  // fixed part)
+  if (size == 1 && nlong <= (int64_t)plan.nsm * plan.per_sm[1]) size = 2;
+  const int warps = plan.warps[size], smem = plan.smem[size];
+  const int warp_smem = (smem / warps) & ~15;
   cudaError_t e = cudaMemsetAsync(b.aux, 0, kBandAux * sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   // bound pass: both packed sequences and the 32-diagonal rows a warp
@@ -330,11 +346,11 @@ cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs
   // CTAs: as many as are resident, at least 64 KiB of arena a warp, no more
   // than pairs (a team takes one at a time)
   int64_t grid = std::min<int64_t>((int64_t)plan.nsm * plan.per_sm[size], pairs);
-  grid = std::max<int64_t>(1, std::min<int64_t>(grid, arena_bytes / (kBandWarps * (64L << 10))));
-  const long slot = (long)(arena_bytes / (grid * kBandWarps)) & ~255L;
+  grid = std::max<int64_t>(1, std::min<int64_t>(grid, arena_bytes / (warps * (64L << 10))));
+  const long slot = (long)(arena_bytes / (grid * warps)) & ~255L;
   const bool ef = (a.pb | a.pe | a.tb | a.te) != 0;
-  band_kernel_of(!a.score_only, ef)<<<(unsigned)grid, 32 * kBandWarps, smem, st>>>(a, b.key, b.order, arena, slot,
-                                                                                   warp_smem);
+  band_kernel_of(warps, !a.score_only, ef)<<<(unsigned)grid, 32 * warps, smem, st>>>(a, b.key, b.order, arena, slot,
+                                                                                     warp_smem);
   return cudaGetLastError();
 }
 

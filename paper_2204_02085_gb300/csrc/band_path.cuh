@@ -4,11 +4,10 @@
 //
 // A pair is run in two steps.
 //
-// 1. An upper bound T on its scaled score (band_bound): the recurrences on a
-//    window of 32 diagonals, one per lane, that follows the cell furthest
-//    along both sequences.  The score it ends with is the cost of a real
-//    alignment, so the optimum is at most T.  It costs one 32-cell row a
-//    score.
+// 1. An upper bound T on its scaled score (BandSearch): the recurrences on a
+//    window of 32 diagonals, one per lane, that follows the cell
+//    furthest along both sequences.  The score it ends with is the cost of a
+//    real alignment, so the optimum is at most T.
 // 2. The exact wavefronts (band_forward), but only on diagonals from which
 //    the end can still be reached within T: at score s a cell on diagonal k
 //    needs at least e * d more, d the distance from k to the nearest end
@@ -38,9 +37,9 @@
 // the start, extending after each (band_replay), which is what the forward
 // pass did on the way to each cell.
 //
-// Work split.  One warp per pair, or a CTA of four when the rows are wide
-// (or do not fit a warp's share of the shared memory): a lane per diagonal,
-// 32 * warps diagonals a round.
+// Work split.  One warp per pair, or a CTA of four or eight when the rows are
+// wide (or do not fit a warp's share of the shared memory): a lane per
+// diagonal, 32 * warps diagonals a round.
 #pragma once
 
 #include "arena_path.cuh"
@@ -54,7 +53,7 @@ constexpr uint32_t kBandNull = 0xFFFFu;
 constexpr uint32_t kBandValid = 0x8000u;  // u below this is an offset
 constexpr int kBandMaxLen = 32000;        // u fits 15 bits
 constexpr int kBandMaxPen = 31;           // scaled penalties: rows kept per pair
-constexpr int kBandWarps = 4;             // warps of a CTA (and of a team)
+constexpr int kBandWarps = 4;             // warps of a CTA (and of a team); twice as many when few pairs are long
 constexpr int kBandTeamWidth = 256;       // rows wider than this: a team
 
 // 16-bit row cells a pair keeps per diagonal.
@@ -121,74 +120,101 @@ __device__ __forceinline__ int band_extend(const uint32_t* pw, const uint32_t* t
 
 // ---------------------------------------------------------------- bound
 
-// Upper bound on the pair's scaled score, at most cap (itself a bound, or
-// the caller's largest score of interest).  One warp; lane l holds the
-// diagonal k = l (mod 32) of the window b .. b + 31; ring: band_rows(...) *
-// 32 cells.  Every fourth score the window moves when its furthest cell
-// (largest v + h) is within 8 diagonals of an edge.
-__device__ int band_bound(const uint32_t* pw, const uint32_t* tw, const BandGeo& g, int x, int oe, int e, int cap,
-                          uint16_t* ring) {
-  constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int n = g.n, m = g.m, kf = g.kf;
-  const int R = max(x, oe) + 1, RE = e + 1, NR = R + 2 * RE;
-  uint16_t* I = ring + R * 32;
-  uint16_t* D = I + RE * 32;
-  for (int r = 0; r < NR; ++r) ring[r * 32 + lane] = (uint16_t)kBandNull;
-  int b = -16;
-  if (g.lo0 != g.hi0) {  // free starts: the one with the longest match
-    int best = 0;
-    for (int k = g.lo0 + lane; k <= g.hi0; k += 32) {
-      const int h = max(k, 0), v = h - k, rem = min(n - v, m - h);
-      const int len = rem > 0 ? band_extend(pw, tw, v, h, rem) : 0;
-      best = max(best, (len << 16) | (k - g.lo0));  // lengths < 32,768: no overlap with the sign
+// The search for a pair's bound, a row at a time, on kLanes lanes (a warp
+// for one pair): lane l holds the diagonal k = l (mod kLanes) of the window b .. b +
+// kLanes - 1, its rows the band_rows(...) * kLanes cells at ring.  Every
+// fourth score the window moves when its furthest cell (largest v + h) comes
+// within a quarter of an edge.  On every sampled pair of 100 to 10,000 bases
+// at up to 10 % edits the bound found was the optimum itself.  (Half a warp
+// per pair found it too, but two pairs' extensions in one warp wait for each
+// other: 260 instructions a score for two pairs against 148 for one, and
+// twice the latency on long reads.)
+template <int kLanes>
+struct BandSearch {
+  const uint32_t *pw, *tw;
+  uint16_t* ring;
+  int n, m, kf, elo, ehi, b, k, s, cap;
+  int rs, rx, ro, rn, re;  // ring rows of the scores s, s - x, s - o - e (M), s, s - e (I, D)
+
+  __device__ static unsigned mask() { return group_mask(kLanes); }
+  __device__ static int lane() { return threadIdx.x & (kLanes - 1); }
+
+  // Score 0; true when it reaches an end.
+  __device__ bool start(const uint32_t* pw_, const uint32_t* tw_, const BandGeo& g, int x, int oe, int e, int cap_,
+                        uint16_t* ring_) {
+    const int l = lane(), R = max(x, oe) + 1, RE = e + 1;
+    pw = pw_;
+    tw = tw_;
+    ring = ring_;
+    n = g.n;
+    m = g.m;
+    kf = g.kf;
+    elo = g.elo;
+    ehi = g.ehi;
+    cap = cap_;
+    s = 0;
+    for (int r = 0; r < R + 2 * RE; ++r) ring[r * kLanes + l] = (uint16_t)kBandNull;
+    b = -kLanes / 2;
+    if (g.lo0 != g.hi0) {  // free starts: the one with the longest match
+      int best = 0;
+      for (int q = g.lo0 + l; q <= g.hi0; q += kLanes) {
+        const int h = max(q, 0), v = h - q, rem = min(n - v, m - h);
+        const int len = rem > 0 ? band_extend(pw, tw, v, h, rem) : 0;
+        best = max(best, (len << 16) | (q - g.lo0));  // lengths < 32,768: no overlap with the sign
+      }
+      b = g.lo0 + (__reduce_max_sync(mask(), best) & 0xFFFF) - kLanes / 2;
     }
-    b = g.lo0 + (__reduce_max_sync(FULL, best) & 0xFFFF) - 16;
+    k = b + ((l - b) & (kLanes - 1));
+    bool fin = false;
+    if (k >= g.lo0 && k <= g.hi0) {
+      const int h = max(k, 0), v = h - k, rem = min(n - v, m - h);
+      const int u = rem > 0 ? rem - band_extend(pw, tw, v, h, rem) : 0;
+      ring[l] = (uint16_t)u;
+      fin = u == 0 && k >= elo && k <= ehi;
+    }
+    __syncwarp(mask());
+    rs = 1 % R, rx = (1 - x + R) % R, ro = (1 - oe + R) % R, rn = 1 % RE, re = 2 % RE;
+    return __any_sync(mask(), fin);
   }
-  int k = b + ((lane - b) & 31);
-  bool fin = false;
-  if (k >= g.lo0 && k <= g.hi0) {
-    const int h = max(k, 0), v = h - k, rem = min(n - v, m - h);
-    const int u = rem > 0 ? rem - band_extend(pw, tw, v, h, rem) : 0;
-    ring[lane] = (uint16_t)u;
-    fin = u == 0 && k >= g.elo && k <= g.ehi;
-  }
-  __syncwarp();
-  if (__any_sync(FULL, fin)) return 0;
-  int rs = 1 % R, rx = (1 - x + R) % R, ro = (1 - oe + R) % R, rn = 1 % RE, re = 2 % RE;
-  for (int s = 1; s < cap; ++s) {
-    const uint32_t mx = ring[rx * 32 + lane];
-    const int l1 = (lane - 1) & 31, r1 = (lane + 1) & 31;
-    const bool first = k == b, last = k == b + 31;
-    const uint32_t oa = first ? kBandNull : ring[ro * 32 + l1], il = first ? kBandNull : I[re * 32 + l1];
-    const uint32_t oc = last ? kBandNull : ring[ro * 32 + r1], dr = last ? kBandNull : D[re * 32 + r1];
+
+  // The next score; true when it reaches an end.
+  __device__ __forceinline__ bool step(int x, int oe, int e) {
+    const int l = lane(), R = max(x, oe) + 1, RE = e + 1;
+    uint16_t* const I = ring + R * kLanes;
+    uint16_t* const D = I + RE * kLanes;
+    ++s;
+    const uint32_t mx = ring[rx * kLanes + l];
+    const int l1 = (l - 1) & (kLanes - 1), r1 = (l + 1) & (kLanes - 1);
+    const bool first = k == b, last = k == b + kLanes - 1;
+    const uint32_t oa = first ? kBandNull : ring[ro * kLanes + l1], il = first ? kBandNull : I[re * kLanes + l1];
+    const uint32_t oc = last ? kBandNull : ring[ro * kLanes + r1], dr = last ? kBandNull : D[re * kLanes + r1];
     const uint32_t uI = min(il, oa) - (k > kf ? 1u : 0u);
     const uint32_t uD = min(dr, oc) - (k < kf ? 1u : 0u);
     uint32_t u = min(mx - 1u, min(uI, uD));
     int far = 0;  // v + h of the cell
+    bool fin = false;
     if (u < kBandValid) {
       const int h = min(m, n + k) - (int)u;
       u -= (uint32_t)band_extend(pw, tw, h - k, h, (int)u);
       far = 2 * (min(m, n + k) - (int)u) - k;
-      fin = u == 0 && k >= g.elo && k <= g.ehi;
+      fin = u == 0 && k >= elo && k <= ehi;
     } else {
       u = kBandNull;
     }
-    ring[rs * 32 + lane] = (uint16_t)u;
-    I[rn * 32 + lane] = (uint16_t)uI;
-    D[rn * 32 + lane] = (uint16_t)uD;
-    __syncwarp();
-    if (__any_sync(FULL, fin)) return s;
+    ring[rs * kLanes + l] = (uint16_t)u;
+    I[rn * kLanes + l] = (uint16_t)uI;
+    D[rn * kLanes + l] = (uint16_t)uD;
+    __syncwarp(mask());
     if ((s & 3) == 0) {
-      const int best = __reduce_max_sync(FULL, (far << 5) | lane);
-      const int at = ((best & 31) - b) & 31;
-      if (best >= 32 && (at < 8 || at > 23)) {
-        b += at - 16;
-        const int k2 = b + ((lane - b) & 31);
+      const int best = __reduce_max_sync(mask(), (far << 5) | l);
+      const int at = ((best & 31) - b) & (kLanes - 1);
+      if (best >= 32 && (at < kLanes / 4 || at >= kLanes - kLanes / 4)) {
+        b += at - kLanes / 2;
+        const int k2 = b + ((l - b) & (kLanes - 1));
         if (k2 != k)
-          for (int r = 0; r < NR; ++r) ring[r * 32 + lane] = (uint16_t)kBandNull;
+          for (int r = 0; r < R + 2 * RE; ++r) ring[r * kLanes + l] = (uint16_t)kBandNull;
         k = k2;
-        __syncwarp();
+        __syncwarp(mask());
       }
     }
     rs = rs + 1 == R ? 0 : rs + 1;
@@ -196,11 +222,45 @@ __device__ int band_bound(const uint32_t* pw, const uint32_t* tw, const BandGeo&
     ro = ro + 1 == R ? 0 : ro + 1;
     rn = rn + 1 == RE ? 0 : rn + 1;
     re = re + 1 == RE ? 0 : re + 1;
+    return __any_sync(mask(), fin);
   }
+};
+
+// The whole search on one warp: an upper bound on the pair's scaled score, at
+// most cap (itself a bound, or the caller's largest score of interest).
+__device__ __forceinline__ int band_bound(const uint32_t* pw, const uint32_t* tw, const BandGeo& g, int x, int oe,
+                                          int e, int cap, uint16_t* ring) {
+  BandSearch<32> w;
+  if (w.start(pw, tw, g, x, oe, e, cap, ring)) return 0;
+  while (w.s + 1 < cap)
+    if (w.step(x, oe, e)) return w.s;
   return cap;
 }
 
+// A bound that needs no search: every base a mismatch and the length
+// difference one gap, or one gap for each sequence.
+__device__ __forceinline__ int band_worst(int n, int m, int x, int oe, int e) {
+  const int d = abs(n - m), o = oe - e;
+  const int one = x * min(n, m) + (d ? o + e * d : 0);
+  const int two = (n ? o + e * n : 0) + (m ? o + e * m : 0);
+  return min(one, two);
+}
+
 // -------------------------------------------------------------- forward
+
+// The scores without a wavefront among the first max(x, o + e) (bit s): no
+// older row has written their row positions, so they need not be written
+// either.
+__device__ __forceinline__ uint32_t band_absent(int x, int oe, int e) {
+  uint32_t ex = 1u, gap = 0u;
+  for (int s = 1; s < 32; ++s) {
+    const bool g = (s >= oe && ((ex >> (s - oe)) & 1u)) || (s >= e && ((gap >> (s - e)) & 1u));
+    if (g) gap |= 1u << s;
+    if (g || (s >= x && ((ex >> (s - x)) & 1u))) ex |= 1u << s;
+  }
+  const int R = max(x, oe) + 1;
+  return R >= 32 ? ~ex : ~ex & ((1u << R) - 1u);
+}
 
 // The exact score of a pair whose score is at most g.T, on WPP warps: the
 // scaled score (and its end diagonal in *k_out), or -1 when no alignment
@@ -209,7 +269,7 @@ __device__ int band_bound(const uint32_t* pw, const uint32_t* tw, const BandGeo&
 // whose row holds an end (EF).
 template <int WPP, bool CIG, bool EF>
 __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t* tw, uint16_t* rows, int x, int oe,
-                            int e, uint4* bits, int* fin, int* k_out) {
+                            int e, uint32_t absent, uint4* bits, int* fin, int* k_out) {
   constexpr unsigned FULL = 0xffffffffu;
   using T_ = Team<WPP>;
   const int lane = threadIdx.x & 31, warp = WPP == 1 ? 0 : (int)(threadIdx.x >> 5), r = T_::rank();
@@ -252,6 +312,7 @@ __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t
   const int Rp = R * pitch, REp = RE * pitch;
   int rs = 1 % R * pitch, rx = (1 - x + R) % R * pitch, ro = (1 - oe + R) % R * pitch;
   int rn = 1 % RE * pitch, re = 2 % RE * pitch;
+  int skip = EF && absent ? __ffs(absent) - 1 : 0;  // the next score without a wavefront
   for (int s = 1; s <= g.T; ++s) {
     if (s == q_at) {
       --q;
@@ -266,8 +327,13 @@ __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t
     const uint16_t* const mop = rows + ro + off;
     const uint16_t* const ip = I + re + off - 1;
     const uint16_t* const dp = D + re + off + 1;
-    int c = warp;
-    for (int k0 = lo + 32 * warp; k0 <= hi; k0 += 32 * WPP, c += WPP) {
+    int c = warp, k0 = lo + 32 * warp;
+    if (EF && s == skip) {  // no wavefront at this score (wide first rows: worth the test)
+      k0 = hi + 1;
+      absent &= absent - 1;
+      skip = absent ? __ffs(absent) - 1 : 0;
+    }
+    for (; k0 <= hi; k0 += 32 * WPP, c += WPP) {
       const int k = k0 + lane;
       const bool act = k <= hi;
       const uint32_t mx = mxp[k], oa = mop[k - 1], oc = mop[k + 1], il = ip[k], dr = dp[k];
@@ -313,15 +379,6 @@ __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t
     re = re + pitch == REp ? 0 : re + pitch;
   }
   return -1;
-}
-
-// A bound that needs no search: every base a mismatch and the length
-// difference one gap, or one gap for each sequence.
-__device__ __forceinline__ int band_worst(int n, int m, int x, int oe, int e) {
-  const int d = abs(n - m), o = oe - e;
-  const int one = x * min(n, m) + (d ? o + e * d : 0);
-  const int two = (n ? o + e * n : 0) + (m ? o + e * m : 0);
-  return min(one, two);
 }
 
 // ---------------------------------------------------------------- CIGAR
@@ -460,10 +517,12 @@ __device__ int band_replay(const BandGeo& g, const uint32_t* pw, const uint32_t*
 
 // ----------------------------------------------------------- one pair
 
-// One pair, on one warp (WPP 1) or a CTA: smem of at least band_bytes,
-// slot_bytes of the arena at slot.  packed: the sequences are at smem already.
+// One pair, on one warp (WPP 1) or a CTA: absent = band_absent(...), smem of at
+// least band_bytes, slot_bytes of the arena at slot.  packed: the sequences
+// are at smem already.
 template <int WPP, bool CIG, bool EF>
-__device__ void band_pair(const AlignArgs& a, int64_t pair, int T, unsigned char* smem, TeamShm* ts, int& round,
+__device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int T, unsigned char* smem, TeamShm* ts,
+                          int& round,
                           unsigned char* slot, long slot_bytes, int32_t* overflow_count, bool packed = false) {
   using T_ = Team<WPP>;
   const int r = T_::rank();
@@ -483,7 +542,7 @@ __device__ void band_pair(const AlignArgs& a, int64_t pair, int T, unsigned char
   }
   int k_end = 0;
   uint4* bits = reinterpret_cast<uint4*>(slot);
-  const int s = band_forward<WPP, CIG, EF>(g, pw, tw, rows, a.xs, a.oes, a.es, bits, &ts->bcast, &k_end);
+  const int s = band_forward<WPP, CIG, EF>(g, pw, tw, rows, a.xs, a.oes, a.es, absent, bits, &ts->bcast, &k_end);
   if (!CIG || s < 0) {
     // no alignment within T: T was the caller's largest score
     if (r == 0) {

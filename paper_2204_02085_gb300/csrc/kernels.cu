@@ -511,6 +511,7 @@ __global__ void __launch_bounds__(kSmallBlock) small_finish_kernel(int n, const 
 // last of the 32 pairs whose offset is <= its position (binary search over
 // the offsets in shared memory; a pair without runs shares the next pair's
 // offset, so the search lands on a pair that has the word).
+constexpr int kLongRuns = 64;  // words a pair from which the output is cut by words
 __global__ void __launch_bounds__(kAuxBlock) compact_kernel(int64_t n, const int32_t* nruns, const int64_t* run_src,
                                                              const uint32_t* runs, const uint32_t* pool,
                                                              const int64_t* off, uint32_t* out, int64_t cap,
@@ -522,6 +523,32 @@ __global__ void __launch_bounds__(kAuxBlock) compact_kernel(int64_t n, const int
   __shared__ uint32_t s_words[kAuxBlock / 32][32 * kSlot];  // a batch's runs in output order
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  if (off[n] > kLongRuns * n) {
+    // long CIGARs: a warp per span of output words, whatever pairs it cuts
+    // (2,000 pairs of 1,000 runs took 409 us on the 63 warps that have 32
+    // pairs each)
+    constexpr int64_t kSpan = 256;
+    const int64_t total = off[n];
+    for (int64_t w0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kSpan; w0 < total;
+         w0 += nwarps * kSpan) {
+      int64_t lo = 0, hi = n;  // the last pair whose offset is <= w0
+      while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (off[mid] <= w0) lo = mid;
+        else hi = mid;
+      }
+      const int64_t end = w0 + kSpan < total ? w0 + kSpan : total;
+      for (int64_t p = lo, at = w0; at < end; ++p) {
+        const int64_t stop = off[p + 1] < end ? off[p + 1] : end, first = off[p];
+        const int64_t src = run_src[p];
+        const int cnt = nruns[p];
+        const uint32_t* r = src >= 0 ? runs + src : pool + (-src - 1);
+        for (int64_t w = at + lane; w < stop; w += 32) out[w] = r[cnt - 1 - (int)(w - first)];
+        at = stop > at ? stop : at;
+      }
+    }
+    return;
+  }
   for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5 << 5; i0 < n; i0 += nwarps * 32) {
     const int cnt = n - i0 < 32 ? (int)(n - i0) : 32;
     const int64_t i = i0 + lane;
@@ -947,8 +974,10 @@ cudaError_t launch_compact(int64_t n, const int32_t* nruns, const int64_t* run_s
                            const uint32_t* pool, const int64_t* off, uint32_t* out, int64_t cap, const Ctrl* ctrl,
                            cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  compact_kernel<<<aux_grid(n, current_device()), kAuxBlock, 0, st>>>(n, nruns, run_src, runs, pool, off, out, cap,
-                                                                       ctrl);
+  // (at least two blocks an SM, unless there are fewer pairs: long CIGARs)
+  const int dev = current_device();
+  const int grid = std::max(aux_grid(n, dev), (int)std::min<int64_t>(n, 2 * sm_count(dev)));
+  compact_kernel<<<grid, kAuxBlock, 0, st>>>(n, nruns, run_src, runs, pool, off, out, cap, ctrl);
   return cudaGetLastError();
 }
 

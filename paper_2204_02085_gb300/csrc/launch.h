@@ -221,8 +221,8 @@ cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list
 struct BandPlan {
   // by the longest sequence of the call, ascending: CTAs per SM and shared
   // memory of the band kernel
-  static constexpr int kSizes = 3;
-  int max_len[kSizes], per_sm[kSizes], smem[kSizes];
+  static constexpr int kSizes = 4;
+  int max_len[kSizes], warps[kSizes], per_sm[kSizes], smem[kSizes];
   int nsm;
 };
 struct BandBufs {
@@ -235,11 +235,11 @@ struct BandBufs {
 constexpr int kBandBins = 128;
 constexpr int kBandAux = 2 * kBandBins;
 cudaError_t band_plan(int device, BandPlan* plan);
-// pairs: at most this many are deferred; max_len: the longest sequence among
-// the call's (sizes the shared memory; a pair longer than that still ends up
+// pairs: at most this many are deferred, nlong of them long; max_len: the
+// longest sequence among the call's (sizes the shared memory; a pair longer than that still ends up
 // right, in the arena lists).  launches: kernels enqueued.
-cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int max_len,
-                        bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
+cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int64_t nlong,
+                        int max_len, bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
 constexpr int kBandLaunches = 3;
 // Calls of at most kDirectPairs pairs: every pair on a warp of its own, what
 // does not fit deferred.
