@@ -100,15 +100,31 @@ __global__ void validate_kernel(int64_t n, const int64_t* poff, const int32_t* p
     te = max(te, to + tl);
     ml = max(ml, max(pl, tl));
   }
+  // one atomic a block and extent: one a warp on the same three words took 21
+  // us for any batch that fills the grid
+  __shared__ long long s_pe[kAuxBlock / 32], s_te[kAuxBlock / 32];
+  __shared__ int s_ml[kAuxBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   pe = warp_max64(pe);
   te = warp_max64(te);
   ml = __reduce_max_sync(0xffffffffu, ml);
-  if ((threadIdx.x & 31) == 0) {
-    if (pe) atomicMax(&ctrl->pat_extent, pe);
-    if (te) atomicMax(&ctrl->txt_extent, te);
-    if (ml) atomicMax(&ctrl->max_len, ml);
+  if (lane == 0) {
+    s_pe[warp] = pe;
+    s_te[warp] = te;
+    s_ml[warp] = ml;
   }
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicExch(&ctrl->bad_input, 1);
+  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctrl->bad_input, 1);
+  __syncthreads();
+  if (warp == 0) {
+    pe = warp_max64(lane < kAuxBlock / 32 ? s_pe[lane] : 0);
+    te = warp_max64(lane < kAuxBlock / 32 ? s_te[lane] : 0);
+    ml = __reduce_max_sync(0xffffffffu, lane < kAuxBlock / 32 ? s_ml[lane] : 0);
+    if (lane == 0) {
+      if (pe) atomicMax(&ctrl->pat_extent, pe);
+      if (te) atomicMax(&ctrl->txt_extent, te);
+      if (ml) atomicMax(&ctrl->max_len, ml);
+    }
+  }
 }
 
 // -------------------------------------------------------------------- scan

@@ -16,7 +16,7 @@ constexpr int kLaneBandSmem = 96 * 1024;       // more than any variant asks for
 // The lane kernels' ordering pass: a block per group of pairs
 // (lane_band.cuh).
 template <int LMAX, int GROUP, int PER>
-__global__ void __launch_bounds__(GROUP / PER, GROUP >= 512 ? 2 : 1)
+__global__ void __launch_bounds__(GROUP / PER, LMAX <= 127 && GROUP == 512 ? 4 : GROUP >= 512 ? 2 : 1)
     lane_order_kernel(const AlignArgs a, int cap, int walk) {
   extern __shared__ __align__(16) unsigned char smem[];
   lane_order_body<LMAX, GROUP, PER>(a, cap, walk != 0, smem);
@@ -45,12 +45,18 @@ __global__ void __launch_bounds__(32 * kLaneBandWarps) lane_band_kernel(const Al
   lane_band_body<U, LMAX, PX, POE, PE, GROUP>(a, lb, smem);
 }
 
-// Pairs of a group: 1,024 (512 above 127 bases) where whole groups fill the
-// GPU, so that a group sorts well; 128 for smaller calls, whose time is the
-// latency of a group: 20,000 pairs of 60 bases took 165 us in groups of 1,024.
+// Pairs of a group of the ordering pass, two a thread.  1,024 where pairs are
+// bounded one by one: larger groups sort better (5M pairs at E = 4 %: 2.05 ms
+// a call against 2.13 in groups of 512).  512 where they are sorted by end
+// diagonal alone, which 512 do as well, in four blocks an SM that wait for
+// each other's loads less (E = 2 %: 0.93 ms against 0.96), and above 127
+// bases, whose planes are larger.  128, one a thread, for calls of up to 16K
+// pairs, whose time is a group's latency.
 constexpr int kSmallGroup = 128;
-constexpr int64_t kSmallGroupPairs = 1 << 17;
-int group_for(int lmax, int64_t n) { return n <= kSmallGroupPairs ? kSmallGroup : lane_group_of(lmax); }
+constexpr int64_t kSmallGroupPairs = 1 << 14;
+int group_for(int lmax, int64_t n, bool walk) {
+  return n <= kSmallGroupPairs ? kSmallGroup : lmax <= 127 && walk ? 1024 : 512;
+}
 
 using LaneBandKernel = void (*)(const AlignArgs, const LaneBand);
 
@@ -59,12 +65,14 @@ using LaneBandKernel = void (*)(const AlignArgs, const LaneBand);
 // run time.
 LaneBandKernel lane_band_kernel_of(int lmax, int group, int x, int oe, int e) {
   const bool p241 = x == 2 && oe == 4 && e == 1, p111 = x == 1 && oe == 1 && e == 1;
-  if (lmax <= 127 && group == 1024)
-    return p241   ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 1024>
-           : p111 ? lane_band_kernel<uint8_t, 127, 1, 1, 1, 1024>
-                  : lane_band_kernel<uint8_t, 127, 0, 0, 0, 0>;
-  if (lmax <= 127)
-    return p241 ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 0> : lane_band_kernel<uint8_t, 127, 0, 0, 0, 0>;
+  if (lmax <= 127) {
+    if (p241)
+      return group == 1024  ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 1024>
+             : group == 512 ? lane_band_kernel<uint8_t, 127, 2, 4, 1, 512>
+                            : lane_band_kernel<uint8_t, 127, 2, 4, 1, 0>;
+    return p111 && group == 512 ? lane_band_kernel<uint8_t, 127, 1, 1, 1, 512>
+                                : lane_band_kernel<uint8_t, 127, 0, 0, 0, 0>;
+  }
   if (lmax <= 191)
     return p241 ? lane_band_kernel<uint8_t, 191, 2, 4, 1, 0> : lane_band_kernel<uint8_t, 191, 0, 0, 0, 0>;
   return lane_band_kernel<uint16_t, 255, 0, 0, 0, 0>;
@@ -95,19 +103,25 @@ cudaError_t launch_order_as(const AlignArgs& a, int grid, int cap, int walk, cud
   return cudaGetLastError();
 }
 
+// grid[0], [1], [2]: groups of 1,024 (up to 127 bases), 512 and 128.
 template <int LMAX>
-cudaError_t plan_orders(int device, int grid[2]) {
-  const cudaError_t e = plan_order<LMAX, lane_group_of(LMAX), 2>(device, &grid[0]);
-  return e != cudaSuccess ? e : plan_order<LMAX, kSmallGroup, 1>(device, &grid[1]);
+cudaError_t plan_orders(int device, int grid[3]) {
+  cudaError_t e;
+  if constexpr (LMAX <= 127)
+    if ((e = plan_order<LMAX, 1024, 2>(device, &grid[0]))) return e;
+  if ((e = plan_order<LMAX, 512, 2>(device, &grid[1]))) return e;
+  return plan_order<LMAX, kSmallGroup, 1>(device, &grid[2]);
 }
 
 template <int LMAX>
 cudaError_t launch_order(const AlignArgs& a, const ShortVariant& v, int group, int cap, int walk, cudaStream_t st) {
   const int64_t groups = (a.n + group - 1) / group;
-  const int most = v.order_grid[group == kSmallGroup ? 1 : 0];
+  const int most = v.order_grid[group == 1024 ? 0 : group == 512 ? 1 : 2];
   const int grid = groups < most ? (int)groups : most;
-  return group == kSmallGroup ? launch_order_as<LMAX, kSmallGroup, 1>(a, grid, cap, walk, st)
-                              : launch_order_as<LMAX, lane_group_of(LMAX), 2>(a, grid, cap, walk, st);
+  if constexpr (LMAX <= 127)
+    if (group == 1024) return launch_order_as<LMAX, 1024, 2>(a, grid, cap, walk, st);
+  return group == 512 ? launch_order_as<LMAX, 512, 2>(a, grid, cap, walk, st)
+                      : launch_order_as<LMAX, kSmallGroup, 1>(a, grid, cap, walk, st);
 }
 
 }  // namespace
@@ -120,7 +134,7 @@ cudaError_t plan_lane_band(int device, ShortVariant* v, int lmax, int store) {
   v->kind = 1;
   const int pens[3][3] = {{2, 4, 1}, {1, 1, 1}, {0, 0, 0}};
   for (int q = 0; q < 3; ++q) {
-    for (int group : {kSmallGroup, lane_group_of(lmax)}) {
+    for (int group : {kSmallGroup, 512, 1024}) {
       const LaneBandKernel k = lane_band_kernel_of(lmax, group, pens[q][0], pens[q][1], pens[q][2]);
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLaneBandSmem);
       if (e != cudaSuccess) return e;
@@ -215,12 +229,12 @@ bool lane_ordered(const AlignArgs& a, const ShortVariant& v) {
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st) {
   LaneBand lb;
   lane_band_plan(a, v, &lb);
-  const int group = lb.group = group_for(v.max_len, a.n);
-  const int64_t groups = (a.n + group - 1) / group;
   // bounds above the store's mean "deferred" (or over the caller's largest
   // score): the greedy walk stops there
   const int cap = std::max(0, std::min(lb.s_store, a.s_cap));
   const int walk = lb.s_store >= a.lane_sort_min ? 1 : 0;
+  const int group = lb.group = group_for(v.max_len, a.n, walk != 0);
+  const int64_t groups = (a.n + group - 1) / group;
   const cudaError_t e = v.max_len <= 127   ? launch_order<127>(a, v, group, cap, walk, st)
                         : v.max_len <= 191 ? launch_order<191>(a, v, group, cap, walk, st)
                                            : launch_order<255>(a, v, group, cap, walk, st);

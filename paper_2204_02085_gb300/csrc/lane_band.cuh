@@ -254,7 +254,8 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
       const int64_t pair = gi * G + q * kThreads + threadIdx.x;
       uint32_t* const P = S.planes[q * (kThreads / 32) + warp] + lane;
       bool active = pair < a.n;
-      int n = 0, m = 0, T = cap, kq = kLaneKeys - 1;
+      int T = cap, kq = kLaneKeys - 1;
+      int n = 0, m = 0;
       int64_t po = 0, to = 0;
       if (active) {
         n = a.plen[pair];
@@ -550,7 +551,7 @@ __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBan
           // pending extensions, and the row's choices: mismatch taken,
           // insertion over deletion, I extended, D extended
           uint32_t pend = 0, cx = 0, ci = 0, ce = 0, cd = 0, bit = 1;
-#pragma unroll 2
+#pragma unroll 4
           for (int k = lo; k <= hi; ++k) {
             const uint32_t oc = mo[(k + 1) * 32], dn = dr[(k + 1) * 32], inext = ir[k * 32];
             const uint32_t ux = (uint32_t)mx[k * 32] - 1u;

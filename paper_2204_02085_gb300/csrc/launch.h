@@ -75,13 +75,11 @@ struct AlignArgs {
 };
 
 // Packed 16-base words per sequence of at most lmax bases the lane kernel in
-// call order reads; 32-base words per bit plane the one on ordered input
-// reads (a position past the last base included); and the pairs the ordering
-// sorts together (two a thread; longer sequences need more registers and
-// shared memory each).
+// call order reads, and 32-base words per bit plane the one on ordered input
+// reads (a position past the last base included).
 __host__ __device__ constexpr int lane_words_of(int lmax) { return lmax / 16 + 2; }
 __host__ __device__ constexpr int lane_plane_words(int lmax) { return lmax / 32 + 1; }
-__host__ __device__ constexpr int lane_group_of(int lmax) { return lmax <= 127 ? 1024 : 512; }
+// Most pairs the ordering sorts together.
 constexpr int kLaneGroupMax = 1024;
 
 // longest sequence handled by a one-warp arena team; longer pairs go to a
@@ -118,7 +116,7 @@ struct ShortVariant {
   // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's (large
   // and small groups).
   // `kernel` takes call order (null: the variant runs on ordered input only)
-  int band_store, band_cell, band_grid[3], order_grid[2];
+  int band_store, band_cell, band_grid[3], order_grid[3];
   size_t band_smem;
 };
 struct ShortPlan {

@@ -97,3 +97,28 @@ def test_lane_band_stores(pkg, oracle_mod, monkeypatch, store, walk_from):
         got = al.align(b, (4, 6, 2))
         assert al.variant_name(al.timing()["short_variant"]) == store
         _check(got, want)
+
+
+@pytest.mark.parametrize("count", [16384, 16385, 17408, 17411])
+@pytest.mark.parametrize("pen", [(4, 6, 2), (1, 0, 1), (5, 8, 3)])
+@pytest.mark.parametrize("walk_from", ["0", "99"])
+def test_lane_band_groups(pkg, oracle_mod, monkeypatch, count, pen, walk_from):
+    """The ordering's group sizes: the last batch of small groups, the first of
+    512 and 1,024, whole and ragged last groups of each."""
+    from paper_2204_02085_gb300 import synth
+
+    monkeypatch.setenv("WFA_GPU_LANE_SORT_MIN", walk_from)
+    b = synth.from_pairs(_pairs(127, count, 23))
+    want = oracle_mod.wfa_batch(b, pen, nthreads=8)
+    with pkg.Aligner(0, 1 << 28) as al:
+        _check(al.align(b, pen), want)
+
+
+@pytest.mark.parametrize("longest", [191, 255])
+def test_lane_band_groups_of_wide_classes(pkg, oracle_mod, longest):
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.from_pairs(_pairs(longest, 16901, longest))
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=8)
+    with pkg.Aligner(0, 1 << 28) as al:
+        _check(al.align(b, (4, 6, 2)), want)
