@@ -149,9 +149,9 @@ __global__ void __launch_bounds__(kPlaceBlock) place_kernel(const AlignArgs a, c
 // Persistent CTAs, pairs from queues.  Bound by instruction issue (82 % of
 // the issue slots busy on mixed lengths).  Calls on the arena kernels before
 // -> with the bound and the band: 200,000 mixed-length pairs (100-2,000 bp)
-// 21.8 -> 12.7 ms, 4,000 x 10 kbp score-only 25.8 -> 6.6 ms, 2,000 x 10 kbp
-// with CIGARs 17.7 -> 5.5 ms, 200,000 reads in 100-300 bp windows with free
-// text ends 42.3 -> 2.1 ms.
+// 21.8 -> 11.8 ms, 4,000 x 10 kbp score-only 25.8 -> 6.6 ms, 2,000 x 10 kbp
+// with CIGARs 17.7 -> 5.2 ms, 200,000 reads in 100-300 bp windows with free
+// text ends 42.3 -> 2.0 ms.
 // WARPS: a CTA of four, or of eight when few pairs are long (launch_band).
 template <bool CIG, bool EF, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
@@ -197,7 +197,8 @@ __global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
 // Small calls: a warp per pair from its bytes to its CIGAR, the bound and the
 // exact wavefronts one after the other, every pair of the call at once.  The
 // time is one pair's latency: 37 reads of 100 bases took the ordering pass
-// and the lane kernel 38 us (one lane runs a pair's cells in turn).  Pairs
+// and the lane kernel 38 us (one lane runs a pair's cells in turn); the call
+// went from 206 to 48 us with this kernel and its outputs in one wait.  Pairs
 // longer than kDirectMaxLen, or whose rows do not fit, are deferred.
 constexpr int kDirectMaxLen = 512;
 template <bool CIG, bool EF>
@@ -264,13 +265,15 @@ constexpr int kMaxSmem = 227 * 1024;
 
 cudaError_t band_plan(int device, BandPlan* plan) {
   cudaError_t e;
-  // CTAs an SM (a CTA costs 1 KB of shared memory besides its own): under
-  // 4/6/2 (9 rows, 18 bytes a diagonal) a team's rows may be about 1,500,
-  // 1,900 and 3,900 diagonals wide: reads of 2,048, 12,000 and 32,000 bases
-  // at up to some 10, 5 and 4 % edits.  Eight CTAs of four warps are what 64
-  // registers allow; the second size has a form with half as many CTAs of
-  // eight warps, the third only that.
-  const int len[BandPlan::kSizes] = {kMediumMaxLen, 12000, 12000, kBandMaxLen};
+  // CTAs an SM (a CTA costs 1 KB of shared memory besides its own).  Eight of
+  // four warps are what 64 registers allow, for short sequences (200,000 reads
+  // in windows 1.93 ms, 2.00 with six); six for longer ones, so that rows of
+  // some 460 diagonals fit a warp (mixed lengths 12.0 ms with eight, 11.8 with
+  // six).  Under 4/6/2 (9 rows, 18 bytes a diagonal) a team's rows may be about
+  // 1,500, 1,900 and 3,900 diagonals wide: the last size holds reads of 32,000
+  // bases at up to some 4 % edits.  The second has a form with half as many
+  // CTAs of eight warps, the last only that.
+  const int len[BandPlan::kSizes] = {kDirectMaxLen, 12000, 12000, kBandMaxLen};
   const int warps[BandPlan::kSizes] = {kBandWarps, kBandWarps, 2 * kBandWarps, 2 * kBandWarps};
   const int want[BandPlan::kSizes] = {8, 6, 3, 3};
   int nsm = 0;
@@ -323,7 +326,7 @@ cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs
   // fewer long pairs than CTAs of four warps: CTAs of eight (400 x 10 kbp with
   // CIGARs 2.7 -> 2.0 ms, 2,000 no faster: every row costs eight warps its
   // fixed part)
-  if (size == 1 && nlong <= (int64_t)plan.nsm * plan.per_sm[1]) size = 2;
+  if (size == 1 && max_len > kMediumMaxLen && nlong <= (int64_t)plan.nsm * plan.per_sm[1]) size = 2;
   const int warps = plan.warps[size], smem = plan.smem[size];
   const int warp_smem = (smem / warps) & ~15;
   cudaError_t e = cudaMemsetAsync(b.aux, 0, kBandAux * sizeof(int32_t), st);

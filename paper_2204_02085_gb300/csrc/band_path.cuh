@@ -54,7 +54,11 @@ constexpr uint32_t kBandValid = 0x8000u;  // u below this is an offset
 constexpr int kBandMaxLen = 32000;        // u fits 15 bits
 constexpr int kBandMaxPen = 31;           // scaled penalties: rows kept per pair
 constexpr int kBandWarps = 4;             // warps of a CTA (and of a team); twice as many when few pairs are long
-constexpr int kBandTeamWidth = 256;       // rows wider than this: a team
+// Rows wider than this (or than a warp's share of the shared memory): a team,
+// whose every row costs each of its warps the fixed part and a barrier
+// (200,000 mixed-length pairs 12.6 ms a call with teams from 256 diagonals, 11.8
+// from what fits a warp).
+constexpr int kBandTeamWidth = 512;
 
 // 16-bit row cells a pair keeps per diagonal.
 __host__ __device__ constexpr int band_rows(int x, int oe, int e) {

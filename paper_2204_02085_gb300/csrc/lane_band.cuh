@@ -4,14 +4,15 @@
 //
 // The ordering pass bounds each pair's scaled score from above by a greedy
 // alignment (T) and sorts every group of pairs by (T, end diagonal m - n), so
-// that the 32 pairs of a warp have nearly the same bound and end diagonal.
+// that the 32 pairs of a warp have nearly the same bound and end diagonal;
+// for stores of low scores T is the store's last score for every pair.
 // The kernel then runs the wavefronts in lockstep, one lane per pair, but a
 // row holds only diagonals that lie on some alignment of cost <= T: those a
 // start reaches (a gap of d costs o + e d) from which an end diagonal is
 // still within reach (a cell d diagonals from the nearest end diagonal of
 // the warp's pairs needs o + e d more, or e d when the gap that closes the
 // distance is already open).  At T = 16, 12 and 8 under 4/6/2 (scaled
-// 2/4/1) that is 85, 37 and 13 cells where the unpruned rows have 195, 104
+// 2/4/1) that is 85, 37 and 9 cells where the unpruned rows have 195, 104
 // and 37.  Every step of the recurrences costs at least what it brings the
 // cell closer by, so the sources of a cell inside the range are inside
 // theirs: values inside are the unpruned method's, and so are the score and
@@ -222,14 +223,17 @@ struct LaneOrderShm {
 
 // The ordering pass (a block of GROUP / PER threads, PER pairs of a group each;
 // sequences in device memory, each lane reading its own pair's aligned
-// 16-byte chunks).  Large groups: two pairs a thread and two blocks an SM, so
-// that one packs while the other waits for its bytes or its slowest warp
-// (with one block of GROUP threads half the issue slots were idle).  cap: the largest bound of interest (the last score the
-// store holds, or the caller's largest); pairs above it get it.  walk =
-// false: every pair at cap, sorted by end diagonal alone (for stores so small
-// that the greedy walk would cost more than it saves).  Pairs longer than LMAX are
-// deferred and pairs with a byte other than A/C/G/T get their status here;
-// both, and the slots past the last pair, become empty slots (pair -1).
+// 16-byte chunks).  Large groups: two pairs a thread and two blocks an SM or
+// more, so that one packs while another waits for its bytes or its slowest
+// warp (with one block of GROUP threads half the issue slots were idle).  Bound
+// by instruction issue and the loads' latency: 1M pairs of 100 bases take 76 us
+// sorted by end diagonal, 117 us with the walk.  cap: the largest bound of
+// interest (the last score the store holds, or the caller's largest); pairs
+// above it get it.  walk = false: every pair at cap, sorted by end diagonal
+// alone (for stores so small that the greedy walk would cost more than it
+// saves).  Pairs longer than LMAX are deferred and pairs with a byte other than
+// A/C/G/T get their status here; both, and the slots past the last pair, become
+// empty slots (pair -1).
 template <int LMAX, int GROUP, int PER>
 __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned char* smem) {
   using S_t = LaneOrderShm<LMAX, GROUP>;
@@ -390,6 +394,10 @@ __host__ __device__ constexpr int lane_band_rows(int x, int oe, int e) { return 
 // caller's bound), as are pairs whose CIGAR needs more than kSlot runs.  A
 // batch whose end diagonals spread too far for the store (around the border
 // of two bounds) runs in two or more passes.
+// Bound by instruction issue; with the large store also by the 16 warps an SM
+// its 12.9 KB a warp leave.  1M pairs of 100 bases: E = 2 % 144 -> 88 us, E =
+// 4 % 508 -> 290 us (73 and 223 warp instructions a pair), before: every
+// diagonal a row can hold (lane_path.cuh).
 template <typename U, int LMAX, int PX, int POE, int PE, int GROUP>
 __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBand& lb, unsigned char* smem) {
   constexpr int NP = lane_plane_words(LMAX);
