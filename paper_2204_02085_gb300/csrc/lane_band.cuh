@@ -382,6 +382,11 @@ __host__ __device__ inline void lane_band_row(int s, int T, int kl, int kh, int 
 // eight cells and two up to 16.
 __host__ __device__ constexpr int lane_band_choice_words(int w) { return w <= 0 ? 0 : w <= 8 ? 1 : 2; }
 constexpr int kLaneBandWidth = 16;  // widest row
+constexpr int kLaneBlock = 2;       // cells of a row whose loads go together, and one at the end of odd rows
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
 
 // Rows of a store: M of the last R scores, then I and D of the last e.
 __host__ __device__ constexpr int lane_band_rows(int x, int oe, int e) { return (x > oe ? x : oe) + 2 * e; }
@@ -395,8 +400,9 @@ __host__ __device__ constexpr int lane_band_rows(int x, int oe, int e) { return 
 // batch whose end diagonals spread too far for the store (around the border
 // of two bounds) runs in two or more passes.
 // Bound by instruction issue; with the large store also by the 16 warps an SM
-// its 12.9 KB a warp leave.  1M pairs of 100 bases: E = 2 % 144 -> 88 us, E =
-// 4 % 508 -> 290 us (73 and 223 warp instructions a pair), before: every
+// its 12.9 KB a warp leave.  1M pairs of 100 bases: E = 2 % 144 -> 89 us, E =
+// 4 % 508 -> 277 us (75 and 220 warp instructions a pair, 70 % of the issue
+// slots at E = 4 %), before: every
 // diagonal a row can hold (lane_path.cuh).
 template <typename U, int LMAX, int PX, int POE, int PE, int GROUP>
 __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBand& lb, unsigned char* smem) {
@@ -559,32 +565,57 @@ __device__ __forceinline__ void lane_band_body(const AlignArgs& a, const LaneBan
           // pending extensions, and the row's choices: mismatch taken,
           // insertion over deletion, I extended, D extended
           uint32_t pend = 0, cx = 0, ci = 0, ce = 0, cd = 0, bit = 1;
-#pragma unroll 4
-          for (int k = lo; k <= hi; ++k) {
-            const uint32_t oc = mo[(k + 1) * 32], dn = dr[(k + 1) * 32], inext = ir[k * 32];
-            const uint32_t ux = (uint32_t)mx[k * 32] - 1u;
-            const bool ei = il <= oa, ed = dn <= oc;  // extension (ties extend)
-            const uint32_t uI = (ei ? il : oa) - (k > kf ? 1u : 0u);
-            const uint32_t uD = (ed ? dn : oc) - (k < kf ? 1u : 0u);
-            const uint32_t ug = min(uI, uD);
-            if (ux <= ug) cx |= bit;
-            if (uI <= uD) ci |= bit;
-            if (ei) ce |= bit;
-            if (ed) cd |= bit;
-            uint32_t u = min(ux, ug);
-            if (u <= (uint32_t)LMAX && run) {
-              const int eq = matches(k, min(m, n + k) - max(k, 0) - (int)u);
-              if (eq == 32) pend |= bit;
-              u -= (uint32_t)eq;
+          // N cells at once: every load before the stores, which the compiler
+          // has to take for aliases of the next cells' sources (1M pairs of 150
+          // bases 701 -> 681 us a call, 5M of 100 at E = 4 % 2,030 -> 1,998; three
+          // or four at once no faster)
+          auto cells = [&](int k, auto count) {
+            constexpr int N = count.value;
+            uint32_t o[N + 2], dn[N], in[N + 1], u[N];
+            int at[N];
+            bool valid[N];
+            o[0] = oa;
+            o[1] = ob;
+            in[0] = il;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+              o[j + 2] = mo[(k + j + 1) * 32];
+              dn[j] = dr[(k + j + 1) * 32];
+              in[j + 1] = ir[(k + j) * 32];
+              u[j] = (uint32_t)mx[(k + j) * 32] - 1u;
             }
-            ms[k * 32] = (U)u;
-            ir[k * 32] = (U)uI;
-            dr[k * 32] = (U)uD;
-            oa = ob;
-            ob = oc;
-            il = inext;
-            bit += bit;
-          }
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+              const bool ei = in[j] <= o[j], ed = dn[j] <= o[j + 2];  // extension (ties extend)
+              const uint32_t uI = (ei ? in[j] : o[j]) - (k + j > kf ? 1u : 0u);
+              const uint32_t uD = (ed ? dn[j] : o[j + 2]) - (k + j < kf ? 1u : 0u);
+              const uint32_t ug = min(uI, uD);
+              if (u[j] <= ug) cx |= bit << j;
+              if (uI <= uD) ci |= bit << j;
+              if (ei) ce |= bit << j;
+              if (ed) cd |= bit << j;
+              u[j] = min(u[j], ug);
+              valid[j] = u[j] <= (uint32_t)LMAX && run;
+              at[j] = valid[j] ? min(m, n + k + j) - max(k + j, 0) - (int)u[j] : 0;
+              ir[(k + j) * 32] = (U)uI;
+              dr[(k + j) * 32] = (U)uD;
+            }
+            int eq[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) eq[j] = matches(k + j, at[j]);
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+              if (valid[j] && eq[j] == 32) pend |= bit << j;
+              ms[(k + j) * 32] = (U)(valid[j] ? u[j] - (uint32_t)eq[j] : u[j]);
+            }
+            oa = o[N];
+            ob = o[N + 1];
+            il = in[N];
+            bit <<= N;
+          };
+          int k = lo;
+          for (; k + kLaneBlock <= hi + 1; k += kLaneBlock) cells(k, IntC<kLaneBlock>());
+          if (k <= hi) cells(k, IntC<1>());
           if (cig) {
             uint32_t* const b = bits + (t >> 16) * 32;
             if (hi - lo < 8) {
