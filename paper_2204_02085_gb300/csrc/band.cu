@@ -166,21 +166,21 @@ __global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
   const int nwarp = *(volatile const int32_t*)&a.ctrl->warp_count;
   unsigned char* cta_slot = arena + (size_t)blockIdx.x * WARPS * (size_t)slot_bytes;
   if (nteam > 0) {
-    TeamShm* ts = reinterpret_cast<TeamShm*>(smem);
-    if (threadIdx.x == 0) ts->flags[0] = ts->flags[1] = ts->flags[2] = 0;
+    BandShm* ts = reinterpret_cast<BandShm*>(smem);
+    if (threadIdx.x == 0) ts->team.flags[0] = ts->team.flags[1] = ts->team.flags[2] = 0;
     __syncthreads();
     int round = 0;
     for (;;) {
-      const int i = Team<WARPS>::broadcast(threadIdx.x == 0 ? atomicAdd(&a.ctrl->team_next, 1) : 0, &ts->bcast);
+      const int i = Team<WARPS>::broadcast(threadIdx.x == 0 ? atomicAdd(&a.ctrl->team_next, 1) : 0, &ts->team.bcast);
       if (i >= nteam) break;
       const int32_t pair = order[i];
-      band_pair<WARPS, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, smem + sizeof(TeamShm), ts, round, cta_slot,
+      band_pair<WARPS, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, smem + sizeof(BandShm), ts, round, cta_slot,
                                      WARPS * slot_bytes, &a.ctrl->overflow_count);
     }
     __syncthreads();
   }
   unsigned char* my = smem + warp * warp_smem;
-  TeamShm* ts = reinterpret_cast<TeamShm*>(my);
+  BandShm* ts = reinterpret_cast<BandShm*>(my);
   int round = 0;
   for (;;) {
     int i = 0;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
     i = __shfl_sync(0xffffffffu, i, 0);
     if (i >= nwarp) break;
     const int32_t pair = order[nteam + i];
-    band_pair<1, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, my + sizeof(TeamShm), ts, round,
+    band_pair<1, CIG, EF>(a, absent, pair, key[pair] & kBoundMask, my + sizeof(BandShm), ts, round,
                           cta_slot + warp * slot_bytes, slot_bytes, &a.ctrl->overflow_count);
     __syncwarp();
   }
@@ -208,9 +208,9 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
   if (*(volatile const int32_t*)&a.ctrl->bad_input) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* my = smem + warp * warp_smem;
-  TeamShm* ts = reinterpret_cast<TeamShm*>(my);
-  my += sizeof(TeamShm);
-  const int room = warp_smem - (int)sizeof(TeamShm);
+  BandShm* ts = reinterpret_cast<BandShm*>(my);
+  my += sizeof(BandShm);
+  const int room = warp_smem - (int)sizeof(BandShm);
   const bool pen_ok = a.xs <= kBandMaxPen && a.oes <= kBandMaxPen && a.es <= kBandMaxPen;
   const int w0 = (int)blockIdx.x * kBandWarps + warp, nw = (int)gridDim.x * kBandWarps;
   const uint32_t absent = EF ? band_absent(a.xs, a.oes, a.es) : 0u;
@@ -222,8 +222,8 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
     if (mine) {
       uint32_t* pw = reinterpret_cast<uint32_t*>(my);
       uint32_t* tw = pw + band_words(n);
-      const bool okp = team_pack32<1>(a.pat + a.poff[pair], n, pw, ts->flags, round);
-      const bool okt = team_pack32<1>(a.txt + a.toff[pair], m, tw, ts->flags, round);
+      const bool okp = team_pack32<1>(a.pat + a.poff[pair], n, pw, ts->team.flags, round);
+      const bool okt = team_pack32<1>(a.txt + a.toff[pair], m, tw, ts->team.flags, round);
       if (!(okp && okt)) {
         if (lane == 0) write_result(a, pair, 2, -1, 0, 0);
         __syncwarp();
@@ -339,8 +339,8 @@ cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs
   int bound_per_sm = std::min(std::max(1, 228 * 1024 / (bound_smem + 1024)), 12);
   const int64_t bound_grid = std::min<int64_t>((pairs + kBandWarps - 1) / kBandWarps, (int64_t)plan.nsm * bound_per_sm);
   bound_kernel<<<(unsigned)bound_grid, 32 * kBandWarps, bound_smem, st>>>(
-      a, b.key, b.aux, (bound_smem / kBandWarps) & ~15, warp_smem - (int)sizeof(TeamShm),
-      smem - (int)sizeof(TeamShm), ordered ? 1 : 0);
+      a, b.key, b.aux, (bound_smem / kBandWarps) & ~15, warp_smem - (int)sizeof(BandShm),
+      smem - (int)sizeof(BandShm), ordered ? 1 : 0);
   if ((e = cudaGetLastError())) return e;
   const int64_t tiles = (pairs + kPlaceBlock * kPlaceItems - 1) / (kPlaceBlock * kPlaceItems);
   place_kernel<<<(unsigned)std::min<int64_t>(tiles, 2 * plan.nsm), kPlaceBlock, 0, st>>>(

@@ -270,7 +270,8 @@ __device__ __forceinline__ uint32_t band_absent(int x, int oe, int e) {
 // scaled score (and its end diagonal in *k_out), or -1 when no alignment
 // costs at most T.  bits: the choice bits of row s, block c at
 // bits[s * g.blocks() + c] (CIG).  fin: a shared word, 0 on entry: the score
-// whose row holds an end (EF).
+// whose row holds an end (EF).  It is this pass's alone until the team's next
+// barrier after the return: a warp may still read it then.
 template <int WPP, bool CIG, bool EF>
 __device__ int band_forward(const BandGeo& g, const uint32_t* pw, const uint32_t* tw, uint16_t* rows, int x, int oe,
                             int e, uint32_t absent, uint4* bits, int* fin, int* k_out) {
@@ -521,11 +522,19 @@ __device__ int band_replay(const BandGeo& g, const uint32_t* pw, const uint32_t*
 
 // ----------------------------------------------------------- one pair
 
+// Shared words of a team (a warp or a CTA).  `fin` has a word of its own: the
+// first thread, past a pair's last row, writes the queue's next index to
+// team.bcast while a slower warp may still be reading `fin` of that row.
+struct alignas(16) BandShm {
+  TeamShm team;
+  int fin;
+};
+
 // One pair, on one warp (WPP 1) or a CTA: absent = band_absent(...), smem of at
 // least band_bytes, slot_bytes of the arena at slot.  packed: the sequences
 // are at smem already.
 template <int WPP, bool CIG, bool EF>
-__device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int T, unsigned char* smem, TeamShm* ts,
+__device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int T, unsigned char* smem, BandShm* ts,
                           int& round,
                           unsigned char* slot, long slot_bytes, int32_t* overflow_count, bool packed = false) {
   using T_ = Team<WPP>;
@@ -539,14 +548,14 @@ __device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int
     if (r == 0) overflow_pair_to(a, pair, overflow_count);
     return;
   }
-  if (EF && r == 0) ts->bcast = 0;
+  if (EF && r == 0) ts->fin = 0;
   if (!packed) {
-    team_pack32<WPP>(a.pat + a.poff[pair], n, pw, ts->flags, round);  // the bound pass checked the bytes
-    team_pack32<WPP>(a.txt + a.toff[pair], m, tw, ts->flags, round);
+    team_pack32<WPP>(a.pat + a.poff[pair], n, pw, ts->team.flags, round);  // the bound pass checked the bytes
+    team_pack32<WPP>(a.txt + a.toff[pair], m, tw, ts->team.flags, round);
   }
   int k_end = 0;
   uint4* bits = reinterpret_cast<uint4*>(slot);
-  const int s = band_forward<WPP, CIG, EF>(g, pw, tw, rows, a.xs, a.oes, a.es, absent, bits, &ts->bcast, &k_end);
+  const int s = band_forward<WPP, CIG, EF>(g, pw, tw, rows, a.xs, a.oes, a.es, absent, bits, &ts->fin, &k_end);
   if (!CIG || s < 0) {
     // no alignment within T: T was the caller's largest score
     if (r == 0) {

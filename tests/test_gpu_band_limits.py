@@ -1,0 +1,49 @@
+"""The band kernels where their forms and limits lie: parity with the oracle
+bit for bit (integer results)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import paper_2204_02085_gb300 as p
+
+    p.load()
+    return p
+
+
+def _check(got, want):
+    for i in (0, 1, 3, 2):
+        np.testing.assert_array_equal(got[i], want[i])
+
+
+def _windows(count, length, flank, rate, seed):
+    """Reads in windows: the text is the edited read between two flanks."""
+    from paper_2204_02085_gb300 import synth
+
+    core = synth.random_pairs(count, length, length, seed=seed, edit_rate=rate)
+    rng = np.random.Generator(np.random.PCG64(seed))
+
+    def seq(n):
+        return rng.choice(list(b"ACGT"), size=int(n)).astype(np.uint8).tobytes()
+
+    return synth.from_pairs([(core.pair(i)[0], seq(rng.integers(flank // 2, flank)) + core.pair(i)[1] +
+                              seq(rng.integers(flank // 2, flank))) for i in range(core.n)])
+
+
+@pytest.mark.parametrize("count,length,flank", [(600, 300, 700), (40, 2100, 700)])
+def test_free_ends_on_teams(pkg, oracle_mod, count, length, flank):
+    """Rows over more free start diagonals than a warp takes: teams of four
+    warps, and of eight where few pairs are long."""
+    b = _windows(count, length, flank, 0.04, count)
+    ends = (0, 0, 2 * flank + length, 2 * flank + length)
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=8, ends=ends)
+    with pkg.Aligner(0, 1 << 30) as al:
+        al.set_ends_free(*ends)
+        for _ in range(3):
+            s, st, _, _ = al.align(b, (4, 6, 2), score_only=True)
+            np.testing.assert_array_equal(s, want[0])
+            np.testing.assert_array_equal(st, want[1])
+        _check(al.align(b, (4, 6, 2)), want)
