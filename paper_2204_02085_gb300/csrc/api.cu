@@ -568,9 +568,11 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
 cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int max_len, bool may_alloc) {
   a.lane_words = nullptr;
   a.lane_slots = nullptr;
+  a.lane_planes = 0;
   if (!c->lane_order || !c->lane_on || n <= 0 || max_len > 255) return cudaSuccess;
   const int64_t slots = (n + wfa::kLaneGroupMax - 1) / wfa::kLaneGroupMax * wfa::kLaneGroupMax;
-  const size_t words = (size_t)slots * 4 * wfa::lane_plane_words(max_len <= 127 ? 127 : max_len <= 191 ? 191 : 255);
+  const int planes = wfa::lane_plane_words(max_len <= 127 ? 127 : max_len <= 191 ? 191 : 255);
+  const size_t words = (size_t)slots * 4 * planes;
   if (may_alloc) {
     cudaError_t e;
     if ((e = c->lane_words.ensure(words)) || (e = c->lane_slots.ensure((size_t)slots))) return e;
@@ -579,6 +581,7 @@ cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int ma
   }
   a.lane_words = c->lane_words.p;
   a.lane_slots = c->lane_slots.p;
+  a.lane_planes = planes;
   a.lane_sort_min = c->lane_sort_min;
   return cudaSuccess;
 }
@@ -692,7 +695,7 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
 // Whether a global call of sequences of 128-255 bases runs on ordered input.
 bool short_ordered(const wfa_gpu_ctx* c, const wfa::AlignArgs& a, int max_len) {
   return max_len <= 255 && (a.pb | a.pe | a.tb | a.te) == 0 &&
-         wfa::lane_ordered(a, c->plan.v[c->lane_255_variants[0]]);
+         wfa::lane_ordered(a, c->plan.v[max_len <= 191 ? c->lane_191_variants[0] : c->lane_255_variants[0]]);
 }
 
 // The plain baseline's short-read variant: the largest store of the call's

@@ -223,10 +223,12 @@ void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb) {
 // reads each pair's bytes with its own loads, which page-locked host memory
 // read in place over the link would turn into many small transfers).
 bool lane_ordered(const AlignArgs& a, const ShortVariant& v) {
-  return a.n > 0 && v.kind == 1 && a.lane_slots && a.lane_words && !a.host_seqs;
+  return a.n > 0 && v.kind == 1 && a.lane_slots && a.lane_words && lane_plane_words(v.max_len) <= a.lane_planes &&
+         !a.host_seqs;
 }
 
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st) {
+  if (!lane_ordered(a, v)) return cudaErrorInvalidValue;
   LaneBand lb;
   lane_band_plan(a, v, &lb);
   // bounds above the store's mean "deferred" (or over the caller's largest

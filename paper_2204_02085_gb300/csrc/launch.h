@@ -71,6 +71,7 @@ struct AlignArgs {
   // lane_slots[j * G + q].
   uint32_t* lane_words;
   int2* lane_slots;
+  int lane_planes;    // plane words lane_words has room for per sequence and plane: the NP of the largest class it takes
   int lane_sort_min;  // smallest store (largest bound) whose ordering bounds each pair
 };
 
@@ -170,7 +171,8 @@ struct LaneBand {
   uint32_t run;
 };
 void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb);
-// Whether launch_short runs the ordering pass and the band kernel of v.
+// Whether launch_short runs the ordering pass and the band kernel of v: only
+// where lane_words has room for the planes of v's length class.
 bool lane_ordered(const AlignArgs& a, const ShortVariant& v);
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st);
 // Bounds of a sample of global pairs (those of at most 255 bases): host[T] =

@@ -47,3 +47,20 @@ def test_free_ends_on_teams(pkg, oracle_mod, count, length, flank):
             np.testing.assert_array_equal(s, want[0])
             np.testing.assert_array_equal(st, want[1])
         _check(al.align(b, (4, 6, 2)), want)
+
+
+@pytest.mark.parametrize("store", ["lane_l191_t12", "lane_l255_t12_i16", "lane_l255_t16_i16"])
+def test_forced_store_of_a_longer_class(pkg, oracle_mod, monkeypatch, store):
+    """Forced onto a call of shorter reads, whose planes it has no room for, a
+    store of a longer class is left out."""
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.uniform_reads(5000, 100, 3, seed=9)
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=8)
+    with pkg.Aligner(0, 1 << 28) as al:
+        index = next(i for i in range(64) if al.variant_name(i) == store)
+    monkeypatch.setenv("WFA_GPU_SHORT_VARIANT", str(index))
+    with pkg.Aligner(0, 1 << 28) as al:
+        _check(al.align(b, (4, 6, 2)), want)
+        assert al.variant_name(al.timing()["short_variant"]).startswith("lane_")
+        assert al.timing()["short_variant"] != index
