@@ -915,6 +915,9 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
     ac.score = a.score + b; ac.status = a.status + b;
     ac.nruns = a.nruns + b; ac.run_src = a.run_src + b;
     ac.runs = a.runs + (score_only ? 0 : b * wfa::kSlot);
+    // a chunk's retries may have replaced the CIGAR pool by a larger one
+    ac.pool = ctx->pool.p;
+    ac.pool_cap = score_only ? 0 : (int64_t)ctx->pool.cap;
     if (sin) {
       // the chunk's bases at ring slot c % kRing: base addresses moved back by
       // the chunk's first offsets (integer arithmetic; the kernels add the

@@ -64,3 +64,40 @@ def test_forced_store_of_a_longer_class(pkg, oracle_mod, monkeypatch, store):
         _check(al.align(b, (4, 6, 2)), want)
         assert al.variant_name(al.timing()["short_variant"]).startswith("lane_")
         assert al.timing()["short_variant"] != index
+
+
+def test_chunked_call_grows_the_cigar_pool(pkg, oracle_mod, monkeypatch):
+    """A host call in chunks whose first chunk's CIGARs outgrow the pool: the
+    chunks after it use the one that replaced it.  (300 unrelated bases take
+    some 300 words of the pool, which starts with room for 6.3 million.)"""
+    import torch
+
+    from paper_2204_02085_gb300 import synth
+
+    chunk, n = 1 << 15, 1 << 21
+    monkeypatch.setenv("WFA_GPU_PIPE_CHUNK", str(chunk))
+    rng = np.random.Generator(np.random.PCG64(21))
+    plen = np.ones(n, np.int32)
+    for c in (0, 1, 5):
+        plen[c * chunk:c * chunk + 24_000] = 300
+    total = int(plen.sum())
+
+    def pinned(a):
+        t = torch.empty(a.shape, dtype=torch.from_numpy(a[:0]).dtype, pin_memory=True)
+        t.numpy()[...] = a
+        return t.numpy()
+
+    letters = np.frombuffer(b"ACGT", np.uint8)
+    pat, txt = (pinned(letters[rng.integers(0, 4, size=total)]) for _ in range(2))
+    plen = pinned(plen)
+    offs = np.cumsum(plen, dtype=np.int64) - plen
+    want = oracle_mod.wfa_batch(synth.Batch(pat, offs, plen, txt, offs, plen), (1, 0, 1), nthreads=16)
+    cap = int(want[3][-1])
+    s, st, off, w = (pinned(np.zeros(k, t)) for k, t in ((n, np.int32), (n, np.int8), (n + 1, np.int64),
+                                                         (cap, np.int32)))
+    with pkg.Aligner(0, 4 << 30) as al:
+        rc = pkg.wfa_gpu_align_batch(al.ctx, n, pat.ctypes.data, None, plen.ctypes.data, txt.ctypes.data, None,
+                                     plen.ctypes.data, pkg.Penalties(1, 0, 1), 0, 0, s.ctypes.data, st.ctypes.data,
+                                     w.ctypes.data, cap, off.ctypes.data)
+    assert rc == pkg.WFA_GPU_OK
+    _check((s, st, w.view(np.uint32), off), want)
