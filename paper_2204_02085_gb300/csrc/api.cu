@@ -519,6 +519,7 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
   wfa::Ctrl* dc = c->ctrl;
   const long arena = (long)c->arena_bytes;
   int teams = c->teams_long;
+  bool whole = false;             // the last retry gave each pair the whole arena
   int32_t* in = a.overflow_list;  // the pairs to retry
   int32_t* out = a.defer_list;    // free again: receives the next overflow
   while (hc->overflow_count > 0) {
@@ -541,7 +542,7 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
       a.pool = nb;
       a.pool_cap = want;
     } else {
-      if (teams == 1) return WFA_GPU_ENOMEM;  // a pair needs more than the whole arena
+      if (whole) return WFA_GPU_ENOMEM;  // a pair needs more than the whole arena
       teams = std::max(1, std::min(teams, hc->overflow_count) / 8);
     }
     hc->retry_count = hc->overflow_count;
@@ -552,6 +553,7 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
     wfa::AlignArgs ar = a;
     ar.overflow_list = out;
     const int nt = std::max(1, std::min(teams, hc->retry_count));
+    whole = nt == 1;
     if (!k.launched(wfa::launch_arena(wfa::kLongTeamWide, ar, in, &dc->retry_count, &dc->next_retry, &dc->overflow_count,
                                       reinterpret_cast<unsigned char*>(c->arena), (arena / nt) & ~255L, nt, st)))
       return WFA_GPU_ECUDA;

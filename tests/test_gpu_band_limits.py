@@ -101,3 +101,14 @@ def test_chunked_call_grows_the_cigar_pool(pkg, oracle_mod, monkeypatch):
                                      w.ctypes.data, cap, off.ctypes.data)
     assert rc == pkg.WFA_GPU_OK
     _check((s, st, w.view(np.uint32), off), want)
+
+
+def test_small_arena_retries_on_the_whole_arena(pkg, oracle_mod):
+    """Pairs that outgrow their slices of an arena too small for two one-CTA
+    teams get the whole of it before the call gives up."""
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.random_pairs(16, 2400, 2400, seed=31, edit_rate=0.06)
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=8)
+    with pkg.Aligner(0, 4 << 20) as al:
+        _check(al.align(b, (4, 6, 2)), want)
