@@ -170,6 +170,11 @@ static void lane_band_solve(const AlignArgs& a, const ShortVariant& v, LaneBand*
     if (g || (s >= X && (ex >> (s - X) & 1u))) ex |= 1u << s;
   }
   const uint32_t run = ex | ~((1u << R) - 1u);
+  int from[kLaneBoundMax + 1], back[kLaneBoundMax + 1], open[kLaneBoundMax + 1], fresh[kLaneBoundMax + 1];
+  for (int s = 0; s <= kLaneBoundMax; ++s) {
+    lane_band_start(s, OE, E, &from[s], &back[s]);
+    lane_band_end(s, OE, E, &open[s], &fresh[s]);
+  }
   // the largest bound whose rows and choices fit, with the end diagonals of
   // a warp spread over a few about 0, or any one of them
   for (int T = 0; T <= kLaneBoundMax; ++T) {
@@ -178,8 +183,9 @@ static void lane_band_solve(const AlignArgs& a, const ShortVariant& v, LaneBand*
       int lo_all = 1 << 20, hi_all = -(1 << 20), sum = 0;
       for (int s = 0; s <= T; ++s) {
         int lo, hi;
-        lane_band_row(s, T, d ? d : -1, d ? d : 2, OE, E, &lo, &hi);
-        if (!(run >> s & 1u) || lo > hi) continue;
+        if (!(run >> s & 1u)) continue;
+        lane_band_span(from[s], back[s], open[T - s], fresh[T - s], d ? d : -1, d ? d : 2, &lo, &hi);
+        if (lo > hi) continue;
         sum += lane_band_choice_words(hi - lo + 1);
         lo_all = lo < lo_all ? lo : lo_all;
         hi_all = hi > hi_all ? hi : hi_all;
@@ -201,21 +207,29 @@ static void lane_band_solve(const AlignArgs& a, const ShortVariant& v, LaneBand*
 }
 
 void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb) {
-  // a pure function of these few numbers, some 100 us to work out and asked
-  // for several times a call: each thread keeps its last answers
+  // a pure function of these few numbers, 1 to 16 us to work out and asked for
+  // some ten times a call: each thread keeps its last answers, the stores of
+  // several penalty sets (kept by a hash, most stores of a call shared an
+  // entry and were worked out again in every call: 200,000 reads of 100 bases
+  // at 0.5 % edits under 5/8/3 245 us a call, now 140; under 4/6/2 162, now 131)
   struct Memo {
     int64_t key[4];
     LaneBand lb;
   };
-  static thread_local Memo memo[16] = {};
+  constexpr unsigned kMemo = 64;
+  static thread_local Memo memo[kMemo] = {};
+  static thread_local unsigned oldest = 0;
   const int64_t key[4] = {((int64_t)a.xs << 32) | a.oes, ((int64_t)a.es << 32) | v.band_store,
                           ((int64_t)v.band_smem << 8) | v.band_cell,
-                          (a.pb | a.pe | a.tb | a.te) == 0 ? 1 : 2};
-  Memo& mm = memo[(v.band_store / 16 + v.max_len) % 16];
-  if (std::memcmp(mm.key, key, sizeof key) != 0) {
-    lane_band_solve(a, v, &mm.lb);
-    std::memcpy(mm.key, key, sizeof key);
-  }
+                          ((int64_t)v.max_len << 2) | ((a.pb | a.pe | a.tb | a.te) == 0 ? 1 : 2)};
+  for (const Memo& mm : memo)
+    if (std::memcmp(mm.key, key, sizeof key) == 0) {
+      *lb = mm.lb;
+      return;
+    }
+  Memo& mm = memo[oldest++ % kMemo];
+  lane_band_solve(a, v, &mm.lb);
+  std::memcpy(mm.key, key, sizeof key);
   *lb = mm.lb;
 }
 

@@ -359,23 +359,39 @@ __device__ void lane_bounds_body(const AlignArgs& a, int cap, int32_t* hist, uns
 
 // ------------------------------------------------------------ the kernel
 
-// Row s of a pair set with bound T, start diagonal 0 and end diagonals kl ..
-// kh: its lowest and highest diagonal (lo > hi: no cell).
-__host__ __device__ inline void lane_band_row(int s, int T, int kl, int kh, int oe, int e, int* lo, int* hi) {
-  const int o = oe - e, left = T - s;
-  if (left < 0) {
-    *lo = 1;
-    *hi = 0;
-    return;
-  }
-  const int g = s < oe ? 0 : (s - o) / e;              // a start reaches -g .. g
-  const int gap = left / e;                            // an open gap still covers this far
-  const int m = left < o + e ? 0 : (left - o) / e;     // a gap still to open
-  const int b = s < 2 * oe ? -1 : (s - 2 * o) / e - 2; // a gap back towards 0 is open up to here
+// How far the gaps of a row reach: of score s, a start to -g .. g and a gap
+// back towards 0 up to b; with `left` still to spend, an open gap covers `gap`
+// diagonals and one still to open m.
+__host__ __device__ inline void lane_band_start(int s, int oe, int e, int* g, int* b) {
+  *g = s < oe ? 0 : (s - (oe - e)) / e;
+  *b = s < 2 * oe ? -1 : (s - 2 * (oe - e)) / e - 2;
+}
+__host__ __device__ inline void lane_band_end(int left, int oe, int e, int* gap, int* m) {
+  *gap = left / e;
+  *m = left < oe ? 0 : (left - (oe - e)) / e;
+}
+
+// The lowest and highest diagonal of such a row (lo > hi: no cell) for end
+// diagonals kl .. kh.
+__host__ __device__ inline void lane_band_span(int g, int b, int gap, int m, int kl, int kh, int* lo, int* hi) {
   const int h1 = g < kh + m ? g : kh + m, h2 = b < kh + gap ? b : kh + gap;
   const int l1 = -g > kl - m ? -g : kl - m, l2 = -b > kl - gap ? -b : kl - gap;
   *hi = h1 > h2 ? h1 : h2;
   *lo = l1 < l2 ? l1 : l2;
+}
+
+// Row s of a pair set with bound T, start diagonal 0 and end diagonals kl ..
+// kh.
+__host__ __device__ inline void lane_band_row(int s, int T, int kl, int kh, int oe, int e, int* lo, int* hi) {
+  if (T < s) {
+    *lo = 1;
+    *hi = 0;
+    return;
+  }
+  int g, b, gap, m;
+  lane_band_start(s, oe, e, &g, &b);
+  lane_band_end(T - s, oe, e, &gap, &m);
+  lane_band_span(g, b, gap, m, kl, kh, lo, hi);
 }
 
 // Words of choices a row of w cells keeps: four bits a cell, in one word up to
