@@ -189,8 +189,7 @@ struct wfa_gpu_ctx {
   DevBuf<int32_t> tune_score, tune_aux;
   DevBuf<int8_t> tune_status;
   DevBuf<int64_t> tune_src;
-  int32_t* h_tune = nullptr;  // pinned [kTuneSample]: sampled scores, or the sample's bounds (histogram)
-  int32_t* h_tune_dev = nullptr;
+  int32_t* h_tune = nullptr;  // pinned [kTuneSample]: sampled scores (call order)
   // captured device work of repeated WFA_GPU_GRAPH calls (a few kinds of
   // call, replaced round robin)
   struct Graph {
@@ -326,17 +325,17 @@ const void* mapped_range(const void* p, size_t bytes) {
 
 constexpr int64_t kTuneSample = 4096;
 
-// The bounds of the call's first pairs (a has its penalties and sequences on
-// the device): a histogram in h_tune once the stream is done.
-bool launch_sample_bounds(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs a) {
+// The scores of the call's first pairs (a has its penalties and sequences on
+// the device), counted in the control block, zero until then.
+bool launch_sample(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs a) {
   a.n = std::min(a.n, kTuneSample);
-  if (c->tune_score.ensure(wfa::kLaneBoundBins) != cudaSuccess) return k.ok(cudaErrorMemoryAllocation);
-  return k.launched(wfa::launch_lane_bounds(a, c->tune_score.p, c->h_tune_dev, c->stream), 2);
+  return k.launched(wfa::launch_sample_scores(a, 255, c->stream));
 }
+bool can_sample(const wfa::AlignArgs& a) { return std::max(a.xs, std::max(a.oes, a.es)) <= wfa::kBandMaxPen; }
 
 // Lengths, offsets and sequences on the device (or mapped from page-locked
 // host memory); validates them.  sample (device-pointer calls): the call's
-// penalties, to bound its first pairs before the wait.  Returns 0 or a
+// penalties, to score its first pairs before the wait.  Returns 0 or a
 // negative WFA_GPU_* code.
 int stage_inputs(wfa_gpu_ctx* c, Call& k, int64_t n, bool dev, const char* pat, const int64_t* poff,
                  const int32_t* plen, const char* txt, const int64_t* toff, const int32_t* tlen,
@@ -409,7 +408,7 @@ int stage_inputs(wfa_gpu_ctx* c, Call& k, int64_t n, bool dev, const char* pat, 
     wfa::AlignArgs a = *sample;
     a.pat = pat; a.poff = *d_poff; a.plen = *d_plen;
     a.txt = txt; a.toff = *d_toff; a.tlen = *d_tlen;
-    if (!launch_sample_bounds(c, k, a)) return WFA_GPU_ECUDA;
+    if (!launch_sample(c, k, a)) return WFA_GPU_ECUDA;
   }
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (c->h_ctrl->bad_input) return WFA_GPU_EINVAL;
@@ -589,13 +588,20 @@ cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int ma
 }
 
 // Pick the short-kernel variant for a batch of sequences <= 127 bases (<= 255
-// on ordered input): the smallest store that holds nearly all of a sample of
-// kTuneSample pairs (more pairs resident per SM, and for the lane-per-pair
-// kernel in call order fewer lockstep cells) runs the batch.  Ordered input:
-// by the sample's score bounds (in h_tune already when `sampled`), nine tenths
-// of which the store has to hold -- the greedy bounds of 2 to 7 % of the
-// paper's pairs overshoot a store that holds all their scores.  Call order:
-// the large-store variant scores the sample (score only).  Gap-affine global
+// on ordered input) by a sample of kTuneSample pairs: a small store runs more
+// pairs per SM (and for the lane-per-pair kernel in call order fewer lockstep
+// cells), but hands the pairs above its last score to the band kernels.
+// Ordered input: the cheapest store by the sample's scores (in h_ctrl already
+// when `sampled`) at what the parts measure.  From one store to the next
+// larger 0.02 ns a pair, 0.06 with 16-bit rows (1M pairs of 80-100 bases at 2 %,
+// 4/6/2: 257 us a call with the smallest, 278, 302, 320 and 333 with the
+// largest; of 160-200 bases 548 and 614).  Pairs above the store 80 us for the
+// launches and the wait, and 6 ns each (4/6/1, 41 % of 1M pairs above: 2,716
+// us, with the store that holds them 346).  Nine tenths of the pairs' greedy
+// bounds, the rule before: 200,000 pairs of 80-100 bases at 0-2 % under 4/6/1
+// 348 us, now 178; under 5/8/3 450, now 155.  Call order: the
+// smallest store that holds 99 % of the sample, which
+// the large-store variant scores (score only).  Gap-affine global
 // calls use the lane-per-pair variants unless the context turned them off.
 // Returns the variant index, or -1 on a CUDA error.
 int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t n, int max_len, bool sampled) {
@@ -649,20 +655,30 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   const int64_t m = std::min(n, kTuneSample);
   cudaStream_t st = c->stream;
   if (ordered) {
+    if (!can_sample(a_in)) return big;
     if (!sampled) {
       wfa::AlignArgs a = a_in;
       a.n = n;
-      if (!launch_sample_bounds(c, k, a) || !k.ok(cudaStreamSynchronize(st))) return -1;
+      if (!launch_sample(c, k, a) || !ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return -1;
     }
-    int64_t all = 0, fit[5] = {0, 0, 0, 0, 0};
-    for (int t = 0; t < wfa::kLaneBoundBins; ++t) {
-      all += c->h_tune[t];
-      for (int j = 0; j < ncand; ++j)
-        if (t <= s_store[j]) fit[j] += c->h_tune[t];
+    constexpr double kAboveNs = 6.0, kAboveOnceNs = 80e3;
+    const double step_ns = max_len > 191 ? 0.06 : 0.02;
+    const int32_t* sample = c->h_ctrl->sample;
+    int best = 0;
+    double best_ns = 0.0;
+    for (int j = 0; j < ncand; ++j) {
+      double all = 0, above = 0;
+      for (int t = 0; t < wfa::kSampleBins; ++t) {
+        all += sample[t];
+        if (t > s_store[j]) above += sample[t];
+      }
+      const double ns = n * step_ns * j + (above > 0 ? kAboveOnceNs + n * (above / all) * kAboveNs : 0.0);
+      if (j == 0 || ns < best_ns) {
+        best = j;
+        best_ns = ns;
+      }
     }
-    for (int j = 0; j < ncand; ++j)
-      if (all == 0 || fit[j] * 10 >= all * 9) return cand[j];
-    return big;
+    return cand[best];
   }
   if (c->tune_score.ensure(m) || c->tune_status.ensure(m) || c->tune_aux.ensure(m) || c->tune_src.ensure(m))
     return big;
@@ -744,9 +760,8 @@ int wfa_gpu_create(wfa_gpu_ctx** out, int device, size_t scratch_bytes) {
       if (cudaEventCreate(&c->ev[i]) != cudaSuccess) { rc = WFA_GPU_ECUDA; break; }
     if (rc) break;
     if (cudaMalloc(reinterpret_cast<void**>(&c->ctrl), 2 * sizeof(wfa::Ctrl)) != cudaSuccess) { rc = WFA_GPU_ENOMEM; break; }
-    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_tune), kTuneSample * sizeof(int32_t), cudaHostAllocMapped) !=
-            cudaSuccess ||
-        cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->h_tune_dev), c->h_tune, 0) != cudaSuccess) {
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_tune), kTuneSample * sizeof(int32_t), cudaHostAllocDefault) !=
+        cudaSuccess) {
       rc = WFA_GPU_ENOMEM;
       break;
     }
@@ -1165,7 +1180,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
                                    text_lengths, pen, max_score, score_only, out_scores, out_status);
     return align_small(ctx, k, a, out_cigars, cap, out_cigar_offsets);
   }
-  // the sample's bounds with the input checks, in one wait
+  // the sample's scores with the input checks, in one wait
   wfa::AlignArgs pens{};
   pens.n = n;
   pens.g = g;
@@ -1176,7 +1191,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   pens.ctrl = ctx->ctrl;
   const int32_t* ef = ctx->ends_free;
   const bool sample = dev && mode == 0 && ctx->lane_on && ctx->lane_order && ctx->variant_forced < 0 &&
-                      (ef[0] | ef[1] | ef[2] | ef[3]) == 0;
+                      (ef[0] | ef[1] | ef[2] | ef[3]) == 0 && can_sample(pens);
   int rc = stage_inputs(ctx, k, n, dev, patterns, pattern_offsets, pattern_lengths, texts, text_offsets,
                         text_lengths, &d_pat, &d_poff, &d_plen, &d_txt, &d_toff, &d_tlen, &host_seqs,
                         sample ? &pens : nullptr);

@@ -243,6 +243,32 @@ __global__ void __launch_bounds__(32 * kBandWarps, 8)
   }
 }
 
+// A sample's scores for the choice of a short-read store: the search for a
+// bound alone, a warp per pair, up to the last bin.  The greedy bounds a lane
+// works out for the ordering pass overshoot the score of 2 to 7 % of the
+// paper's pairs, so that a choice by them had to leave a tenth of the pairs
+// to the band kernels, at some 6 ns a pair.
+__global__ void __launch_bounds__(32 * kBandWarps) sample_kernel(const AlignArgs a, int lmax, int warp_smem) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (*(volatile const int32_t*)&a.ctrl->bad_input) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t pair = (int64_t)blockIdx.x * kBandWarps + warp;
+  if (pair >= a.n) return;
+  const int n = a.plen[pair], m = a.tlen[pair];
+  if (n > lmax || m > lmax) return;
+  unsigned char* my = smem + warp * warp_smem;
+  uint16_t* ring = reinterpret_cast<uint16_t*>(my);
+  uint32_t* pw = reinterpret_cast<uint32_t*>(my + 64 * band_rows(a.xs, a.oes, a.es));
+  uint32_t* tw = pw + band_words(n);
+  int round = 0, flags[3];
+  const bool okp = team_pack32<1>(a.pat + a.poff[pair], n, pw, flags, round);
+  const bool okt = team_pack32<1>(a.txt + a.toff[pair], m, tw, flags, round);
+  if (!(okp && okt)) return;
+  const int cap = min(min(band_worst(n, m, a.xs, a.oes, a.es), a.s_cap), kSampleBins - 1);
+  const int T = band_bound(pw, tw, band_geo(a, n, m, 0), a.xs, a.oes, a.es, cap, ring);
+  if (lane == 0) atomicAdd(&a.ctrl->sample[T], 1);
+}
+
 using BandKernel = void (*)(const AlignArgs, const int32_t*, const int32_t*, unsigned char*, long, int);
 template <int WARPS>
 BandKernel band_kernel_as(bool cig, bool ef) {
@@ -303,6 +329,15 @@ cudaError_t band_plan(int device, BandPlan* plan) {
     }
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_sample_scores(const AlignArgs& a, int lmax, cudaStream_t st) {
+  if (a.n <= 0 || std::max(a.xs, std::max(a.oes, a.es)) > kBandMaxPen) return cudaErrorInvalidValue;
+  const int warp_smem = (64 * band_rows(a.xs, a.oes, a.es) + 8 * band_words(lmax) + 15) & ~15;
+  if (kBandWarps * warp_smem > 48 * 1024) return cudaErrorInvalidValue;
+  sample_kernel<<<(unsigned)((a.n + kBandWarps - 1) / kBandWarps), 32 * kBandWarps, kBandWarps * warp_smem, st>>>(
+      a, lmax, warp_smem);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned char* arena, long arena_bytes,

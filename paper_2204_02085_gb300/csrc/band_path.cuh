@@ -52,7 +52,6 @@ namespace wfa {
 constexpr uint32_t kBandNull = 0xFFFFu;
 constexpr uint32_t kBandValid = 0x8000u;  // u below this is an offset
 constexpr int kBandMaxLen = 32000;        // u fits 15 bits
-constexpr int kBandMaxPen = 31;           // scaled penalties: rows kept per pair
 constexpr int kBandWarps = 4;             // warps of a CTA (and of a team); twice as many when few pairs are long
 // Rows wider than this (or than a warp's share of the shared memory): a team,
 // whose every row costs each of its warps the fixed part and a barrier

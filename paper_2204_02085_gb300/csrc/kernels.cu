@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(kSmallBlock) small_front_kernel(int n, const i
                                                                   const int64_t* toff, const int32_t* tlen,
                                                                   int64_t* out_poff, int64_t* out_toff, Ctrl* ctrl) {
   __shared__ int64_t sh[32];
-  if (threadIdx.x == 0) *ctrl = Ctrl{};
+  if (threadIdx.x < sizeof(Ctrl) / 4) reinterpret_cast<int32_t*>(ctrl)[threadIdx.x] = 0;
   const int i0 = threadIdx.x * kSmallItems;
   int pl[kSmallItems], tl[kSmallItems];
   int64_t ps = 0, ts = 0;

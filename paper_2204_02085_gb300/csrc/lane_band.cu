@@ -22,21 +22,6 @@ __global__ void __launch_bounds__(GROUP / PER, LMAX <= 127 && GROUP == 512 ? 4 :
   lane_order_body<LMAX, GROUP, PER>(a, cap, walk != 0, smem);
 }
 
-// The sample's bounds (autotuner).
-constexpr int kBoundsBlock = 64;
-__global__ void __launch_bounds__(kBoundsBlock) lane_bounds_kernel(const AlignArgs a, int cap, int32_t* hist) {
-  // a row past the planes: a window that starts in the last word of the
-  // text's last plane reads the word behind it
-  __shared__ __align__(16) unsigned char smem[(kBoundsBlock / 32 * 4 * lane_plane_words(255) + 1) * 128];
-  lane_bounds_body<255, kBoundsBlock>(a, cap, hist, smem);
-}
-
-// Its histogram to the host's mirror.
-__global__ void lane_bounds_out_kernel(const int32_t* hist, int32_t* host) {
-  host[threadIdx.x] = hist[threadIdx.x];
-  __threadfence_system();
-}
-
 // One lane per pair on the ordering pass's output, over the diagonals within
 // the pairs' bounds.
 template <typename U, int LMAX, int PX, int POE, int PE, int GROUP>
@@ -259,16 +244,6 @@ cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaS
   const int q = a.xs == 2 && a.oes == 4 && a.es == 1 ? 0 : a.xs == 1 && a.oes == 1 && a.es == 1 ? 1 : 2;
   lane_band_kernel_of(v.max_len, group, a.xs, a.oes, a.es)<<<(unsigned)std::min<int64_t>(v.band_grid[q], need),
                                                       32 * kLaneBandWarps, v.band_smem, st>>>(a, lb);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_lane_bounds(const AlignArgs& a, int32_t* hist, int32_t* host, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(hist, 0, kLaneBoundBins * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  static_assert(kLaneBoundMax < kLaneBoundBins, "bins");
-  lane_bounds_kernel<<<(unsigned)((a.n + kBoundsBlock - 1) / kBoundsBlock), kBoundsBlock, 0, st>>>(
-      a, std::max(0, std::min(kLaneBoundMax, a.s_cap)), hist);
-  lane_bounds_out_kernel<<<1, kLaneBoundBins, 0, st>>>(hist, host);
   return cudaGetLastError();
 }
 

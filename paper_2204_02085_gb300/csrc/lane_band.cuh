@@ -340,23 +340,6 @@ __device__ void lane_order_body(const AlignArgs& a, int cap, bool walk, unsigned
   }
 }
 
-// The bounds alone, of the first pairs of a call whose longest sequence is
-// not known yet: hist[T] counts the pairs with bound T (at most cap).  A
-// thread per pair; longer sequences and other bytes count nowhere.
-template <int LMAX, int BLOCK>
-__device__ void lane_bounds_body(const AlignArgs& a, int cap, int32_t* hist, unsigned char* smem) {
-  constexpr int NP = lane_plane_words(LMAX);
-  if (*(volatile int32_t*)&a.ctrl->bad_input) return;
-  uint32_t* const P = reinterpret_cast<uint32_t*>(smem) + (threadIdx.x >> 5) * (4 * NP * 32) + (threadIdx.x & 31);
-  const int64_t pair = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (pair >= a.n) return;
-  const int n = a.plen[pair], m = a.tlen[pair];
-  const int64_t po = a.poff[pair], to = a.toff[pair];
-  if (n > LMAX || m > LMAX) return;
-  if (lane_pack_planes<NP>(a.pat + po, n, P) | lane_pack_planes<NP>(a.txt + to, m, P + 2 * NP * 32)) return;
-  atomicAdd(&hist[lane_estimate<NP>(P, n, m, a.xs, a.oes, a.es, cap)], 1);
-}
-
 // ------------------------------------------------------------ the kernel
 
 // How far the gaps of a row reach: of score s, a start to -g .. g and a gap

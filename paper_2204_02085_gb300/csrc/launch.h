@@ -9,6 +9,9 @@
 
 namespace wfa {
 
+// Bins of a sample's scaled scores: one each, the last that much or more.
+constexpr int kSampleBins = 32;
+
 // Per-call device control block, zeroed before each batch.
 struct Ctrl {
   int32_t bad_input;        // a length or offset out of range
@@ -32,7 +35,9 @@ struct Ctrl {
   int32_t bound_next, team_next, warp_next;
   int32_t team_count, warp_count, arena_count, arena_long_count;
   int32_t pad;
+  int32_t sample[kSampleBins];  // scores of a sample (launch_sample_scores)
 };
+static_assert(sizeof(Ctrl) % 4 == 0 && sizeof(Ctrl) <= 1024, "moved in words, by one small block at most");
 
 struct AlignArgs {
   int64_t n;
@@ -175,11 +180,6 @@ void lane_band_plan(const AlignArgs& a, const ShortVariant& v, LaneBand* lb);
 // where lane_words has room for the planes of v's length class.
 bool lane_ordered(const AlignArgs& a, const ShortVariant& v);
 cudaError_t launch_lane_ordered(const AlignArgs& a, const ShortVariant& v, cudaStream_t st);
-// Bounds of a sample of global pairs (those of at most 255 bases): host[T] =
-// the pairs with score bound T (the last bin: that much or more), through
-// hist on the device; two kernels.
-constexpr int kLaneBoundBins = 32;
-cudaError_t launch_lane_bounds(const AlignArgs& a, int32_t* hist, int32_t* host, cudaStream_t st);
 // Fill the ordered half of a lane variant, or a variant that has no other,
 // for sequences of up to lmax bases and `store` bytes a warp.
 cudaError_t plan_lane_band(int device, ShortVariant* v, int lmax, int store);
@@ -209,6 +209,7 @@ cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list
                          int32_t* next, int32_t* overflow_count, unsigned char* arena, long slot_bytes, int nteams,
                          cudaStream_t st);
 
+constexpr int kBandMaxPen = 31;  // scaled penalties the band kernels take: rows kept per pair
 // The band kernels over the deferred pairs (a.defer_list, a.defer_long_list
 // and their counts in a.ctrl): each pair's score bound, the pairs ordered by
 // cost (largest first; in call order when `ordered` is false), then the band
@@ -244,6 +245,10 @@ constexpr int kBandLaunches = 3;
 // Calls of at most kDirectPairs pairs: every pair on a warp of its own, what
 // does not fit deferred.
 constexpr int kDirectPairs = 4096;
+// Scores of the first pairs of a global call (a.n of them; those of at most
+// lmax bases, scaled penalties up to kBandMaxPen), found by the band kernels'
+// search for a bound, counted in ctrl->sample.
+cudaError_t launch_sample_scores(const AlignArgs& a, int lmax, cudaStream_t st);
 cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned char* arena, long arena_bytes,
                           cudaStream_t st);
 

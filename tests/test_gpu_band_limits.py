@@ -112,3 +112,26 @@ def test_small_arena_retries_on_the_whole_arena(pkg, oracle_mod):
     want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=8)
     with pkg.Aligner(0, 4 << 20) as al:
         _check(al.align(b, (4, 6, 2)), want)
+
+
+@pytest.mark.parametrize("pen,holds", [((4, 6, 1), 20), ((16, 6, 2), 16), ((5, 8, 3), 30)])
+def test_store_chosen_holds_the_scores(pkg, oracle_mod, pen, holds):
+    """Batches with one pair in twelve above the middle stores and none above
+    the largest (its last score, scaled, in `holds`): the store chosen from the
+    sample holds every pair."""
+    from math import gcd
+
+    from paper_2204_02085_gb300 import synth
+
+    g = gcd(gcd(pen[0], pen[1]), pen[2])
+    pool = synth.uniform_reads(60_000, 100, 1, seed=3), synth.uniform_reads(30_000, 100, 2, seed=4)
+    score = [oracle_mod.wfa_batch(b, pen, nthreads=16, want_cigar=False)[0] // g for b in pool]
+    easy = np.nonzero(score[0] <= 12)[0][:22_000]
+    hard = np.nonzero((score[1] > 12) & (score[1] <= holds))[0][:2_000]
+    pairs = [pool[0].pair(int(i)) for i in easy] + [pool[1].pair(int(i)) for i in hard]
+    order = np.random.default_rng(5).permutation(len(pairs))
+    b = synth.from_pairs([pairs[i] for i in order])
+    want = oracle_mod.wfa_batch(b, pen, nthreads=16)
+    with pkg.Aligner(0, 1 << 28) as al:
+        _check(al.align(b, pen), want)
+        assert al.timing()["deferred_pairs"] == 0
