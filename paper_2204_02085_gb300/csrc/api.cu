@@ -327,11 +327,29 @@ constexpr int64_t kTuneSample = 4096;
 
 // The scores of the call's first pairs (a has its penalties and sequences on
 // the device), counted in the control block, zero until then.
-bool launch_sample(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs a) {
+bool launch_sample(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs a, int longest) {
   a.n = std::min(a.n, kTuneSample);
-  return k.launched(wfa::launch_sample_scores(a, 255, c->stream));
+  return k.launched(wfa::launch_sample_scores(a, longest, c->stream));
 }
-bool can_sample(const wfa::AlignArgs& a) { return std::max(a.xs, std::max(a.oes, a.es)) <= wfa::kBandMaxPen; }
+
+// Whether the band kernels take the call's penalties, and the ordered lane
+// kernel stores any score under them.
+bool band_penalties(const wfa::AlignArgs& a) { return std::max(a.xs, std::max(a.oes, a.es)) <= wfa::kBandMaxPen; }
+
+// The longest sequences of a call of n global pairs that run on ordered input
+// (0: the call runs in call order).  Not under penalties beyond the band's:
+// the call-order kernels store scores up to 31, the ordered ones none (100-base
+// reads at 0.5 % under 19/39/3, 200,000 a call: 1,003 us ordered, 687 in call
+// order).  Above 127 bases only from the batch on that pays for the sample and
+// the ordering pass: reads of 120-150 bases at 0.5-1 %, 4/6/2, 20,000 a call 112-
+// 122 us against 98-104 in call order, 100,000 126-134 against 132-141, 1M
+// 349-368 against 560-598; the gap-linear kernel in call order stores M alone,
+// and its line lies higher (1/0/1: 200,000 157-159 against 142-146, 500,000
+// 242-250 against 234-246, 1M 369-378 against 367-395).
+int ordered_longest(const wfa::AlignArgs& a, int64_t n) {
+  if (!band_penalties(a)) return 0;
+  return n >= (a.oes == a.es ? 1 << 19 : 1 << 16) ? 255 : 127;
+}
 
 // Lengths, offsets and sequences on the device (or mapped from page-locked
 // host memory); validates them.  sample (device-pointer calls): the call's
@@ -408,7 +426,7 @@ int stage_inputs(wfa_gpu_ctx* c, Call& k, int64_t n, bool dev, const char* pat, 
     wfa::AlignArgs a = *sample;
     a.pat = pat; a.poff = *d_poff; a.plen = *d_plen;
     a.txt = txt; a.toff = *d_toff; a.tlen = *d_tlen;
-    if (!launch_sample(c, k, a)) return WFA_GPU_ECUDA;
+    if (!launch_sample(c, k, a, ordered_longest(a, a.n))) return WFA_GPU_ECUDA;
   }
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (c->h_ctrl->bad_input) return WFA_GPU_EINVAL;
@@ -565,12 +583,12 @@ int run_retries(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a) {
 // The lane ordering's buffers for calls of up to n pairs of sequences up to
 // max_len: allocated here (eager calls), or only taken when already large
 // enough (captured work, which must not allocate); left null when the
-// context keeps call order, or for longer sequences.
+// call runs in call order.
 cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int max_len, bool may_alloc) {
   a.lane_words = nullptr;
   a.lane_slots = nullptr;
   a.lane_planes = 0;
-  if (!c->lane_order || !c->lane_on || n <= 0 || max_len > 255) return cudaSuccess;
+  if (!c->lane_order || !c->lane_on || n <= 0 || max_len > ordered_longest(a, n)) return cudaSuccess;
   const int64_t slots = (n + wfa::kLaneGroupMax - 1) / wfa::kLaneGroupMax * wfa::kLaneGroupMax;
   const int planes = wfa::lane_plane_words(max_len <= 127 ? 127 : max_len <= 191 ? 191 : 255);
   const size_t words = (size_t)slots * 4 * planes;
@@ -597,7 +615,9 @@ cudaError_t lane_order_args(wfa_gpu_ctx* c, wfa::AlignArgs& a, int64_t n, int ma
 // 4/6/2: 257 us a call with the smallest, 278, 302, 320 and 333 with the
 // largest; of 160-200 bases 548 and 614).  Pairs above the store 80 us for the
 // launches and the wait, and 6 ns each (4/6/1, 41 % of 1M pairs above: 2,716
-// us, with the store that holds them 346).  Nine tenths of the pairs' greedy
+// us, with the store that holds them 346).  The kernel in call order takes 0.2
+// ns a pair more (above 127 bases, where it may be chosen: 1M pairs of 120-150
+// bases at 1 %, 4/6/2: 598 us, ordered 368).  Nine tenths of the pairs' greedy
 // bounds, the rule before: 200,000 pairs of 80-100 bases at 0-2 % under 4/6/1
 // 348 us, now 178; under 5/8/3 450, now 155.  Call order: the
 // smallest store that holds 99 % of the sample, which
@@ -655,30 +675,38 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   const int64_t m = std::min(n, kTuneSample);
   cudaStream_t st = c->stream;
   if (ordered) {
-    if (!can_sample(a_in)) return big;
     if (!sampled) {
       wfa::AlignArgs a = a_in;
       a.n = n;
-      if (!launch_sample(c, k, a) || !ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return -1;
+      if (!launch_sample(c, k, a, 255) || !ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return -1;
     }
-    constexpr double kAboveNs = 6.0, kAboveOnceNs = 80e3;
+    constexpr double kAboveNs = 6.0, kAboveOnceNs = 80e3, kCallOrderNs = 0.2;
     const double step_ns = max_len > 191 ? 0.06 : 0.02;
     const int32_t* sample = c->h_ctrl->sample;
-    int best = 0;
-    double best_ns = 0.0;
-    for (int j = 0; j < ncand; ++j) {
+    const auto above_ns = [&](int last) {  // pairs above a store whose last score this is
       double all = 0, above = 0;
       for (int t = 0; t < wfa::kSampleBins; ++t) {
         all += sample[t];
-        if (t > s_store[j]) above += sample[t];
+        if (t > last || t == wfa::kSampleBins - 1) above += sample[t];  // (the last bin: that much or more)
       }
-      const double ns = n * step_ns * j + (above > 0 ? kAboveOnceNs + n * (above / all) * kAboveNs : 0.0);
-      if (j == 0 || ns < best_ns) {
-        best = j;
+      return above > 0 ? kAboveOnceNs + n * (above / all) * kAboveNs : 0.0;
+    };
+    int best = cand[0];
+    double best_ns = above_ns(s_store[0]);
+    for (int j = 1; j < ncand; ++j) {
+      const double ns = n * step_ns * j + above_ns(s_store[j]);
+      if (ns < best_ns) {
+        best = cand[j];
         best_ns = ns;
       }
     }
-    return cand[best];
+    if (max_len > 127) {  // the kernel in call order, where it stores higher scores
+      const wfa::ShortVariant& v = c->plan.v[c->variant_mid[model]];
+      wfa::UGeo tab[64];
+      if (n * kCallOrderNs + above_ns(wfa::build_ugeo(tab, v.scap, v.cells, pen, 0, 0)) < best_ns)
+        best = c->variant_mid[model];
+    }
+    return best;
   }
   if (c->tune_score.ensure(m) || c->tune_status.ensure(m) || c->tune_aux.ensure(m) || c->tune_src.ensure(m))
     return big;
@@ -1191,7 +1219,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   pens.ctrl = ctx->ctrl;
   const int32_t* ef = ctx->ends_free;
   const bool sample = dev && mode == 0 && ctx->lane_on && ctx->lane_order && ctx->variant_forced < 0 &&
-                      (ef[0] | ef[1] | ef[2] | ef[3]) == 0 && can_sample(pens);
+                      (ef[0] | ef[1] | ef[2] | ef[3]) == 0 && ordered_longest(pens, n) > 0;
   int rc = stage_inputs(ctx, k, n, dev, patterns, pattern_offsets, pattern_lengths, texts, text_offsets,
                         text_lengths, &d_pat, &d_poff, &d_plen, &d_txt, &d_toff, &d_tlen, &host_seqs,
                         sample ? &pens : nullptr);

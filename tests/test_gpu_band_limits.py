@@ -135,3 +135,86 @@ def test_store_chosen_holds_the_scores(pkg, oracle_mod, pen, holds):
     with pkg.Aligner(0, 1 << 28) as al:
         _check(al.align(b, pen), want)
         assert al.timing()["deferred_pairs"] == 0
+
+
+def _tiled(b, want, times):
+    """The batch repeated, and its results."""
+    from paper_2204_02085_gb300 import synth
+
+    pairs = [b.pair(i) for i in range(b.n)] * times
+    words = want[3][-1] * np.arange(times, dtype=np.int64)
+    off = np.concatenate([(want[3][:-1] + words[:, None]).ravel(), [want[3][-1] * times]])
+    return synth.from_pairs(pairs), (np.tile(want[0], times), np.tile(want[1], times), np.tile(want[2], times), off)
+
+
+def _class_pairs(longest, count, seed, gap=14):
+    """Pairs of up to `longest` bases, most with up to two edits: lengths at
+    word borders of the bit planes, gaps of up to `gap`, some empty,
+    unrelated or with other bytes."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+
+    def seq(n):
+        return rng.choice(list(b"ACGT"), size=int(n)).astype(np.uint8).tobytes()
+
+    out = [(b"", b""), (b"", seq(5)), (seq(9), b""), (seq(longest), seq(longest)), (seq(longest), seq(longest - 20)),
+           (seq(40).lower(), seq(41)), (seq(60) + b"-", seq(61))]
+    lens = [128, 129, 159, 160, 161, longest - 32, longest - 31, longest - 1, longest]
+    while len(out) < count:
+        t = bytearray(seq(rng.choice(lens) if rng.random() < 0.4 else rng.integers(60, longest + 1)))
+        p = bytes(t)
+        for _ in range(int(rng.integers(0, 3)) if rng.random() < 0.97 else 6):
+            i, kind = int(rng.integers(0, len(t))), int(rng.integers(0, 3))
+            if kind == 0:
+                t[i] = int(rng.choice(list(b"ACGT")))
+            elif kind == 1:
+                t[i:i] = seq(rng.choice([1, 1, 1, 2, gap]))
+            else:
+                del t[i:i + int(rng.choice([1, 1, 1, 2, gap]))]
+        out.append((p, bytes(t[:longest])))
+    return out
+
+
+@pytest.mark.parametrize("pen,gap", [((4, 6, 2), 14), ((5, 8, 3), 14), ((1, 1, 1), 14), ((1, 0, 1), 14), ((3, 0, 2), 14),
+                                     ((1, 0, 1), 3), ((3, 0, 2), 3)])
+@pytest.mark.parametrize("longest", [191, 255])
+def test_ordered_classes_above_127_bases(pkg, oracle_mod, longest, pen, gap):
+    """The ordered kernel's classes of up to 191 and 255 bases, in batches from
+    the size on that they take, and in call order below it.  (Under the
+    gap-linear model the kernel in call order stores the higher scores: it
+    keeps a batch with wide gaps.)"""
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.from_pairs(_class_pairs(longest, 5000, longest + sum(pen), gap))
+    want = oracle_mod.wfa_batch(b, pen, nthreads=16)
+    big, big_want = _tiled(b, want, 106 if pen[1] == 0 else 14)
+    with pkg.Aligner(0, 1 << 30) as al:
+        _check(al.align(b, pen), want)
+        assert al.variant_name(al.timing()["short_variant"]).startswith("g")
+        _check(al.align(big, pen), big_want)
+        if pen[1] > 0 or gap < 14:
+            assert al.variant_name(al.timing()["short_variant"]).startswith("lane_l%d_" % longest)
+        s, st, _, _ = al.align(big, pen, score_only=True)
+        np.testing.assert_array_equal(s, big_want[0])
+        np.testing.assert_array_equal(st, big_want[1])
+
+
+def test_call_order_where_it_stores_higher_scores(pkg, oracle_mod):
+    """Reads of 200 bases with two mismatches under 16/6/2 (scaled score 16):
+    the ordered stores end at 14, the kernel in call order holds them."""
+    from paper_2204_02085_gb300 import synth
+
+    rng = np.random.Generator(np.random.PCG64(8))
+    t = rng.choice(list(b"ACGT"), size=(3000, 200)).astype(np.uint8)
+    p = t.copy()
+    swap = dict(zip(b"ACGT", b"GTAC"))
+    for row in p:
+        for i in rng.choice(np.arange(10, 190, 9), size=2, replace=False):
+            row[i] = swap[row[i]]
+    b = synth.from_pairs([(x.tobytes(), y.tobytes()) for x, y in zip(p, t)])
+    want = oracle_mod.wfa_batch(b, (16, 6, 2), nthreads=16)
+    assert np.mean(want[0] == 32) > 0.5  # (a mismatch may also be a gap each way)
+    big, big_want = _tiled(b, want, 23)
+    with pkg.Aligner(0, 1 << 30) as al:
+        _check(al.align(big, (16, 6, 2)), big_want)
+        assert al.variant_name(al.timing()["short_variant"]) == "g4_l255_c197_i16"
+        assert al.timing()["deferred_pairs"] == 0
