@@ -491,11 +491,16 @@ bool launch_arena_lists(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a, const 
                                                   (arena / tl) & ~255L, tl, st)));
 }
 
+// The pairs of the arena lists no arena kernel has taken yet (a kernel over a
+// list leaves its queue's head past the end).
+int arena_left(const wfa::Ctrl* hc) { return hc->next_medium >= hc->arena_count ? 0 : hc->arena_count; }
+int arena_long_left(const wfa::Ctrl* hc) { return hc->next_long >= hc->arena_long_count ? 0 : hc->arena_long_count; }
+
 // The arena kernels over the pairs the band kernels left (h_ctrl mirrors the
 // device control block on entry and on return).
 bool finish_arena_lists(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a) {
   wfa::Ctrl* dc = c->ctrl;
-  const int nm = c->h_ctrl->arena_count, nl = c->h_ctrl->arena_long_count;
+  const int nm = arena_left(c->h_ctrl), nl = arena_long_left(c->h_ctrl);
   if (nm == 0 && nl == 0) return true;
   return launch_arena_lists(c, k, a, c->arena_list.p, &dc->arena_count, nm, c->arena_long_list.p,
                             &dc->arena_long_count, nl) &&
@@ -521,7 +526,11 @@ int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode) {
   if (!k.launched(wfa::launch_band(a, c->band, band_bufs(c), (int64_t)hc->defer_count + hc->defer_long_count,
                                    hc->defer_long_count, hc->max_len, mode == 0, reinterpret_cast<unsigned char*>(c->arena),
                                    (long)c->arena_bytes, st),
-                  wfa::kBandLaunches))
+                  wfa::band_launches(a)))
+    return WFA_GPU_ECUDA;
+  // penalties beyond the band's: every deferred pair is on the arena lists
+  if (!band_penalties(a) && !launch_arena_lists(c, k, a, c->arena_list.p, &dc->arena_count, hc->defer_count,
+                                                c->arena_long_list.p, &dc->arena_long_count, hc->defer_long_count))
     return WFA_GPU_ECUDA;
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
   if (!finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
@@ -1061,13 +1070,20 @@ wfa::AlignArgs device_args(wfa_gpu_ctx* c, int64_t n, const char* pat, const int
                            const char* txt, const int64_t* toff, const int32_t* tlen, wfa_gpu_penalties pen,
                            int32_t max_score, bool score_only, int32_t* out_scores, int8_t* out_status);
 
-// Calls that take the small-call path: a warp per pair, one block for the
+// Calls that take the small-call path: a warp per pair (under penalties beyond
+// the band's the call-order kernel that takes up to 255 bases, which stores
+// scores up to 31: direct_kernel would defer every pair), one block for the
 // offsets and one for the CIGAR offsets.  On 37 reads of 100 bases the
 // sampling, ordering and lane kernels took 126 us in six waits; the line lies
 // where the sample of a larger call begins (4,096 pairs of 100 bases at E =
 // 4 % fill the GPU's warps once).
 bool small_call(const wfa_gpu_ctx* c, int64_t n) {
   return n <= wfa::kDirectPairs && c->lane_on && c->variant_forced < 0;
+}
+bool launch_small_align(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a) {
+  if (!band_penalties(a)) return k.launched(wfa::launch_short(a, c->plan.v[fixed_variant(c, a, 255)], c->stream));
+  return k.launched(wfa::launch_direct(a, c->band, reinterpret_cast<unsigned char*>(c->arena), (long)c->arena_bytes,
+                                       c->stream));
 }
 
 cudaError_t ensure_work(wfa_gpu_ctx* c, int64_t n, int64_t slot_words, bool score_only) {
@@ -1092,10 +1108,10 @@ bool enqueue_small(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int64_t* out_off,
   if (!a.poff) a.poff = c->poff.p;
   if (!a.toff) a.toff = c->toff.p;
   k.rec(1);
-  if (!k.launched(wfa::launch_direct(a, c->band, ab, (long)c->arena_bytes, st))) return false;
+  if (!launch_small_align(c, k, a)) return false;
   k.rec(2);
   if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), a.n, nlong, max_len, true, ab, (long)c->arena_bytes, st),
-                          wfa::kBandLaunches))
+                          wfa::band_launches(a)))
     return false;
   k.rec(3);
   if (!k.launched(wfa::launch_small_finish(a.n, a.nruns, a.score_only ? nullptr : out_off, c->ctrl, c->h_ctrl_dev,
@@ -1113,7 +1129,7 @@ int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* 
                 int64_t cap) {
   const wfa::Ctrl* hc = c->h_ctrl;
   const bool deferred = hc->defer_count > 0 || hc->defer_long_count > 0;
-  const bool left = hc->overflow_count > 0 || (band ? hc->arena_count > 0 || hc->arena_long_count > 0 : deferred);
+  const bool left = hc->overflow_count > 0 || (band ? arena_left(hc) > 0 || arena_long_left(hc) > 0 : deferred);
   if (!left) return 0;
   cudaStream_t st = c->stream;
   cudaError_t e;
@@ -1202,7 +1218,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   cudaError_t e;
   const bool small = mode == 0 && small_call(ctx, n);
   if (small && dev) {
-    if ((e = ctx->poff.ensure(n + 1)) || (e = ctx->toff.ensure(n + 1)) || (e = ensure_work(ctx, n, 1, score_only)))
+    if ((e = ctx->poff.ensure(n + 1)) || (e = ctx->toff.ensure(n + 1)) || (e = ensure_work(ctx, n, n * (int64_t)wfa::kSlot, score_only)))
       return map_alloc(e);
     wfa::AlignArgs a = device_args(ctx, n, patterns, pattern_offsets, pattern_lengths, texts, text_offsets,
                                    text_lengths, pen, max_score, score_only, out_scores, out_status);
@@ -1298,9 +1314,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   if (arena_only) {
     if (!k.launched(wfa::launch_route_all(a, st))) return fail_cuda(k);
   } else if (small) {
-    if (!k.launched(wfa::launch_direct(a, ctx->band, reinterpret_cast<unsigned char*>(ctx->arena),
-                                       (long)ctx->arena_bytes, st)))
-      return fail_cuda(k);
+    if (!launch_small_align(ctx, k, a)) return fail_cuda(k);
   } else {
     if (!plain && (e = lane_order_args(ctx, a, n, ctx->h_ctrl->max_len, true))) return map_alloc(e);
     int vi = fixed_variant(ctx, a, ctx->h_ctrl->max_len);
@@ -1497,7 +1511,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
   // replay
   if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), n, nlong, max_len, true,
                                            reinterpret_cast<unsigned char*>(c->arena), (long)c->arena_bytes, st),
-                          wfa::kBandLaunches))
+                          wfa::band_launches(a)))
     return WFA_GPU_ECUDA;
   if (!k.ok(cudaEventRecordWithFlags(c->ev[3], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
   if (!score_only) {

@@ -25,6 +25,13 @@ __device__ __forceinline__ int cost_bin(int cls, unsigned cost) {
   return cls * kClassBins + (kClassBins - 1 - i);
 }
 
+// The arena kernels' pairs by length, longest first, in even steps up to the
+// call's longest: reads of one batch differ by less than a power of two.
+__device__ __forceinline__ int arena_bin(int cls, int len, int max_len) {
+  const int i = (int)((long long)len * kClassBins / ((long long)max(max_len, len) + 1));
+  return cls * kClassBins + (kClassBins - 1 - i);
+}
+
 // The deferred pairs, long ones first (their bounds take longest).
 __device__ __forceinline__ int32_t deferred(const AlignArgs& a, int i, int nlong) {
   return i < nlong ? a.defer_long_list[i] : a.defer_list[i - nlong];
@@ -46,6 +53,7 @@ __global__ void __launch_bounds__(32 * kBandWarps) bound_kernel(const AlignArgs 
   const int total = nlong + *(volatile const int32_t*)&a.ctrl->defer_count;
   const bool pen_ok = a.xs <= kBandMaxPen && a.oes <= kBandMaxPen && a.es <= kBandMaxPen;
   const int ring_bytes = 64 * band_rows(a.xs, a.oes, a.es);
+  const int max_len = *(volatile const int32_t*)&a.ctrl->max_len;
   int round = 0, flags[3];
   for (;;) {
     int i = 0;
@@ -54,7 +62,7 @@ __global__ void __launch_bounds__(32 * kBandWarps) bound_kernel(const AlignArgs 
     if (i >= total) return;
     const int32_t pair = deferred(a, i, nlong);
     const int n = a.plen[pair], m = a.tlen[pair];
-    int T = 0, bin = cost_bin(max(n, m) > kMediumMaxLen ? kArenaLong : kArena, (unsigned)max(n, m));
+    int T = 0, bin = arena_bin(max(n, m) > kMediumMaxLen ? kArenaLong : kArena, max(n, m), max_len);
     const bool lens_ok = n < kBandMaxLen && m < kBandMaxLen;
     if (pen_ok && lens_ok && ring_bytes + 4 * (band_words(n) + band_words(m)) <= warp_smem) {
       uint16_t* ring = reinterpret_cast<uint16_t*>(my);
@@ -353,6 +361,8 @@ cudaError_t launch_direct(const AlignArgs& a, const BandPlan& plan, unsigned cha
   return cudaGetLastError();
 }
 
+int band_launches(const AlignArgs& a) { return std::max(a.xs, std::max(a.oes, a.es)) <= kBandMaxPen ? 3 : 2; }
+
 cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int64_t nlong,
                         int max_len, bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st) {
   if (pairs <= 0) return cudaSuccess;
@@ -380,7 +390,7 @@ cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs
   const int64_t tiles = (pairs + kPlaceBlock * kPlaceItems - 1) / (kPlaceBlock * kPlaceItems);
   place_kernel<<<(unsigned)std::min<int64_t>(tiles, 2 * plan.nsm), kPlaceBlock, 0, st>>>(
       a, b.key, b.aux, b.aux + kBandBins, b.order, b.arena_list, b.arena_long_list);
-  if ((e = cudaGetLastError())) return e;
+  if ((e = cudaGetLastError()) || band_launches(a) < 3) return e;
   // CTAs: as many as are resident, at least 64 KiB of arena a warp, no more
   // than pairs (a team takes one at a time)
   int64_t grid = std::min<int64_t>((int64_t)plan.nsm * plan.per_sm[size], pairs);

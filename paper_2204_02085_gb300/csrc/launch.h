@@ -241,7 +241,9 @@ cudaError_t band_plan(int device, BandPlan* plan);
 // right, in the arena lists).  launches: kernels enqueued.
 cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int64_t nlong,
                         int max_len, bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
-constexpr int kBandLaunches = 3;
+// Kernels it enqueues: under scaled penalties above kBandMaxPen only those
+// that order the arena lists.
+int band_launches(const AlignArgs& a);
 // Calls of at most kDirectPairs pairs: every pair on a warp of its own, what
 // does not fit deferred.
 constexpr int kDirectPairs = 4096;

@@ -218,3 +218,78 @@ def test_call_order_where_it_stores_higher_scores(pkg, oracle_mod):
         _check(al.align(big, (16, 6, 2)), big_want)
         assert al.variant_name(al.timing()["short_variant"]) == "g4_l255_c197_i16"
         assert al.timing()["deferred_pairs"] == 0
+
+
+class _Device:
+    """A batch on the device, and room for its results."""
+
+    def __init__(self, b, words):
+        import torch
+
+        t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")  # noqa: E731
+        self.ins = [t(b.patterns), None, t(b.pattern_lengths), t(b.texts), None, t(b.text_lengths)]
+        self.s = torch.full((b.n,), -9, dtype=torch.int32, device="cuda:0")
+        self.st = torch.full((b.n,), 9, dtype=torch.int8, device="cuda:0")
+        self.w = torch.zeros(max(int(words), 1), dtype=torch.int32, device="cuda:0")
+        self.off = torch.full((b.n + 1,), -1, dtype=torch.int64, device="cuda:0")
+        torch.cuda.synchronize()
+
+    def run(self, al, **kw):
+        self.s.fill_(-9)
+        self.off.fill_(-1)
+        assert al.align_device(*self.ins, self.s, self.st, self.w, self.off, **kw) == 0
+        if kw.get("score_only"):
+            return self.s.cpu().numpy(), self.st.cpu().numpy()
+        off = self.off.cpu().numpy()
+        return self.s.cpu().numpy(), self.st.cpu().numpy(), self.w.cpu().numpy()[:off[-1]].view(np.uint32), off
+
+
+def _substituted(n, length, subs, seed):
+    from paper_2204_02085_gb300 import synth
+
+    rng = np.random.Generator(np.random.PCG64(seed))
+    t = rng.choice(list(b"ACGT"), size=(n, length)).astype(np.uint8)
+    p = t.copy()
+    for i in range(n):
+        at = rng.choice(length, size=int(rng.integers(0, subs + 1)), replace=False)
+        p[i, at] = rng.choice(list(b"ACGT"), size=len(at))
+    return synth.from_pairs([(x.tobytes(), y.tobytes()) for x, y in zip(p, t)])
+
+
+@pytest.mark.parametrize("n", [37, 4096, 6000])
+@pytest.mark.parametrize("length", [100, 200])
+def test_penalties_beyond_the_band_keep_short_reads(pkg, oracle_mod, n, length):
+    """Under a gap open of 41 the band kernels take no pair; reads with a few
+    substituted bases stay with the short-read kernels all the same."""
+    b = _substituted(n, length, 3, n + length)
+    want = oracle_mod.wfa_batch(b, (4, 41, 1), nthreads=16)
+    with pkg.Aligner(0, 1 << 28) as al:
+        d = _Device(b, want[3][-1])
+        for kw in ({}, {"graph": True}, {"graph": True}):
+            _check(d.run(al, pen=(4, 41, 1), **kw), want)
+            assert al.timing()["deferred_pairs"] == 0
+        _check(al.align(b, (4, 41, 1)), want)
+        assert al.timing()["deferred_pairs"] == 0
+
+
+@pytest.mark.parametrize("ends", [(0, 0, 0, 0), (0, 0, 30, 30)])
+@pytest.mark.parametrize("pen", [(19, 39, 3), (97, 103, 41), (4, 0, 33)])
+def test_penalties_beyond_the_band(pkg, oracle_mod, pen, ends):
+    """What the short-read kernels leave under such penalties: medium and long
+    pairs on the arena kernels, one call, host and device, graph replays."""
+    from paper_2204_02085_gb300 import synth
+
+    parts = [synth.random_pairs(60, 60, 240, seed=1, edit_rate=0.03), synth.random_pairs(20, 300, 900, seed=2, edit_rate=0.04),
+             synth.random_pairs(5, 2100, 2600, seed=3, edit_rate=0.02)]
+    b = synth.from_pairs([p.pair(i) for p in parts for i in range(p.n)])
+    want = oracle_mod.wfa_batch(b, pen, nthreads=16, ends=ends)
+    with pkg.Aligner(0, 4 << 30) as al:
+        al.set_ends_free(*ends)
+        _check(al.align(b, pen), want)
+        d = _Device(b, want[3][-1])
+        for kw in ({}, {"graph": True}, {"graph": True}, {"score_only": True}):
+            got = d.run(al, pen=pen, **kw)
+            if "score_only" in kw:
+                np.testing.assert_array_equal(got[0], want[0])
+            else:
+                _check(got, want)
