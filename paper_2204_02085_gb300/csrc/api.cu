@@ -246,8 +246,10 @@ struct Call {
   bool timing;
   int launches = 0;
   cudaError_t err = cudaSuccess;
+  bool capture = false;  // external event records become graph nodes: replays time their phases
   void rec(int i) {
-    if (timing && err == cudaSuccess) err = cudaEventRecord(c->ev[i], c->stream);
+    if ((timing || capture) && err == cudaSuccess)
+      err = cudaEventRecordWithFlags(c->ev[i], c->stream, capture ? cudaEventRecordExternal : cudaEventRecordDefault);
   }
   bool ok(cudaError_t e) {
     if (err == cudaSuccess) err = e;
@@ -1117,8 +1119,11 @@ bool enqueue_small(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int64_t* out_off,
   if (!k.launched(wfa::launch_small_finish(a.n, a.nruns, a.score_only ? nullptr : out_off, c->ctrl, c->h_ctrl_dev,
                                            c->h_total_dev, st)))
     return false;
-  return a.score_only || k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars,
-                                                        cap, c->ctrl, st));
+  if (!a.score_only && !k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars,
+                                                       cap, c->ctrl, st)))
+    return false;
+  k.rec(4);
+  return k.err == cudaSuccess;
 }
 
 // After a call's device work with a wait behind it (h_ctrl mirrors the
@@ -1136,6 +1141,7 @@ int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* 
   if (band && !finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
   const int rc = band || !deferred ? run_retries(c, k, a) : run_arena(c, k, a, 0);
   if (rc) return rc;
+  k.rec(3);
   if (!a.score_only) {
     if ((e = c->scan_tmp.ensure(wfa::scan_tmp_elems(a.n)))) return map_alloc(e);
     if (!k.launched(wfa::launch_scan(a.nruns, a.n, 0, out_off, c->scan_tmp.p, st), 3) ||
@@ -1144,6 +1150,7 @@ int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* 
         !total_to_host(k, out_off + a.n, st))
       return WFA_GPU_ECUDA;
   }
+  k.rec(4);
   return k.ok(cudaStreamSynchronize(st)) ? 0 : WFA_GPU_ECUDA;
 }
 
@@ -1158,13 +1165,10 @@ int align_small(wfa_gpu_ctx* ctx, Call& k, wfa::AlignArgs& a, uint32_t* out_ciga
   if (rc) return rc;
   if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
   if (k.timing) {
-    k.rec(4);
-    k.rec(5);
-    if (!k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
     ctx->last.align_ms = elapsed(ctx, 1, 2);
     ctx->last.general_ms = elapsed(ctx, 2, 3);
     ctx->last.cigar_ms = elapsed(ctx, 3, 4);
-    ctx->last.total_ms = elapsed(ctx, 0, 5);
+    ctx->last.total_ms = elapsed(ctx, 0, 4);
   }
   ctx->last.kernel_launches = k.launches;
   ctx->last.short_variant = -1;
@@ -1468,15 +1472,11 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
                         bool band, int64_t nlong, int max_len) {
   cudaStream_t st = c->stream;
   const bool score_only = flags & WFA_GPU_SCORE_ONLY;
-  // external event records become graph nodes: replays time their phases
-  if (!k.ok(cudaEventRecordWithFlags(c->ev[0], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+  k.rec(0);
   if (small_call(c, n)) {
     wfa::AlignArgs a =
         device_args(c, n, pat, poff, plen, txt, toff, tlen, pen, max_score, score_only, out_scores, out_status);
-    for (int i : {1, 2, 3})
-      if (!k.ok(cudaEventRecordWithFlags(c->ev[i], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
-    if (!enqueue_small(c, k, a, out_off, out_cigars, cap, band, nlong, max_len)) return WFA_GPU_ECUDA;
-    return k.ok(cudaEventRecordWithFlags(c->ev[4], st, cudaEventRecordExternal)) ? 0 : WFA_GPU_ECUDA;
+    return enqueue_small(c, k, a, out_off, out_cigars, cap, band, nlong, max_len) ? 0 : WFA_GPU_ECUDA;
   }
   if (!k.ok(cudaMemsetAsync(c->ctrl, 0, sizeof(wfa::Ctrl), st))) return WFA_GPU_ECUDA;
   const int64_t* d_poff = poff;
@@ -1498,7 +1498,7 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
     }
     if (!k.launched(wfa::launch_validate(n, d_poff, plen, d_toff, tlen, c->ctrl, st))) return WFA_GPU_ECUDA;
   }
-  if (!k.ok(cudaEventRecordWithFlags(c->ev[1], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+  k.rec(1);
   wfa::AlignArgs a = device_args(c, n, pat, d_poff, plen, txt, d_toff, tlen, pen, max_score, score_only,
                                  out_scores, out_status);
   if (c->last_variant < 0) return WFA_GPU_ECUDA;
@@ -1506,22 +1506,22 @@ int enqueue_device_work(wfa_gpu_ctx* c, Call& k, int64_t n, const char* pat, con
   if (!k.launched(wfa::launch_short(a, c->plan.v[c->last_variant], st),
                   wfa::short_launches(a, c->plan.v[c->last_variant])))
     return WFA_GPU_ECUDA;
-  if (!k.ok(cudaEventRecordWithFlags(c->ev[2], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+  k.rec(2);
   // pairs the band kernels leave to the arena kernels are finished after the
   // replay
   if (band && !k.launched(wfa::launch_band(a, c->band, band_bufs(c), n, nlong, max_len, true,
                                            reinterpret_cast<unsigned char*>(c->arena), (long)c->arena_bytes, st),
                           wfa::band_launches(a)))
     return WFA_GPU_ECUDA;
-  if (!k.ok(cudaEventRecordWithFlags(c->ev[3], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
+  k.rec(3);
   if (!score_only) {
     if (!k.launched(wfa::launch_scan(c->nruns.p, n, 0, out_off, c->scan_tmp.p, st), 3) ||
         !k.launched(wfa::launch_compact(n, c->nruns.p, c->run_src.p, c->runs.p, c->pool.p, out_off, out_cigars, cap,
                                         c->ctrl, st)))
       return WFA_GPU_ECUDA;
   }
-  if (!k.ok(cudaEventRecordWithFlags(c->ev[4], st, cudaEventRecordExternal))) return WFA_GPU_ECUDA;
-  return 0;
+  k.rec(4);
+  return k.err == cudaSuccess ? 0 : WFA_GPU_ECUDA;
 }
 
 // Key of a graph: the call's arguments and every internal buffer the
@@ -1578,6 +1578,7 @@ int align_graph(wfa_gpu_ctx* ctx, int64_t n, const char* pat, const int64_t* pof
     const wfa_gpu_timing eager_timing = ctx->last;
     cudaStream_t st = ctx->stream;
     Call k{ctx, false};
+    k.capture = true;
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return WFA_GPU_ECUDA;
     // the band kernels only when the eager run deferred pairs: with nothing

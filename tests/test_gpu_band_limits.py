@@ -293,3 +293,20 @@ def test_penalties_beyond_the_band(pkg, oracle_mod, pen, ends):
                 np.testing.assert_array_equal(got[0], want[0])
             else:
                 _check(got, want)
+
+
+def test_small_replays_time_their_phases(pkg):
+    """The phases of a small call, eager and replayed: of a replay, which has
+    no host work between them, the alignment is the larger part, and the
+    phases make up the call."""
+    b = _substituted(4096, 200, 12, 4)
+    with pkg.Aligner(0, 1 << 28) as al:
+        d = _Device(b, 64 * b.n)
+        for i, kw in enumerate(({}, {"graph": True}, {"graph": True}, {"graph": True})):
+            d.run(al, timing=True, **kw)
+            t = al.timing()
+            assert t["deferred_pairs"] == 0
+            assert t["align_ms"] > 0 and t["cigar_ms"] > 0
+            if i >= 2:  # (the call before captures)
+                assert t["align_ms"] > 0.4 * t["total_ms"]
+            assert t["align_ms"] + t["general_ms"] + t["cigar_ms"] <= 1.001 * t["total_ms"]
