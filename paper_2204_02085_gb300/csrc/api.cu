@@ -153,6 +153,7 @@ struct wfa_gpu_ctx {
   DevBuf<int2> lane_slots;
   int variant_forced = -1;  // tuning override (WFA_GPU_SHORT_VARIANT)
   int last_variant = -1;
+  bool above_store = false;  // the call's sample held pairs above the chosen store
   wfa::Ctrl* ctrl = nullptr;    // device
   wfa::Ctrl* h_ctrl = nullptr;  // pinned host mirror
   int64_t* h_total = nullptr;   // pinned host scalar
@@ -513,8 +514,14 @@ bool finish_arena_lists(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a) {
 // over what those leave (mode 2, arena only: over every pair), then retries
 // of the pairs that did not fit: fewer, larger arena slices on one-CTA
 // teams, or a larger CIGAR pool.  A pair that does not fit the whole arena
-// gives ENOMEM.
-int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode) {
+// gives ENOMEM.  layout: lays out the CIGARs of a device-pointer call, before
+// the wait on the band kernels (nearly always the last one) and again after
+// whatever they left.
+struct NoLayout {
+  bool operator()() const { return true; }
+};
+template <class Layout>
+int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode, Layout layout) {
   cudaStream_t st = c->stream;
   wfa::Ctrl* hc = c->h_ctrl;
   wfa::Ctrl* dc = c->ctrl;
@@ -534,9 +541,12 @@ int run_arena(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, int mode) {
   if (!band_penalties(a) && !launch_arena_lists(c, k, a, c->arena_list.p, &dc->arena_count, hc->defer_count,
                                                 c->arena_long_list.p, &dc->arena_long_count, hc->defer_long_count))
     return WFA_GPU_ECUDA;
-  if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+  if (!layout() || !ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return WFA_GPU_ECUDA;
+  if (arena_left(hc) == 0 && arena_long_left(hc) == 0 && hc->overflow_count == 0) return 0;
   if (!finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
-  return run_retries(c, k, a);
+  const int rc = run_retries(c, k, a);
+  if (rc) return rc;
+  return layout() && k.ok(cudaStreamSynchronize(st)) ? 0 : WFA_GPU_ECUDA;
 }
 
 // Retries of the pairs on the overflow list (h_ctrl mirrors the device
@@ -704,18 +714,23 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
     };
     int best = cand[0];
     double best_ns = above_ns(s_store[0]);
+    c->above_store = best_ns > 0;
     for (int j = 1; j < ncand; ++j) {
-      const double ns = n * step_ns * j + above_ns(s_store[j]);
+      const double above = above_ns(s_store[j]), ns = n * step_ns * j + above;
       if (ns < best_ns) {
         best = cand[j];
         best_ns = ns;
+        c->above_store = above > 0;
       }
     }
     if (max_len > 127) {  // the kernel in call order, where it stores higher scores
       const wfa::ShortVariant& v = c->plan.v[c->variant_mid[model]];
       wfa::UGeo tab[64];
-      if (n * kCallOrderNs + above_ns(wfa::build_ugeo(tab, v.scap, v.cells, pen, 0, 0)) < best_ns)
+      const double above = above_ns(wfa::build_ugeo(tab, v.scap, v.cells, pen, 0, 0));
+      if (n * kCallOrderNs + above < best_ns) {
         best = c->variant_mid[model];
+        c->above_store = above > 0;
+      }
     }
     return best;
   }
@@ -740,6 +755,7 @@ int autotune_short(wfa_gpu_ctx* c, Call& k, const wfa::AlignArgs& a_in, int64_t 
   int64_t fit[5] = {0, 0, 0, 0, 0}, tot = 0;
   for (int64_t i = 0; i < m; ++i) {
     const int sc = c->h_tune[i];
+    c->above_store = c->above_store || sc < 0;
     if (sc < 0) continue;  // deferred, invalid or over the bound: not informative
     ++tot;
     for (int j = 0; j < ncand; ++j) fit[j] += (sc / a.g <= s_store[j]);
@@ -1019,7 +1035,7 @@ int align_pipelined(wfa_gpu_ctx* ctx, Call& k, const wfa::AlignArgs& a, int64_t 
     const int64_t dc = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
     deferred += dc;
     if (dc > 0) {
-      const int rc = run_arena(ctx, k, ac, mode);
+      const int rc = run_arena(ctx, k, ac, mode, NoLayout());
       if (rc) return rc;
       if (!scan() || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
     }
@@ -1138,20 +1154,23 @@ int finish_left(wfa_gpu_ctx* c, Call& k, wfa::AlignArgs& a, bool band, int64_t* 
   if (!left) return 0;
   cudaStream_t st = c->stream;
   cudaError_t e;
+  if (!a.score_only && (e = c->scan_tmp.ensure(wfa::scan_tmp_elems(a.n)))) return map_alloc(e);
+  const auto layout = [&]() {
+    k.rec(3);
+    if (!a.score_only &&
+        (!k.launched(wfa::launch_scan(a.nruns, a.n, 0, out_off, c->scan_tmp.p, st), 3) ||
+         !k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars, cap, c->ctrl,
+                                         st)) ||
+         !total_to_host(k, out_off + a.n, st)))
+      return false;
+    k.rec(4);
+    return k.err == cudaSuccess;
+  };
+  if (deferred && !band) return run_arena(c, k, a, 0, layout);
   if (band && !finish_arena_lists(c, k, a)) return WFA_GPU_ECUDA;
-  const int rc = band || !deferred ? run_retries(c, k, a) : run_arena(c, k, a, 0);
+  const int rc = run_retries(c, k, a);
   if (rc) return rc;
-  k.rec(3);
-  if (!a.score_only) {
-    if ((e = c->scan_tmp.ensure(wfa::scan_tmp_elems(a.n)))) return map_alloc(e);
-    if (!k.launched(wfa::launch_scan(a.nruns, a.n, 0, out_off, c->scan_tmp.p, st), 3) ||
-        !k.launched(wfa::launch_compact(a.n, a.nruns, a.run_src, a.runs, a.pool, out_off, out_cigars, cap, c->ctrl,
-                                        st)) ||
-        !total_to_host(k, out_off + a.n, st))
-      return WFA_GPU_ECUDA;
-  }
-  k.rec(4);
-  return k.ok(cudaStreamSynchronize(st)) ? 0 : WFA_GPU_ECUDA;
+  return layout() && k.ok(cudaStreamSynchronize(st)) ? 0 : WFA_GPU_ECUDA;
 }
 
 // A small device-pointer call on the default path.
@@ -1197,6 +1216,7 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
   if (cudaSetDevice(ctx->device) != cudaSuccess) return WFA_GPU_ECUDA;
   std::memset(&ctx->last, 0, sizeof ctx->last);
   ctx->last_variant = -1;
+  ctx->above_store = false;
   cudaStream_t st = ctx->stream;
   Call k{ctx, (flags & WFA_GPU_TIMING) != 0};
   if (n == 0) {
@@ -1331,30 +1351,48 @@ int align_eager(wfa_gpu_ctx* ctx, int64_t n, const char* patterns, const int64_t
       return fail_cuda(k);
   }
   k.rec(2);
-  const auto scan_compact = [&]() {  // device-pointer calls (the compaction checks the capacity)
-    return score_only || (k.launched(wfa::launch_scan(ctx->nruns.p, n, 0, out_cigar_offsets, ctx->scan_tmp.p, st), 3) &&
-                          total_to_host(k, out_cigar_offsets + n, st) &&
-                          k.launched(wfa::launch_compact(n, ctx->nruns.p, ctx->run_src.p, ctx->runs.p, ctx->pool.p,
-                                                         out_cigar_offsets, out_cigars, cap, ctx->ctrl, st)));
-  };
-  // a device-pointer call whose pairs all fit their kernel is done with this
-  // wait; deferred pairs are aligned and the CIGARs laid out again after it
+  // A device-pointer call on the default path lays out its CIGARs (the
+  // compaction checks the capacity) before the wait that ends it: the first one
+  // when no pair is deferred, else the one on the band kernels.  Not ahead of
+  // the first when the sample held pairs above the store: the layout would be
+  // done twice (200,000 reads of 160-200 bases at 0-4 % under 1/1/1 484 us a
+  // call, now 456).
   const bool ahead = dev && mode == 0;
-  if (ahead && !k.timing && !scan_compact()) return fail_cuda(k);
+  const auto layout = [&]() {
+    if (!ahead) return true;
+    k.rec(3);
+    if (!score_only &&
+        (!k.launched(wfa::launch_scan(ctx->nruns.p, n, 0, out_cigar_offsets, ctx->scan_tmp.p, st), 3) ||
+         !total_to_host(k, out_cigar_offsets + n, st) ||
+         !k.launched(wfa::launch_compact(n, ctx->nruns.p, ctx->run_src.p, ctx->runs.p, ctx->pool.p, out_cigar_offsets,
+                                         out_cigars, cap, ctx->ctrl, st))))
+      return false;
+    k.rec(4);
+    return k.err == cudaSuccess;
+  };
+  const bool laid = !ctx->above_store;
+  if (laid && !layout()) return fail_cuda(k);
   if (!ctrl_to_host(k, st) || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
   ctx->last.deferred_pairs = (int64_t)ctx->h_ctrl->defer_count + ctx->h_ctrl->defer_long_count;
-  const bool deferred = ctx->last.deferred_pairs > 0;
-  if (deferred || ctx->h_ctrl->overflow_count > 0) {
-    rc = deferred ? run_arena(ctx, k, a, mode) : run_retries(ctx, k, a);
+  if (ctx->last.deferred_pairs > 0) {
+    rc = run_arena(ctx, k, a, mode, layout);
     if (rc) return rc;
+  } else if (ctx->h_ctrl->overflow_count > 0 || !laid) {
+    rc = run_retries(ctx, k, a);
+    if (rc) return rc;
+    if (!layout() || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
   }
   if (ctx->h_ctrl->internal_error) return WFA_GPU_ECUDA;
-  if (ahead && !k.timing) {
-    if (deferred || ctx->h_ctrl->overflow_count > 0) {
-      if (!scan_compact() || !k.ok(cudaStreamSynchronize(st))) return fail_cuda(k);
-    }
+  if (ahead) {
     ctx->last.kernel_launches = k.launches;
     ctx->last.short_variant = ctx->last_variant;
+    if (k.timing) {
+      ctx->last.h2d_ms = elapsed(ctx, 0, 1);
+      ctx->last.align_ms = elapsed(ctx, 1, 2);
+      ctx->last.general_ms = elapsed(ctx, 2, 3);
+      ctx->last.cigar_ms = elapsed(ctx, 3, 4);
+      ctx->last.total_ms = elapsed(ctx, 0, 4);
+    }
     return !score_only && *ctx->h_total > cap ? WFA_GPU_ECIGAR_CAPACITY : WFA_GPU_OK;
   }
   k.rec(3);

@@ -310,3 +310,29 @@ def test_small_replays_time_their_phases(pkg):
             if i >= 2:  # (the call before captures)
                 assert t["align_ms"] > 0.4 * t["total_ms"]
             assert t["align_ms"] + t["general_ms"] + t["cigar_ms"] <= 1.001 * t["total_ms"]
+
+
+@pytest.mark.parametrize("hard", [0, 1, 40])
+def test_timed_calls_run_the_same_kernels(pkg, oracle_mod, hard):
+    """WFA_GPU_TIMING only measures: as many kernels as without, with no pair
+    deferred, one the sample does not see, and many; the phases make up the
+    call."""
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.uniform_reads(6000, 100, 2, seed=12)
+    pairs = [b.pair(i) for i in range(b.n)]
+    unrelated = synth.random_pairs(hard, 100, 100, seed=13) if hard else None
+    for j in range(hard):
+        pairs[(5990 + 211 * j) % 6000] = unrelated.pair(j)
+    b = synth.from_pairs(pairs)
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=16)
+    with pkg.Aligner(0, 1 << 28) as al:
+        d = _Device(b, want[3][-1])
+        _check(d.run(al), want)
+        launches = al.timing()["kernel_launches"]
+        assert al.timing()["deferred_pairs"] == hard
+        _check(d.run(al, timing=True), want)
+        t = al.timing()
+        assert t["kernel_launches"] == launches and t["deferred_pairs"] == hard
+        assert t["align_ms"] > 0 and t["cigar_ms"] > 0 and (t["general_ms"] > 0.01) == (hard > 0)
+        assert t["h2d_ms"] + t["align_ms"] + t["general_ms"] + t["cigar_ms"] <= 1.001 * t["total_ms"]
