@@ -336,3 +336,102 @@ def test_timed_calls_run_the_same_kernels(pkg, oracle_mod, hard):
         assert t["kernel_launches"] == launches and t["deferred_pairs"] == hard
         assert t["align_ms"] > 0 and t["cigar_ms"] > 0 and (t["general_ms"] > 0.01) == (hard > 0)
         assert t["h2d_ms"] + t["align_ms"] + t["general_ms"] + t["cigar_ms"] <= 1.001 * t["total_ms"]
+
+
+def _launches(al):
+    return al.timing()["kernel_launches"]
+
+
+def test_direct_pairs_that_outgrow_their_slice(pkg, oracle_mod):
+    """Small calls of unrelated pairs of some 500 bases under 3/0/2: 600 rows of
+    ten blocks, more than the 64 KiB a warp gets of 2 MiB, within the whole of
+    it."""
+    from paper_2204_02085_gb300 import synth
+
+    b = synth.random_pairs(32, 470, 500, seed=41)
+    pen = (3, 0, 2)
+    want = oracle_mod.wfa_batch(b, pen, nthreads=16)
+    count = []
+    for arena in (1 << 30, 2 << 20):
+        with pkg.Aligner(0, arena) as al:
+            d = _Device(b, want[3][-1])
+            for kw in ({}, {"graph": True}, {"graph": True}):
+                _check(d.run(al, pen=pen, **kw), want)
+                count.append(_launches(al))
+            assert al.timing()["deferred_pairs"] < 16  # (those whose rows do not fit a warp)
+            _check(al.align(b, pen), want)
+    assert all(small > big for big, small in zip(count[:3], count[3:]))
+
+
+@pytest.mark.parametrize("n", [16, 4200])
+def test_band_pairs_that_outgrow_their_slice(pkg, oracle_mod, n):
+    """Unrelated medium pairs in 4 MiB: more choice bits than a team's 256 KiB;
+    eager, replayed and through host memory, the retries lay the CIGARs out
+    again."""
+    from paper_2204_02085_gb300 import synth
+
+    hard = synth.random_pairs(16, 640, 670, seed=42)
+    b = synth.from_pairs([hard.pair(i) for i in range(16)] + [(b"ACGTTG" * 15, b"ACGTTG" * 15)] * (n - 16))
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=16)
+    count = []
+    for arena in (1 << 30, 4 << 20):
+        with pkg.Aligner(0, arena) as al:
+            d = _Device(b, want[3][-1])
+            for kw in ({}, {"graph": True}, {"graph": True}):
+                _check(d.run(al, **kw), want)
+                count.append(_launches(al))
+            assert al.timing()["deferred_pairs"] == 16
+            _check(al.align(b, (4, 6, 2)), want)
+    assert all(small > big for big, small in zip(count[:3], count[3:]))
+
+
+def test_longest_band_pairs(pkg, oracle_mod):
+    """Lengths around the band kernels' last two sizes (12,000 and 32,000
+    bases), the longest handed to the arena kernels."""
+    from paper_2204_02085_gb300 import synth
+
+    pairs = []
+    for j, n in enumerate((12_000, 12_001, 31_999, 32_000)):
+        b = synth.random_pairs(2, n, n, seed=50 + j, edit_rate=0.004)
+        pairs += [(p[:n], t) for p, t in (b.pair(0), b.pair(1))]
+    pairs += [(pairs[4][1][:31_990], pairs[4][1]), (pairs[4][1], pairs[4][1][9:])]
+    b = synth.from_pairs(pairs)
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=10)
+    with pkg.Aligner(0, 4 << 30) as al:
+        _check(al.align(b, (4, 6, 2)), want)
+        s, st, _, _ = al.align(b, (4, 6, 2), score_only=True)
+        np.testing.assert_array_equal(s, want[0])
+        np.testing.assert_array_equal(st, want[1])
+
+
+def test_many_long_pairs_on_four_warps(pkg, oracle_mod):
+    """More long pairs than blocks of four warps: no blocks of eight, narrow
+    pairs a warp each, wide ones on teams of four."""
+    from paper_2204_02085_gb300 import synth
+
+    easy = synth.random_pairs(60, 2049, 2300, seed=60, edit_rate=0.01)
+    wide = synth.random_pairs(24, 2049, 2300, seed=61, edit_rate=0.18)
+    b = synth.from_pairs([easy.pair(i % 60) for i in range(1140)] + [wide.pair(i) for i in range(24)])
+    want = oracle_mod.wfa_batch(b, (4, 6, 2), nthreads=16)
+    with pkg.Aligner(0, 4 << 30) as al:
+        _check(al.align(b, (4, 6, 2)), want)
+        s, _, _, _ = al.align(b, (4, 6, 2), score_only=True)
+        np.testing.assert_array_equal(s, want[0])
+
+
+@pytest.mark.parametrize("pen", [(10, 3, 2), (9, 1, 2)])
+@pytest.mark.parametrize("ends", [(0, 0, 300, 300), (40, 40, 40, 40), (0, 7, 9, 0)])
+def test_free_ends_with_dear_mismatches(pkg, oracle_mod, pen, ends):
+    """Scores without a wavefront between older gaps (x well above o + 2 e):
+    the rows left out there keep gap cells of lower scores."""
+    from paper_2204_02085_gb300 import synth
+
+    parts = [synth.random_pairs(80, 1, 300, seed=70, edit_rate=0.05), synth.random_pairs(20, 260, 300, seed=71),
+             _windows(60, 200, 120, 0.05, 72)]
+    b = synth.from_pairs([p.pair(i) for p in parts for i in range(p.n)])
+    want = oracle_mod.wfa_batch(b, pen, nthreads=16, ends=ends)
+    with pkg.Aligner(0, 1 << 30) as al:
+        al.set_ends_free(*ends)
+        _check(al.align(b, pen), want)  # a warp per pair from bytes to CIGAR
+        big, big_want = _tiled(b, want, 30)
+        _check(al.align(big, pen), big_want)  # the deferred pairs on the band kernels
