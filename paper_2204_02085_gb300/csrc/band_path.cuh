@@ -567,7 +567,7 @@ __device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int
   // first warp: the CIGAR, into a reservation of the run pool
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int most = s / min(a.xs, a.oes);  // events
+  const int most = min(s / min(a.xs, a.oes), n + m);  // events: each costs that much, and takes a base
   const unsigned long long want = 2ull * most + 3;
   unsigned long long pos = 0;
   if (lane == 0) pos = atomicAdd(&a.ctrl->pool_top, want);

@@ -435,3 +435,30 @@ def test_free_ends_with_dear_mismatches(pkg, oracle_mod, pen, ends):
         _check(al.align(b, pen), want)  # a warp per pair from bytes to CIGAR
         big, big_want = _tiled(b, want, 30)
         _check(al.align(big, pen), big_want)  # the deferred pairs on the band kernels
+
+
+def test_dear_gaps_reserve_no_more_than_their_bases(pkg, oracle_mod):
+    """Under 1/0/31 a gap of 130 bases scores 4,030 and a mismatch 1: the pool's
+    room for a CIGAR is bounded by the bases, not by the score alone, and 1,000
+    such pairs fit as 20 do (no retry: as many kernels)."""
+    from paper_2204_02085_gb300 import synth
+
+    rng = np.random.Generator(np.random.PCG64(80))
+
+    def seq(n):
+        return rng.choice(list(b"ACGT"), size=n).astype(np.uint8).tobytes()
+
+    pairs = []
+    for _ in range(20):
+        t = seq(600)
+        pairs.append((t, t[:300] + seq(130) + t[300:]))
+    b = synth.from_pairs(pairs)
+    want = oracle_mod.wfa_batch(b, (1, 0, 31), nthreads=16)
+    big, big_want = _tiled(b, want, 50)
+    count = []
+    for one, w in ((b, want), (big, big_want)):
+        with pkg.Aligner(0, 1 << 30) as al:  # (a context's first call: a retry would grow the pool)
+            _check(_Device(one, w[3][-1]).run(al, pen=(1, 0, 31)), w)
+            assert al.timing()["deferred_pairs"] == one.n
+            count.append(_launches(al))
+    assert count[0] == count[1]
