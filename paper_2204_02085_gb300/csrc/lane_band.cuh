@@ -163,6 +163,10 @@ __device__ __forceinline__ uint32_t lane_planes16(uint4 v, uint32_t* bad16) {
   return code;
 }
 
+// Aligned 16-byte chunks that hold a base of a sequence starting h bytes into
+// the first (none of an empty one, whose address need not be anyone's).
+__host__ __device__ inline int lane_chunks(int h, int len) { return len > 0 ? (h + len + 15) >> 4 : 0; }
+
 // One lane packs one sequence of at most 32 * NP - 1 bases from device memory
 // into NP words of each bit plane (word j of plane q at out[(q * NP + j) *
 // 32]): every aligned 16-byte chunk holding a base is loaded at once, then
@@ -173,7 +177,7 @@ __device__ __forceinline__ bool lane_pack_planes(const char* seq, int len, uint3
   constexpr int NCH = 2 * NP + 1;
   const unsigned long long a0 = reinterpret_cast<uintptr_t>(seq), b0 = a0 & ~15ull;
   const int h = (int)(a0 - b0);
-  const int nch = (h + len + 15) >> 4;
+  const int nch = lane_chunks(h, len);
   uint4 raw[NCH];
 #pragma unroll
   for (int c = 0; c < NCH; ++c)  // all loads first: their latencies overlap

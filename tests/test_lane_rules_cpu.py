@@ -19,7 +19,7 @@ def ask(tmp_path_factory):
     def run(body):
         src, exe = str(work / "rules.cu"), str(work / "rules")
         with open(src, "w") as f:
-            f.write('#include <cstdio>\n#include <ctime>\n#include "launch.h"\nusing namespace wfa;\nint main() {\n' + body + "\n}\n")
+            f.write('#include <cstdio>\n#include <ctime>\n#include "lane_band.cuh"\nusing namespace wfa;\nint main() {\n' + body + "\n}\n")
         cmd = [build.nvcc(), *build.ARCH, "-std=c++17", "-cudart", "shared", "-I" + build.INCLUDE, "-I" + build.CSRC,
                src, "-o", exe, build.OUT, "-Xlinker", "-rpath=" + os.path.dirname(build.OUT)]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -102,3 +102,20 @@ def test_plans_of_a_call_are_worked_out_once(ask):
       printf("%d %f", same ? 1 : 0, ((t1.tv_sec - t0.tv_sec) * 1e6 + (t1.tv_nsec - t0.tv_nsec) * 1e-3) / (500 * 20));""")
     assert got[0] == "1"
     assert float(got[1]) < 2.0, got  # us an answer
+
+
+def test_empty_sequences_have_no_bytes(ask):
+    """The ordering pass loads the aligned 16-byte chunks that hold a base: of
+    an empty sequence none, wherever its offset points."""
+    got = ask("""
+      for (int h = 0; h < 16; ++h) {
+        int most = 0;
+        bool ok = lane_chunks(h, 0) == 0;
+        for (int len = 1; len <= 255; ++len) {
+          int chunks = 0;
+          for (int c = 0; c < 17; ++c) chunks += 16 * c < h + len && 16 * c + 16 > h;
+          ok = ok && lane_chunks(h, len) == chunks;
+        }
+        printf("%d ", ok ? 1 : 0);
+      }""")
+    assert got == ["1"] * 16
