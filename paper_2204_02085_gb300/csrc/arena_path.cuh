@@ -1,5 +1,5 @@
-// arena_path.cuh -- the gap-affine WFA for pairs that do not fit the
-// short-read kernel: medium and long reads, or high scores.
+// arena_path.cuh -- the gap-affine WFA for pairs the band kernels leave
+// (launch_band says which) and arena-only calls.
 //
 // A team -- one warp, or a whole CTA of WPP warps for long reads -- owns one
 // pair at a time; its threads stride over the diagonals of each wavefront.

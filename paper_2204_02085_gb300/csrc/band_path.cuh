@@ -51,7 +51,6 @@ namespace wfa {
 
 constexpr uint32_t kBandNull = 0xFFFFu;
 constexpr uint32_t kBandValid = 0x8000u;  // u below this is an offset
-constexpr int kBandMaxLen = 32000;        // u fits 15 bits
 constexpr int kBandWarps = 4;             // warps of a CTA (and of a team); twice as many when few pairs are long
 // Rows wider than this (or than a warp's share of the shared memory): a team,
 // whose every row costs each of its warps the fixed part and a barrier
@@ -123,23 +122,22 @@ __device__ __forceinline__ int band_extend(const uint32_t* pw, const uint32_t* t
 
 // ---------------------------------------------------------------- bound
 
-// The search for a pair's bound, a row at a time, on kLanes lanes (a warp
-// for one pair): lane l holds the diagonal k = l (mod kLanes) of the window b .. b +
-// kLanes - 1, its rows the band_rows(...) * kLanes cells at ring.  Every
-// fourth score the window moves when its furthest cell (largest v + h) comes
-// within a quarter of an edge.  On every sampled pair of 100 to 10,000 bases
-// at up to 10 % edits the bound found was the optimum itself.  (Half a warp
-// per pair found it too, but two pairs' extensions in one warp wait for each
-// other: 260 instructions a score for two pairs against 148 for one, and
-// twice the latency on long reads.)
-template <int kLanes>
+// The search for a pair's bound, a row at a time, on one warp: lane l holds
+// the diagonal k = l (mod 32) of the window b .. b + 31, its rows the
+// band_rows(...) * 32 cells at ring.  Every fourth score the window moves when
+// its furthest cell (largest v + h) comes within a quarter of an edge.  On
+// every sampled pair of 100 to 10,000 bases at up to 10 % edits the bound found
+// was the optimum itself.  (Half a warp per pair found it too, but two pairs'
+// extensions in one warp wait for each other: 260 instructions a score for two
+// pairs against 148 for one, and twice the latency on long reads.)
 struct BandSearch {
+  static constexpr int kLanes = 32;
+  static constexpr unsigned kAll = 0xffffffffu;
   const uint32_t *pw, *tw;
   uint16_t* ring;
   int n, m, kf, elo, ehi, b, k, s, cap;
   int rs, rx, ro, rn, re;  // ring rows of the scores s, s - x, s - o - e (M), s, s - e (I, D)
 
-  __device__ static unsigned mask() { return group_mask(kLanes); }
   __device__ static int lane() { return threadIdx.x & (kLanes - 1); }
 
   // Score 0; true when it reaches an end.
@@ -165,7 +163,7 @@ struct BandSearch {
         const int len = rem > 0 ? band_extend(pw, tw, v, h, rem) : 0;
         best = max(best, (len << 16) | (q - g.lo0));  // lengths < 32,768: no overlap with the sign
       }
-      b = g.lo0 + (__reduce_max_sync(mask(), best) & 0xFFFF) - kLanes / 2;
+      b = g.lo0 + (__reduce_max_sync(kAll, best) & 0xFFFF) - kLanes / 2;
     }
     k = b + ((l - b) & (kLanes - 1));
     bool fin = false;
@@ -175,9 +173,9 @@ struct BandSearch {
       ring[l] = (uint16_t)u;
       fin = u == 0 && k >= elo && k <= ehi;
     }
-    __syncwarp(mask());
+    __syncwarp(kAll);
     rs = 1 % R, rx = (1 - x + R) % R, ro = (1 - oe + R) % R, rn = 1 % RE, re = 2 % RE;
-    return __any_sync(mask(), fin);
+    return __any_sync(kAll, fin);
   }
 
   // The next score; true when it reaches an end.
@@ -207,9 +205,9 @@ struct BandSearch {
     ring[rs * kLanes + l] = (uint16_t)u;
     I[rn * kLanes + l] = (uint16_t)uI;
     D[rn * kLanes + l] = (uint16_t)uD;
-    __syncwarp(mask());
+    __syncwarp(kAll);
     if ((s & 3) == 0) {
-      const int best = __reduce_max_sync(mask(), (far << 5) | l);
+      const int best = __reduce_max_sync(kAll, (far << 5) | l);
       const int at = ((best & 31) - b) & (kLanes - 1);
       if (best >= 32 && (at < kLanes / 4 || at >= kLanes - kLanes / 4)) {
         b += at - kLanes / 2;
@@ -217,7 +215,7 @@ struct BandSearch {
         if (k2 != k)
           for (int r = 0; r < R + 2 * RE; ++r) ring[r * kLanes + l] = (uint16_t)kBandNull;
         k = k2;
-        __syncwarp(mask());
+        __syncwarp(kAll);
       }
     }
     rs = rs + 1 == R ? 0 : rs + 1;
@@ -225,7 +223,7 @@ struct BandSearch {
     ro = ro + 1 == R ? 0 : ro + 1;
     rn = rn + 1 == RE ? 0 : rn + 1;
     re = re + 1 == RE ? 0 : re + 1;
-    return __any_sync(mask(), fin);
+    return __any_sync(kAll, fin);
   }
 };
 
@@ -233,7 +231,7 @@ struct BandSearch {
 // most cap (itself a bound, or the caller's largest score of interest).
 __device__ __forceinline__ int band_bound(const uint32_t* pw, const uint32_t* tw, const BandGeo& g, int x, int oe,
                                           int e, int cap, uint16_t* ring) {
-  BandSearch<32> w;
+  BandSearch w;
   if (w.start(pw, tw, g, x, oe, e, cap, ring)) return 0;
   while (w.s + 1 < cap)
     if (w.step(x, oe, e)) return w.s;
@@ -251,9 +249,16 @@ __device__ __forceinline__ int band_worst(int n, int m, int x, int oe, int e) {
 
 // -------------------------------------------------------------- forward
 
-// The scores without a wavefront among the first max(x, o + e) (bit s): no
-// older row has written their row positions, so they need not be written
-// either.
+// The scores without a wavefront among the first max(x, o + e) + 1 (bit s):
+// their rows need not be written.  M's ring positions of such a score are
+// still null: each score up to max(x, o + e) is the first to use its own.  I
+// and D's rings are shorter: where e >= 2 and x lies well above o + 2 e, a row
+// left out may show the gap cells of e + 1 scores before (x = 10, o + e = 5, e =
+// 2: score 8 has no wavefront, and its I and D positions hold score 5).  Results
+// do not change: such a cell belongs to a real alignment, counted dearer than
+// it is, so that an end it leads to at score s was found at s - e - 1 at the
+// latest; no cell on the way to the end at the optimum, and no tie there, comes
+// from one.
 __device__ __forceinline__ uint32_t band_absent(int x, int oe, int e) {
   uint32_t ex = 1u, gap = 0u;
   for (int s = 1; s < 32; ++s) {

@@ -1,13 +1,13 @@
 // kernels.cu -- the CUDA kernels of libwfa_gpu.so (sm_103a) and their
 // launchers.
 //
-//   short_kernel    fused pack + gap-affine WFA + backtrace for pairs whose
-//                   sequences are at most kShortLmax long and whose
-//                   wavefronts fit the group's shared memory (the paper's
-//                   100 bp workload, Sec. II); everything else is deferred
-//   general_kernel  one warp per deferred pair, wavefronts in a slice of the
-//                   global scratch arena, pairs taken from a device work
-//                   queue (atomic counter)
+//   short_kernel, lane_kernel  short pairs (the paper's 100 bp workload, Sec.
+//                   II) in call order, wavefronts in shared memory; what does
+//                   not fit is deferred (lane_band.cu has the kernels of
+//                   ordered input, band.cu those of deferred pairs)
+//   arena_kernel    a warp or CTA per pair the band kernels leave, wavefronts
+//                   in a slice of the global scratch arena, pairs taken from
+//                   a device work queue (atomic counter)
 //   validate/scan/compact/pack  bookkeeping around them
 #include <algorithm>
 #include <type_traits>
@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(kShortBlock, 8) short_kernel(const AlignArgs a
   __shared__ int s_last;
   short_body<G, LMAX, CELLS, SCAP, Off, LIN, EF>(a, smem, &s_last);
 }
-
 
 // One lane per pair, the warp's pairs in lockstep (lane_path.cuh); Fwd is
 // the forward pass: geometry from the table (any penalties) or fixed at

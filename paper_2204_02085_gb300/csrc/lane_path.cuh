@@ -173,13 +173,13 @@ struct LaneSt {
   int s_fin;           // scaled score once finished
 };
 
-// Matches from pattern position v and text position h, up to 32 (NW packed
+// Matches from pattern position v and text position h, up to 32 (kLaneWords packed
 // words at pw[j * 32], tw[j * 32]): the XOR of the two 32-base windows in two
 // 32-bit halves, leading zeros halved.  A window's third word past the last
-// one (j + 2 = NW) would hold only positions beyond any sequence's end, which
+// one (j + 2 = kLaneWords) would hold only positions beyond any sequence's end, which
 // no caller counts: the last word stands in for it.
-template <int NW>
 __device__ __forceinline__ int lane_match32(const uint32_t* pw, int v, const uint32_t* tw, int h) {
+  constexpr int NW = kLaneWords;
   const int jp = v >> 4, sp = (v & 15) << 1, jt = h >> 4, st = (h & 15) << 1;
   const uint32_t p1 = pw[(jp + 1) * 32];
   const uint32_t t1 = tw[(jt + 1) * 32];
@@ -205,7 +205,7 @@ __device__ __forceinline__ void lane_pending(LaneSt& st, uint32_t pend, int lo, 
       ch = cb - (int)st.H[(base + ci) * 32];
     }
     if (ci >= 0) {
-      const int eq = lane_match32<lane_words_of(127)>(st.pw, ch - ck, st.tw, ch);
+      const int eq = lane_match32(st.pw, ch - ck, st.tw, ch);
       ch += eq;
       if (eq < 32 || ch >= cb) {
         st.H[(base + ci) * 32] = (uint8_t)(cb - min(ch, cb));
@@ -466,7 +466,7 @@ __device__ __forceinline__ int lane_backtrace(const UGeo* tab, const uint8_t* H,
 
 // The lane-per-pair kernel body (global gap-affine alignment, both sequences
 // <= LMAX).  Pairs longer than LMAX, or whose score passes the last stored
-// wavefront (but not the caller's max_score), are deferred to the arena
+// wavefront (but not the caller's max_score), are deferred to the band
 // kernels, as are pairs whose CIGAR needs more than kSlot runs.
 template <int LMAX, int CELLS, int RW, int SPAN_BYTES, class Fwd>
 __device__ __forceinline__ void lane_body(const AlignArgs& a, const LaneGeo& lg, unsigned char* smem) {
@@ -548,7 +548,7 @@ __device__ __forceinline__ void lane_body(const AlignArgs& a, const LaneGeo& lg,
     if (real) {
       if (st.active) {
         // every stored score was tried: beyond the caller's bound, or beyond
-        // what this kernel stores (then the arena kernel takes the pair)
+        // what this kernel stores (then the pair is deferred)
         if (a.s_cap <= s_store) write_result(a, pair, 1, -1, 0, 0);
         else defer_pair(a, pair);
       } else if (st.s_fin >= 0) {

@@ -22,7 +22,7 @@ struct Ctrl {
   int32_t next_long;
   int32_t retry_count;      // pairs of the current retry list
   int32_t next_retry;
-  int32_t overflow_count;   // pairs an arena kernel could not fit
+  int32_t overflow_count;   // pairs that outgrew their slice of the arena, or the CIGAR pool
   int32_t pool_short;       // the CIGAR pool ran out
   unsigned long long pool_top;  // words used in the CIGAR pool
   long long pat_extent;     // max(offset + length) over patterns
@@ -61,7 +61,7 @@ struct AlignArgs {
   int64_t* run_src;   // where a pair's runs (last run first) are: >= 0 an
                       // index into `runs`, < 0 the index -src-1 into `pool`
   uint32_t* runs;     // [n * kSlot] per-pair slots of the short kernel
-  uint32_t* pool;     // runs of arena-kernel pairs, reserved by atomics
+  uint32_t* pool;     // runs of band- and arena-kernel pairs, reserved by atomics
   int64_t pool_cap;   // words in the pool
   int32_t* defer_list;       // [n] deferred medium pairs
   int32_t* defer_long_list;  // [n] deferred long pairs
@@ -80,10 +80,11 @@ struct AlignArgs {
   int lane_sort_min;  // smallest store (largest bound) whose ordering bounds each pair
 };
 
-// Packed 16-base words per sequence of at most lmax bases the lane kernel in
-// call order reads, and 32-base words per bit plane the one on ordered input
-// reads (a position past the last base included).
-__host__ __device__ constexpr int lane_words_of(int lmax) { return lmax / 16 + 2; }
+// Packed 16-base words per sequence (of at most 127 bases) the lane kernel in
+// call order reads, and 32-base words per bit plane of a sequence of at most
+// lmax bases the one on ordered input reads (a position past the last base
+// included).
+constexpr int kLaneWords = 127 / 16 + 2;
 __host__ __device__ constexpr int lane_plane_words(int lmax) { return lmax / 32 + 1; }
 // Most pairs the ordering sorts together.
 constexpr int kLaneGroupMax = 1024;
@@ -119,8 +120,8 @@ struct ShortVariant {
   // kind 1, ordered input (lane_band.cu): bytes of masks, rows and choices a
   // warp of the kernel over the diagonals within the bound keeps, the cell
   // size of its rows, its shared memory, its resident blocks (for scaled
-  // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's (large
-  // and small groups).
+  // penalties 2/4/1, 1/1/1 and any others) and the ordering pass's (with the
+  // walk, without it, and in small groups).
   // `kernel` takes call order (null: the variant runs on ordered input only)
   int band_store, band_cell, band_grid[3], order_grid[3];
   size_t band_smem;
@@ -194,22 +195,22 @@ constexpr int kLaneStore8 = lane_band_store(1536, 896, 6, 127), kLaneStore10 = l
               kLaneStore12 = lane_band_store(2304, 1408, 10, 127), kLaneStore16 = lane_band_store(3072, 2688, 14, 127),
               kLaneStore18 = lane_band_store(3456, 3328, 16, 127), kLaneStoreLin6 = lane_band_store(960, 896, 8, 127);
 
-// Arena kernels for pairs deferred by the short kernel: pairs list[0 ..
-// *count), taken through the work-queue head *next; `nteams` teams (one
-// warp each when long_team is false, one CTA of 8 warps otherwise), each
-// with slot_bytes of the arena; pairs that do not fit go to a.overflow_list.
-// The plain path: every pair onto the arena work lists.
+// Every pair onto the arena work lists (arena-only calls).
 cudaError_t launch_route_all(const AlignArgs& a, cudaStream_t st);
 
 // Resident teams per SM of an arena kernel with teams of team_warps warps
 // (1: one-warp teams of medium pairs; kLongTeamWide or kLongTeamNarrow:
 // one-CTA teams of long pairs).
 cudaError_t arena_occupancy(int team_warps, int* teams_per_sm);
+// An arena kernel over the pairs list[0 .. *count), taken through the
+// work-queue head *next by `nteams` teams with slot_bytes of the arena each;
+// pairs that do not fit go to a.overflow_list.
 cudaError_t launch_arena(int team_warps, const AlignArgs& a, const int32_t* list, const int32_t* count,
                          int32_t* next, int32_t* overflow_count, unsigned char* arena, long slot_bytes, int nteams,
                          cudaStream_t st);
 
-constexpr int kBandMaxPen = 31;  // scaled penalties the band kernels take: rows kept per pair
+constexpr int kBandMaxPen = 31;     // scaled penalties the band kernels take: rows kept per pair
+constexpr int kBandMaxLen = 32000;  // sequences they take are shorter: a row cell's offset fits 15 bits
 // The band kernels over the deferred pairs (a.defer_list, a.defer_long_list
 // and their counts in a.ctrl): each pair's score bound, the pairs ordered by
 // cost (largest first; in call order when `ordered` is false), then the band
@@ -237,8 +238,8 @@ constexpr int kBandBins = 128;
 constexpr int kBandAux = 2 * kBandBins;
 cudaError_t band_plan(int device, BandPlan* plan);
 // pairs: at most this many are deferred, nlong of them long; max_len: the
-// longest sequence among the call's (sizes the shared memory; a pair longer than that still ends up
-// right, in the arena lists).  launches: kernels enqueued.
+// longest sequence among the call's (sizes the shared memory; a longer pair in
+// a replay still ends up right, in the arena lists).
 cudaError_t launch_band(const AlignArgs& a, const BandPlan& plan, const BandBufs& b, int64_t pairs, int64_t nlong,
                         int max_len, bool ordered, unsigned char* arena, long arena_bytes, cudaStream_t st);
 // Kernels it enqueues: under scaled penalties above kBandMaxPen only those

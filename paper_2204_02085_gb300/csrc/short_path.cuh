@@ -158,7 +158,7 @@ __device__ __forceinline__ int bt_D(const LinUView<Off, P>& v, int s, int k) {
 // 32 lanes), then walk the backtrace (the pair's first lane) and write the
 // CIGAR runs (last first) into the pair's slot.  Pairs longer than LMAX, or
 // whose score passes the last storable wavefront (but not the caller's
-// max_score), are deferred to the arena kernel.  LIN: the gap-linear model
+// max_score), are deferred to the band kernels.  LIN: the gap-linear model
 // (o = 0, the edit distance at x = e = 1), only M stored.  EF: ends-free
 // calls (free pattern / text ends; the first wavefront spans the free
 // starts, the end test scans the free diagonals).
@@ -183,7 +183,7 @@ __device__ __forceinline__ void short_body(const AlignArgs& a, unsigned char* sm
   if (threadIdx.x == 0) s_last = build_ugeo(tab, SCAP, CELLS, pen, lo0, hi0);
   __syncthreads();
   // -1: the first wavefront does not fit; also when a global variant is
-  // handed an ends-free call (then the arena kernels take every pair)
+  // handed an ends-free call (then every pair is deferred)
   const int s_store = (!EF && (a.pb | a.pe | a.tb | a.te) != 0) ? -1 : s_last;
   const int s_hi = min(s_store, a.s_cap);
   const unsigned gmask = group_mask(G);
@@ -339,7 +339,7 @@ __device__ __forceinline__ void short_body(const AlignArgs& a, unsigned char* sm
     if (lane == 0) {
       if (active) {
         // every stored score was tried: beyond the caller's bound, or beyond
-        // what this kernel stores (then the arena kernel takes the pair)
+        // what this kernel stores (then the pair is deferred)
         if (a.s_cap <= s_store) write_result(a, pair, 1, -1, 0, 0);
         else defer_pair(a, pair);
       } else if (s_fin >= 0) {
