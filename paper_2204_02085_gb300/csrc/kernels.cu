@@ -526,7 +526,6 @@ __global__ void __launch_bounds__(kSmallBlock) small_finish_kernel(int n, const 
 // last of the 32 pairs whose offset is <= its position (binary search over
 // the offsets in shared memory; a pair without runs shares the next pair's
 // offset, so the search lands on a pair that has the word).
-constexpr int kLongRuns = 64;  // words a pair from which the output is cut by words
 __global__ void __launch_bounds__(kAuxBlock) compact_kernel(int64_t n, const int32_t* nruns, const int64_t* run_src,
                                                              const uint32_t* runs, const uint32_t* pool,
                                                              const int64_t* off, uint32_t* out, int64_t cap,
@@ -538,13 +537,14 @@ __global__ void __launch_bounds__(kAuxBlock) compact_kernel(int64_t n, const int
   __shared__ uint32_t s_words[kAuxBlock / 32][32 * kSlot];  // a batch's runs in output order
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if (off[n] > kLongRuns * n) {
+  const CompactSpans spans{n, off[0], off[n]};
+  if (spans.by_words()) {
     // long CIGARs: a warp per span of output words, whatever pairs it cuts
     // (2,000 pairs of 1,000 runs took 409 us on the 63 warps that have 32
     // pairs each)
-    constexpr int64_t kSpan = 256;
-    const int64_t total = off[n];
-    for (int64_t w0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kSpan; w0 < total;
+    constexpr int64_t kSpan = CompactSpans::kSpan;
+    const int64_t total = spans.last;
+    for (int64_t w0 = spans.begin(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); w0 < total;
          w0 += nwarps * kSpan) {
       int64_t lo = 0, hi = n;  // the last pair whose offset is <= w0
       while (hi - lo > 1) {

@@ -284,6 +284,17 @@ constexpr int kScanTile = 2048;
 int64_t scan_tmp_elems(int64_t n);
 cudaError_t launch_scan(const int32_t* in, int64_t n, int kind, int64_t* out, int64_t* tmp, cudaStream_t st);
 
+// The output words of a compaction: off[0] .. off[n] of its n pairs.  off[0] is
+// not 0 for a chunk of a call: the words before it are other chunks', maybe on
+// their way to the host.
+struct CompactSpans {
+  int64_t n, first, last;
+  static constexpr int64_t kSpan = 256;  // words a warp takes at a time
+  // cut by words, not by pairs: 64 words and more a pair
+  __host__ __device__ constexpr bool by_words() const { return last - first > 64 * n; }
+  // first word of a warp's first span
+  __host__ __device__ constexpr int64_t begin(int64_t warp) const { return first + warp * kSpan; }
+};
 // CIGAR compaction: pair i's runs (stored last first, see run_src) to
 // out[off[i] .. off[i+1]) in order; writes nothing if off[n] > cap or the
 // inputs were rejected (ctrl may be NULL).
