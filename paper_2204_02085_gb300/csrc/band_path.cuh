@@ -572,7 +572,10 @@ __device__ void band_pair(const AlignArgs& a, uint32_t absent, int64_t pair, int
   // first warp: the CIGAR, into a reservation of the run pool
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int most = min(s / min(a.xs, a.oes), n + m);  // events: each costs that much, and takes a base
+  // events: each costs that much, and takes a base (the lengths read again:
+  // with n and m kept in registers across the rows the row loop compiles to a
+  // form 3 % slower on long reads, 2,000 x 10 kbp 5.42 against 5.24 ms a call)
+  const int most = min(s / min(a.xs, a.oes), a.plen[pair] + a.tlen[pair]);
   const unsigned long long want = 2ull * most + 3;
   unsigned long long pos = 0;
   if (lane == 0) pos = atomicAdd(&a.ctrl->pool_top, want);

@@ -402,8 +402,8 @@ __host__ __device__ constexpr int lane_band_rows(int x, int oe, int e) { return 
 // caller's bound), as are pairs whose CIGAR needs more than kSlot runs.  A
 // batch whose end diagonals spread too far for the store (around the border
 // of two bounds) runs in two or more passes.
-// Bound by instruction issue and the latency between a cell's steps (66 and
-// 63 % of the issue slots by instructions and duration); with the large store
+// Bound by instruction issue and the latency between a cell's steps (67 and
+// 64 % of the issue slots by instructions and duration); with the large store
 // by the 16 warps an SM its 12.9 KB a warp leave.  1M pairs of 100 bases: E =
 // 2 % 144 -> 90 us, E = 4 % 508 -> 276 us (75 and 220 warp instructions a pair),
 // before: every diagonal a row can hold (lane_path.cuh).
