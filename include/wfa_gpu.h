@@ -103,13 +103,13 @@ enum {
 typedef struct {
   float h2d_ms;      /* host -> device copies of inputs (host-pointer mode) */
   float align_ms;    /* the short-read phase: ordering pass and short-read kernel */
-  float general_ms;  /* the scratch-arena wavefront kernel (pairs it took over) */
+  float general_ms;  /* the band and arena kernels (pairs the short-read phase deferred) */
   float cigar_ms;    /* CIGAR offset scan and compaction */
   float d2h_ms;      /* device -> host copies of outputs (host-pointer mode) */
   float total_ms;    /* whole call, first to last event */
   int32_t kernel_launches; /* kernels this library launched during the call */
   int32_t short_variant;   /* index of the short-read kernel variant that ran (-1: none) */
-  int64_t deferred_pairs;  /* pairs handed from the short-read kernel to the arena kernel */
+  int64_t deferred_pairs;  /* pairs handed from the short-read phase to the band and arena kernels */
 } wfa_gpu_timing;
 
 /* Create a context on CUDA device `device`.
@@ -347,15 +347,19 @@ int64_t wfa_gpu_server_submit(wfa_gpu_server *server, const wfa_gpu_request *req
 int wfa_gpu_server_wait(wfa_gpu_server *server, int64_t id, double timeout_s, wfa_gpu_request_stats *stats);
 
 /* Estimated device bytes a request holds while it runs: its sequence
- * bytes, 150 bytes a pair (lengths, offsets, outputs, work buffers, CIGAR
- * slots), 4 bytes a word of CIGAR capacity, and the arena its wavefronts
- * take -- for pairs longer than 127 bases (the short-read kernels keep
- * theirs in shared memory), 3 offsets of 2 bytes (4 from 32,000 bases) on
- * about (s'/e' + 1)^2 cells plus 16 (s' + 1) bytes of per-score records,
- * s' = WFA_GPU_SERVER_EDIT_RATE x max(n, m) x max(x, o + e) / g and
- * e' = e / g (g = gcd(x, o, e)), summed over the 4,096 largest such pairs
- * (no more run at once).  The arena part is what the server admits
- * requests by.  Returns -1 for a NULL or malformed request (n_pairs < 0,
+ * bytes, 150 bytes a pair (lengths, offsets, outputs, work lists, CIGAR
+ * slots; not the copies of its sequences that batches of more than 4,096
+ * short pairs are ordered into, another 72 bytes a pair up to 127 bases and
+ * at most 136 up to 255), 4 bytes a word of CIGAR capacity, and the arena
+ * its wavefronts may take -- for pairs longer than 127 bases, 3 offsets of 2
+ * bytes (4 from 32,000 bases) on about (s'/e' + 1)^2 cells plus 16 (s' + 1)
+ * bytes of per-score records, s' = WFA_GPU_SERVER_EDIT_RATE x max(n, m) x
+ * max(x, o + e) / g and e' = e / g (g = gcd(x, o, e)), summed over the 4,096
+ * largest such pairs (no more run at once).  That is what the arena kernels
+ * keep of a pair; the band kernels, which take nearly all of them, keep half a
+ * byte on about half of the cells, and reads of up to 255 bases that stay with
+ * the short-read kernels nothing, so that the arena part is an upper estimate.
+ * It is what the server admits requests by.  Returns -1 for a NULL or malformed request (n_pairs < 0,
  * or missing length arrays).  Host-only. */
 int64_t wfa_gpu_request_bytes(const wfa_gpu_request *req);
 

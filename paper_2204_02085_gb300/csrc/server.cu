@@ -36,8 +36,8 @@ using Clock = std::chrono::steady_clock;
 // not passed any more once it has waited this long: the slots then drain
 // until it fits.
 constexpr double kMaxWaitS = 0.05;
-// The smallest arena slice a call runs on (short pairs the short-read kernel
-// defers go to the arena kernels too).
+// The smallest arena slice a call runs on (short pairs the short-read kernels
+// defer need some of it too).
 constexpr int64_t kMinSlice = 64ll << 20;
 // Calls in flight at once, whatever the slots: two keep the GPU busy while
 // one call's batch is gathered or scattered on the host; more only queued
@@ -127,13 +127,14 @@ struct Slot {
   Dev<uint32_t> dcig;
 };
 
-// Scratch-arena bytes a request's wavefronts hold at once.  Pairs longer than
-// the short-read kernels take (127 bases) go to the arena kernels, which
-// keep every score's M, I and D offsets (2 bytes each below 32,000 bases, 4
-// above) over about (s'/e' + 1)^2 cells, s' the scaled score of
-// WFA_GPU_SERVER_EDIT_RATE edits per base at the costliest edit
-// (max(x, o + e) / g each), e' = e / g; at most kConcurrentTeams pairs are in
-// flight at once, so the estimate sums the kConcurrentTeams largest.
+// Scratch-arena bytes a request's wavefronts may hold at once, by what the
+// arena kernels keep of a pair longer than 127 bases: every score's M, I and D
+// offsets (2 bytes each below 32,000 bases, 4 above) over about (s'/e' + 1)^2
+// cells, s' the scaled score of WFA_GPU_SERVER_EDIT_RATE edits per base at the
+// costliest edit (max(x, o + e) / g each), e' = e / g; at most kConcurrentTeams
+// pairs are in flight at once, so the estimate sums the kConcurrentTeams
+// largest.  An upper estimate: the band kernels, which take nearly all of these
+// pairs, keep half a byte on about half of the cells.
 constexpr int kConcurrentTeams = 4096;
 int gcd2(int a, int b) {
   while (b) {
